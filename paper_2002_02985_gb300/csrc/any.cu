@@ -1,0 +1,146 @@
+// Plans, candidates and instantiations of the any-length kernels (any.cuh); the
+// reciprocal-space kernels are instantiated in any_ax0.cu.
+#include <algorithm>
+#include <cstdio>
+
+#include "any.cuh"
+
+namespace ofdft {
+
+static const int kRadices[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
+
+AnyPlan any_plan(int n, int last) {
+    AnyPlan q;
+    q.n = n;
+    q.np = 0;
+    if (n < 4 || n > 1024) return q;
+    // two passes where the radices allow, else three; of equal pass counts the plan whose
+    // largest radix is smallest (most butterflies per pass, fewest registers)
+    int best[3] = {0, 0, 0}, np = 0, score = 1 << 30;
+    for (int a : kRadices)
+        for (int b : kRadices) {
+            if (n % (a * b)) continue;
+            const int c = n / (a * b);
+            if (c == 1) {
+                if (last && b != last) continue;
+                if (!last && a < b) continue;
+                const int s = std::max(a, b) * 32 + a;
+                if (np != 2 || s < score) {
+                    np = 2;
+                    score = s;
+                    best[0] = a;
+                    best[1] = b;
+                }
+            } else if (np != 2 && std::find(std::begin(kRadices), std::end(kRadices), c) != std::end(kRadices)) {
+                if (last && c != last) continue;
+                if (a < b || (!last && b < c)) continue;
+                const int s = (std::max(a, std::max(b, c)) * 32 + a) * 32 + b;
+                if (s < score) {
+                    np = 3;
+                    score = s;
+                    best[0] = a;
+                    best[1] = b;
+                    best[2] = c;
+                }
+            }
+        }
+    q.np = np;
+    int ns = 1;
+    for (int i = 0; i < np; i++) {
+        AnyPass &p = q.p[i];
+        p.R = best[i];
+        p.ns = ns;
+        p.nb = n / p.R;
+        p.stride = n / (ns * p.R);
+        p.magic = ((1 << 20) + ns - 1) / ns;
+        ns *= p.R;
+    }
+    return q;
+}
+
+// the same radices in reverse order (an inverse transform that starts where the forward ended)
+AnyPlan any_reversed(const AnyPlan &q) {
+    AnyPlan r = q;
+    int ns = 1;
+    for (int i = 0; i < q.np; i++) {
+        AnyPass &p = r.p[i];
+        p.R = q.p[q.np - 1 - i].R;
+        p.ns = ns;
+        p.nb = q.n / p.R;
+        p.stride = q.n / (ns * p.R);
+        p.magic = ((1 << 20) + ns - 1) / ns;
+        ns *= p.R;
+    }
+    return r;
+}
+
+// the reciprocal-space kernels (any_ax0.cu): null where RL is not compiled for T
+template <typename T> const void *any_axis0_kernel(int RL, bool mgp);
+
+template <typename T> const void *any_row_kernel(int E, bool inverse) {
+    if (E <= 1) return inverse ? (const void *)row_inv_any_kernel<T, 1> : (const void *)row_fwd_any_kernel<T, 1>;
+    if (E <= 2) return inverse ? (const void *)row_inv_any_kernel<T, 2> : (const void *)row_fwd_any_kernel<T, 2>;
+    return inverse ? (const void *)row_inv_any_kernel<T, 4> : (const void *)row_fwd_any_kernel<T, 4>;
+}
+
+template <typename T> void any_candidates(int role, int n, std::vector<KernelCand> &out) {
+    KernelCand c;
+    c.any = 1;
+    auto add = [&](const void *k1, const void *k2, int B, int nt, const char *kind) {
+        c.k1 = c.g1 = k1;
+        c.k2 = c.g2 = k2;
+        c.B = B;
+        c.nt = nt;
+        std::snprintf(c.name, sizeof(c.name), "%s %dx%d", kind, B, nt);
+        out.push_back(c);
+    };
+    const AnyPlan q = any_plan(n);
+    if (role == ROLE_PENCIL && q.np >= 2) {
+        // 16-column tiles (128-byte rows in FP32) while three blocks fit an SM, else 8
+        for (int lg : {4, 3}) {
+            if (any_pencil_smem<T>(q, lg) > 74 * 1024 && lg > 3) continue;
+            if (any_pencil_smem<T>(q, lg) > 200 * 1024) continue;
+            add((const void *)pencil_any_kernel<T, -1>, (const void *)pencil_any_kernel<T, +1>, 1 << lg, 256, "anypencil");
+            break;
+        }
+    }
+    if (role == ROLE_ROW2 && q.np >= 1) {
+        c.batched = true;
+        int last = 0;
+        // the channel group fills half or a third of an SM's shared memory per block
+        for (int kb : {40, 76}) {
+            const int G = std::min(34, (int)(kb * 1024 / (2 * (size_t)(n + 2) * 2 * sizeof(T))));
+            if (G < 1 || G == last) continue;
+            last = G;
+            c.batched = true;
+            add(any_row_kernel<T>(1, false), any_row_kernel<T>(1, true), G, 320, "anyrows");
+        }
+    }
+    if (role == ROLE_AXIS0) {
+        int made = 0;
+        for (int RL : {16, 15, 12, 10, 9, 8, 5, 4}) {
+            const void *k = any_axis0_kernel<T>(RL, false), *km = any_axis0_kernel<T>(RL, true);
+            if (!k || n % RL || any_plan(n, RL).np < 2 || made >= 3) continue;
+            const int tmax = sizeof(T) == 4 ? (RL >= 12 ? 256 : 512) : 256;
+            // 16 columns where the block and its tiles leave room for two blocks per SM, else 8, else 4
+            for (int lg : {4, 3, 2}) {
+                const int nt = ((n / RL << lg) + 31) / 32 * 32;
+                if (nt > tmax || any_axis0_smem<T>(n, lg) > (lg == 4 ? 100 : 200) * 1024) continue;
+                c.RL = RL;
+                add(k, km, 1 << lg, nt, "anyrecip");
+                std::snprintf(c.name, sizeof(c.name), "anyrecip r%d %dx%d", RL, 1 << lg, nt);
+                std::snprintf(out.back().name, sizeof(c.name), "%s", c.name);
+                made++;
+                break;
+            }
+        }
+    }
+}
+
+#define INST(T)                                                              \
+    template const void *any_row_kernel<T>(int, bool);                       \
+    template void any_candidates<T>(int, int, std::vector<KernelCand> &);
+INST(float)
+INST(double)
+
+}  // namespace ofdft

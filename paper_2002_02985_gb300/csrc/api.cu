@@ -86,6 +86,10 @@ template <typename T> struct Workspace {
     LaunchSet ks;                     // FFT-carrying kernels (size-specialised where compiled)
     int Brow = 0, thr_rowf = 0, thr_rowi = 0, TW1 = 0, thr_p1 = 0, TW0 = 0, thr_ax0 = 0, nb_row = 0, nb_ax0 = 0;
     int grid_p1 = 0;
+    // any-length kernels in use per role, their tile widths (log2), plans, largest row group
+    int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0;
+    AnyPlan q0, q0i;
+    int TW0_p = 0, thr_ax0_p = 0;     // the runtime-size n0 transform of plain fields
     int row2_G = 0;                   // channel-batched row kernels in use: channels per group
     int ax0_scr = 0;                  // the reciprocal-space kernel transforms out of place
     // plain one-channel transforms (preconditioner, interpolation, TD-OFDFT): the per-channel row
@@ -252,6 +256,8 @@ template <typename T> int apply_cand(ofdft_grid *g, Workspace<T> &w, int role, c
         w.ks.row_inv = c.k2;
         w.ks.row_fwd_g = c.g1;
         w.ks.row_inv_g = c.g2;
+        w.any2 = c.any;
+        w.any_Gmax = c.B;
         w.Brow = c.batched ? 1 : c.B;
         w.row2_G = c.batched ? c.B : 0;
         w.thr_rowf = w.thr_rowi = c.nt;
@@ -267,6 +273,11 @@ template <typename T> int apply_cand(ofdft_grid *g, Workspace<T> &w, int role, c
         w.ks_plain.pen_inv_g = c.g2;
         w.TW1 = c.B;
         w.thr_p1 = c.nt;
+        w.any1 = c.any;
+        if (c.any) {
+            for (w.lg1 = 0; (1 << w.lg1) < c.B;) w.lg1++;
+            return OFDFT_OK;
+        }
         // persistent pencil grid: every resident block slot of the device, once
         int per_sm = 0;
         cudaError_t e = allow_max_dynamic_smem(c.k1);
@@ -276,6 +287,12 @@ template <typename T> int apply_cand(ofdft_grid *g, Workspace<T> &w, int role, c
         w.grid_p1 = std::max(1, per_sm) * g->nsm;
     } else {
         const long long P = (long long)g->n[1] * g->n2h;
+        w.any0 = c.any;
+        if (c.any) {
+            for (w.lg0 = 0; (1 << w.lg0) < c.B;) w.lg0++;
+            w.q0 = any_plan(g->n[0], c.RL);
+            w.q0i = any_reversed(w.q0);
+        }
         if (c.recip.k) {
             w.ks.recip = c.recip;
             w.recip_grid = (int)std::min((P + c.recip.tw - 1) / c.recip.tw, (long long)c.recip.per_sm * g->nsm);
@@ -329,6 +346,12 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
             TW /= 2;
         w.TW0 = TW;
         w.thr_ax0 = std::min(std::max(threads_for(g->plan[0], TW, cap), 128), tmax);
+        w.TW0_p = w.TW0;
+        w.thr_ax0_p = w.thr_ax0;
+        w.Brow_p = w.Brow;
+        w.thr_rowf_p = w.thr_rowi_p = w.thr_rowf;
+        w.any0 = w.any1 = w.any2 = 0;
+        w.ks_plain = w.ks;
         w.ks.recip = RecipLaunch();
     }
     const long long P = (long long)g->n[1] * g->n2h;
@@ -351,6 +374,17 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
                               g->kernel_choice == OFDFT_KERNELS_PER_CHANNEL_ROWS || P % 2 != 0 || !tensor_encoder()))
                 continue;
             w.cand[TUNE_AXIS0].push_back(k);
+        }
+        // any-length kernels: the default where nothing is compiled for the length
+        if (g->kernel_choice == OFDFT_KERNELS_AUTO) {
+            any_candidates<T>(ROLE_ROW2, g->n[2], w.cand[TUNE_ROWS]);
+            any_candidates<T>(ROLE_PENCIL, g->n[1], w.cand[TUNE_PENCIL]);
+            any_candidates<T>(ROLE_AXIS0, g->n[0], w.cand[TUNE_AXIS0]);
+            for (int E : {1, 2, 4}) {
+                cudaError_t e = allow_max_dynamic_smem(any_row_kernel<T>(E, false));
+                if (e == cudaSuccess) e = allow_max_dynamic_smem(any_row_kernel<T>(E, true));
+                if (e != cudaSuccess) return fail(g, OFDFT_ERR_CUDA, "kernel attributes", e);
+            }
         }
     }
     // partial buffers sized for every configuration; the first of each role is the default
@@ -384,12 +418,11 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
         int rc = apply_cand<T>(g, w, TUNE_PENCIL, KernelCand{w.ks.pen_fwd, w.ks.pen_inv, w.ks.pen_fwd_g, w.ks.pen_inv_g, w.TW1, w.thr_p1});
         if (rc) return rc;
     }
-    // plain one-channel transforms: the per-channel row kernels where compiled
-    w.ks_plain = w.ks;
-    w.Brow_p = w.Brow;
-    w.thr_rowf_p = w.thr_rowf;
-    w.thr_rowi_p = w.thr_rowi;
-    w.row2_G_p = w.row2_G;
+    // plain one-channel transforms: the per-channel row kernels where compiled, else the
+    // runtime-size ones
+    w.ks_plain.pen_fwd = w.ks.pen_fwd;
+    w.ks_plain.pen_inv = w.ks.pen_inv;
+    w.row2_G_p = 0;
     for (const KernelCand &k : w.cand[TUNE_ROWS])
         if (!k.batched) {
             w.ks_plain.row_fwd = k.k1;
@@ -752,6 +785,52 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
     return OFDFT_OK;
 }
 
+// the any-length plans of an evaluation or a plain transform (its rows are not any-length)
+template <typename T> void any_args_of(const ofdft_grid *g, const Workspace<T> &w, EvalArgs<T> &a) {
+    a.any0 = w.any0;
+    a.any1 = w.any1;
+    if (w.any0) {
+        a.lg0 = w.lg0;
+        a.q0 = w.q0;
+        a.q0i = w.q0i;
+    }
+    if (w.any1) {
+        a.lg1 = w.lg1;
+        a.q1 = any_plan(g->n[1]);
+    }
+}
+
+// The any-length rows of an evaluation: channels in equal groups of at most the configuration's,
+// a thread per butterfly of the widest pass, and the kernel for the points a thread then owns.
+template <typename T> void choose_any_rows(Workspace<T> &w, EvalArgs<T> &a) {
+    const int n = a.n2, n2h = a.n2h;
+    a.q2 = any_plan(n);
+    a.magic_n2h = (unsigned)(((1ull << 32) + n2h - 1) / n2h);
+    a.magic_2n2h = (unsigned)(((1ull << 32) + 2 * n2h - 1) / (2 * n2h));
+    int nbmax = 1;
+    for (int i = 0; i < a.q2.np; i++) nbmax = std::max(nbmax, a.q2.p[i].nb);
+    for (int inv = 0; inv < 2; inv++) {
+        const int nch = std::max(1, inv ? a.ninv : a.nfwd), groups = (nch + w.any_Gmax - 1) / w.any_Gmax;
+        const int G = (nch + groups - 1) / groups;
+        int nt = std::min(320, std::max(64, (nbmax * G + 31) / 32 * 32));
+        int E = (n + nt - 1) / nt;
+        if (E > 2) {
+            E = 4;
+            nt = std::min(256, std::max(nt, ((n + 3) / 4 + 31) / 32 * 32));
+        }
+        a.any_G[inv] = G;
+        a.magic_G[inv] = (unsigned)(((1ull << 32) + G - 1) / G);
+        const void *k = any_row_kernel<T>(E, inv != 0);
+        if (inv) {
+            w.ks.row_inv = w.ks.row_inv_g = k;
+            a.thr_rowi = nt;
+        } else {
+            w.ks.row_fwd = w.ks.row_fwd_g = k;
+            a.thr_rowf = nt;
+        }
+    }
+}
+
 // Fill the arguments of one evaluation (host work: the workspace, V_ext(G), the tuner's picks
 // and the tensor maps are made ready first; nothing is launched).
 template <typename T>
@@ -830,6 +909,8 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     a.grid_p1 = w.grid_p1;
     a.row2_G = w.row2_G;
     a.ax0_scr = w.ax0_scr;
+    any_args_of(g, w, a);
+    a.any2 = w.any2;
     a.wait_polls = g->wait_polls;
     a.exact_sums = g->exact_sums;
     // the normalised density spectrum for the forces, written by the reciprocal-space kernel
@@ -877,6 +958,7 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
             }
         }
     }
+    if (w.any2) choose_any_rows<T>(w, a);
     if (w.ks.recip.k && (w.maps_chan != w.chan || w.maps_vext != w.vext || w.maps_nslots != w.nslots ||
                          w.maps_tw != w.ks.recip.tw)) {
         const long long PL = (long long)g->n[1] * g->n2h;
@@ -966,6 +1048,7 @@ template <typename T> EvalArgs<T> plain_args(ofdft_grid *g, Workspace<T> &w, con
     a.Brow = w.Brow_p; a.thr_rowf = w.thr_rowf_p; a.thr_rowi = w.thr_rowi_p;
     a.TW1 = w.TW1; a.thr_p1 = w.thr_p1; a.TW0 = w.TW0; a.thr_ax0 = w.thr_ax0; a.grid_p1 = w.grid_p1;
     a.row2_G = w.row2_G_p; a.ax0_scr = w.ax0_scr;
+    any_args_of(g, w, a);
     a.nfwd = 1; a.fwd_ch[0] = CH_HPP; a.ncol = 1; a.col_ch[0] = CH_HPP;
     return a;
 }
@@ -974,7 +1057,7 @@ template <typename T> EvalArgs<T> plain_args(ofdft_grid *g, Workspace<T> &w, con
 template <typename T> int forward_plain(ofdft_grid *g, Workspace<T> &w, const T *field) {
     EvalArgs<T> a = plain_args<T>(g, w, field);
     CK(launch_forward_rows_cols<T>(a, w.ks_plain, g->stream), "forward transform");
-    CK(launch_axis0_fft<T>(w.chan, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0], w.tw[0], w.TW0, w.thr_ax0,
+    CK(launch_axis0_fft<T>(w.chan, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0], w.tw[0], w.TW0_p, w.thr_ax0_p,
                            1.0 / (double)g->N, g->stream, -1),
        "forward transform along n0");
     return OFDFT_OK;
@@ -992,7 +1075,7 @@ template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot
     a.inv_ch[0] = slot;
     a.inv_kind[0] = CONS_ADD;
     CK(launch_axis0_fft<T>((C *)w.chan + (size_t)slot * g->NH, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0],
-                           w.tw[0], w.TW0, w.thr_ax0, 1.0, g->stream, +1),
+                           w.tw[0], w.TW0_p, w.thr_ax0_p, 1.0, g->stream, +1),
        "inverse transform along n0");
     CK(launch_inverse_cols_rows<T>(a, w.ks_plain, g->stream), "inverse transform");
     return OFDFT_OK;
@@ -2118,7 +2201,8 @@ template <typename T> std::vector<unsigned char> launch_signature(const LaunchSe
     append_kernels(k, ks);
     const int v[] = {a.n0,       a.n1,       a.n2,    a.nb_stats, a.nb_ax0, a.nb_row, a.Brow,     a.thr_rowf,
                      a.thr_rowi, a.TW1,      a.thr_p1, tile[0],   tile[1],  tile[2],  a.grid_p1,  a.row2_G,
-                     a.nfwd,     a.ncol,     a.ncol_inv, a.exact_sums, a.mgp_tab != nullptr};
+                     a.nfwd,     a.ncol,     a.ncol_inv, a.exact_sums, a.mgp_tab != nullptr,
+                     a.any0,     a.any1,     a.any2,  a.lg0,      a.lg1,    a.any_G[0], a.any_G[1]};
     append_bytes(k, v);
     return k;
 }

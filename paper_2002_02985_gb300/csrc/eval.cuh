@@ -45,6 +45,17 @@ constexpr int kMaxThreads = 512;     // block size bound of the FFT kernels
 // complex values a thread stages per FFT pass (register budget per precision)
 template <typename T> struct Cap { static constexpr int value = sizeof(T) == 4 ? 16 : 8; };
 
+// Plan of the any-length kernels (any.cuh): passes of radix R after ns = the product of the
+// earlier radices, nb = n / R butterflies, stride = n / (ns R) the twiddle step, and
+// (j magic) >> 20 = j / ns for every j < 1024 (magic = ceil(2^20 / ns)).  np = 0: no plan.
+struct AnyPass {
+    int R, ns, nb, stride, magic;
+};
+struct AnyPlan {
+    int n, np;
+    AnyPass p[3];
+};
+
 template <typename T> struct EvalArgs {
     typedef typename Vec2<T>::type C;
     int n0, n1, n2, n2h;
@@ -82,6 +93,11 @@ template <typename T> struct EvalArgs {
     int ax0_scr;                         // the reciprocal-space kernel has a scratch tile (out-of-place transforms)
     unsigned wait_polls;                 // polls of a bounded wait for bulk copies before it gives up
     int exact_sums;                      // FP32-mixed test option: every energy term added in FP64
+    // any-length kernels in use (any.cuh): the n0 (forward and inverse), n1 and n2 plans, log2 of
+    // the column tiles, channels per row group (forward, inverse), reciprocals of the row indices
+    int any0, any1, any2, lg0, lg1, any_G[2];
+    AnyPlan q0, q0i, q1, q2;
+    unsigned magic_n2h, magic_2n2h, magic_G[2];
     C *rhohat_out;                       // if set: the normalised rho_hat (Hartree/PP channel) for the forces
     int nfwd, fwd_ch[kMaxChan];          // channels formed by row_fwd (slot ids)
     int ncol, col_ch[kMaxChan];          // channels transformed forward along n1
@@ -145,14 +161,30 @@ template <typename T> __host__ __device__ inline size_t row2_smem_bytes(int n2, 
     return (size_t)n2 * sizeof(C) + 2 * scr * sizeof(C) + 16;
 }
 template <typename T> __host__ __device__ inline size_t rowf_smem(const EvalArgs<T> &a) {
+    if (a.any2) return row2_smem_bytes<T>(a.n2, a.any_G[0]);
     return a.row2_G ? row2_smem_bytes<T>(a.n2, a.row2_G) : row_fwd_smem_bytes<T>(a.n2, a.Brow);
 }
 template <typename T> __host__ __device__ inline size_t rowi_smem(const EvalArgs<T> &a) {
+    if (a.any2) return row2_smem_bytes<T>(a.n2, a.any_G[1]);
     return a.row2_G ? row2_smem_bytes<T>(a.n2, a.row2_G) : row_inv_smem_bytes<T>(a.n2, a.Brow);
 }
 
+// any-length pencils: one tile per exchange (three passes: two); the any-length
+// reciprocal-space pass: two load buffers and the exchange tile
+template <typename T> inline size_t any_pencil_smem(const AnyPlan &q, int lg) {
+    return ((size_t)(q.np > 2 ? 2 : 1) * q.n << lg) * 2 * sizeof(T);
+}
+template <typename T> inline size_t any_axis0_smem(int n, int lg) { return ((size_t)3 * n << lg) * 2 * sizeof(T); }
+template <typename T> inline size_t pen_smem(const EvalArgs<T> &a) {
+    return a.any1 ? any_pencil_smem<T>(a.q1, a.lg1) : pencil_smem_bytes<T>(a.n1, a.TW1);
+}
+template <typename T> inline size_t ax0_smem(const EvalArgs<T> &a) {
+    return a.any0 ? any_axis0_smem<T>(a.n0, a.lg0) : axis0_smem_bytes<T>(a.n0, a.TW0, a.ax0_scr);
+}
 // persistent pencil grid: at most grid_p1 blocks (resident capacity), never more than tiles
+// (the any-length pencils run one tile per block)
 template <typename T> inline unsigned pencil_tiles(const EvalArgs<T> &a, int nch) {
+    if (a.any1) return (unsigned)((((long long)a.n0 * a.n2h + (1 << a.lg1) - 1) >> a.lg1) * nch);
     const long long t = (((long long)a.n0 * a.n2h + a.TW1 - 1) / a.TW1) * nch;
     return (unsigned)(t < a.grid_p1 ? t : a.grid_p1);
 }
@@ -196,6 +228,7 @@ struct KernelCand {
     const void *g1 = nullptr, *g2 = nullptr;   // their grouped forms
     int B = 0, nt = 0;
     bool batched = false;                 // channel-batched row kernels (B = channels per group)
+    int any = 0, RL = 0;                  // any-length kernels (any.cuh): B = tile width or largest channel group
     RecipLaunch recip;
     char name[48] = {0};
 };
@@ -203,6 +236,13 @@ struct KernelCand {
 // The compiled configurations of a role for axis length n (empty: only the runtime-size
 // kernels exist), the default first.  ROLE_AXIS0 lists the persistent kernels first.
 template <typename T> void kernel_candidates(int role, int n, std::vector<KernelCand> &out);
+// the any-length configurations of a role for axis length n (any.cu), appended to out
+template <typename T> void any_candidates(int role, int n, std::vector<KernelCand> &out);
+// the any-length plan of n (last: the radix of the last pass, 0 = free); np = 0 if there is none
+AnyPlan any_plan(int n, int last = 0);
+AnyPlan any_reversed(const AnyPlan &q);
+// the any-length row kernel (forward or inverse) for E elements per thread
+template <typename T> const void *any_row_kernel(int E, bool inverse);
 // The default configuration of a role for size n; false when none is compiled.
 template <typename T> bool find_specialised(int role, int n, const void **k1, const void **k2, int *B, int *nt);
 // the persistent reciprocal-space kernels compiled for n0 = n (recip.cu)

@@ -65,7 +65,10 @@ cudaError_t prepare_kernels(const LaunchSet &ks) {
 
 template <typename T>
 static cudaError_t launch(const void *k, dim3 g, int nt, size_t smem, const EvalArgs<T> &a, cudaStream_t s) {
-    void *args[] = {(void *)&a};
+    // (the any-length kernels also take a batch's argument list: none here)
+    const EvalArgs<T> *ga = nullptr;
+    int bps = 0;
+    void *args[] = {(void *)&a, (void *)&ga, (void *)&bps};
     return cudaLaunchKernel(k, g, dim3(nt), args, smem, s);
 }
 
@@ -91,7 +94,7 @@ cudaError_t launch_eval(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t 
     }
     if (a.ncol > 0) {
         mark(K_PENCIL_FWD, 0);
-        e = launch(ks.pen_fwd, dim3(pencil_tiles(a, a.ncol)), a.thr_p1, pencil_smem_bytes<T>(a.n1, a.TW1), a, s);
+        e = launch(ks.pen_fwd, dim3(pencil_tiles(a, a.ncol)), a.thr_p1, pen_smem(a), a, s);
         if (e) return e;
         mark(K_PENCIL_FWD, 1);
     }
@@ -102,13 +105,13 @@ cudaError_t launch_eval(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t 
                              ks.recip.smem, s);
     } else {
         e = launch(a.mgp_tab ? ks.axis0_mgp : ks.axis0, dim3(a.nb_ax0), a.thr_ax0,
-                   axis0_smem_bytes<T>(a.n0, a.TW0, a.ax0_scr), a, s);
+                   ax0_smem(a), a, s);
     }
     if (e) return e;
     mark(K_AXIS0, 1);
     if (a.ncol_inv > 0) {
         mark(K_PENCIL_INV, 0);
-        e = launch(ks.pen_inv, dim3(pencil_tiles(a, a.ncol_inv)), a.thr_p1, pencil_smem_bytes<T>(a.n1, a.TW1),
+        e = launch(ks.pen_inv, dim3(pencil_tiles(a, a.ncol_inv)), a.thr_p1, pen_smem(a),
                    a, s);
         if (e) return e;
         mark(K_PENCIL_INV, 1);
@@ -130,7 +133,7 @@ template <typename T> cudaError_t launch_forward_rows_cols(const EvalArgs<T> &a,
     stats_kernel<T><<<a.nb_stats, 256, 0, s>>>(a);
     cudaError_t e = launch(ks.row_fwd, dim3(nrt), a.thr_rowf, rowf_smem<T>(a), a, s);
     if (e) return e;
-    e = launch(ks.pen_fwd, dim3(pencil_tiles(a, a.ncol)), a.thr_p1, pencil_smem_bytes<T>(a.n1, a.TW1), a, s);
+    e = launch(ks.pen_fwd, dim3(pencil_tiles(a, a.ncol)), a.thr_p1, pen_smem(a), a, s);
     if (e) return e;
     return cudaGetLastError();
 }
@@ -141,7 +144,7 @@ cudaError_t launch_inverse_cols_rows(const EvalArgs<T> &a, const LaunchSet &ks, 
     const long long pairs = (R + 1) / 2;
     const int nrt = (int)((pairs + a.Brow - 1) / a.Brow);
     cudaError_t e = launch(ks.pen_inv, dim3(pencil_tiles(a, a.ncol_inv)), a.thr_p1,
-                           pencil_smem_bytes<T>(a.n1, a.TW1), a, s);
+                           pen_smem(a), a, s);
     if (e) return e;
     e = launch(ks.row_inv, dim3(nrt), a.thr_rowi, rowi_smem<T>(a), a, s);
     if (e) return e;

@@ -35,16 +35,17 @@ cudaError_t launch_group(const EvalArgs<T> &a, const EvalArgs<T> *ga, int K, con
     if (K < 1 || K > kGroupMax || !grouped_ok(ks, a)) return cudaErrorInvalidValue;
     const long long R = (long long)a.n0 * a.n1;
     const int nrt = (int)(((R + 1) / 2 + a.Brow - 1) / a.Brow);
-    auto launch = [&](const void *k, int bps, int nt, size_t smem) {
-        void *args[] = {(void *)&ga, (void *)&bps};
-        return cudaLaunchKernel(k, dim3((unsigned)(K * bps)), dim3(nt), args, smem, s);
+    // (the any-length kernels take the single form's arguments first)
+    auto launch = [&](const void *k, int bps, int nt, size_t smem, int any) {
+        void *args[] = {(void *)&a, (void *)&ga, (void *)&bps};
+        return cudaLaunchKernel(k, dim3((unsigned)(K * bps)), dim3(nt), any ? args : args + 1, smem, s);
     };
     group_clear_kernel<T><<<1, 4 * kGroupMax, 0, s>>>(ga, K);
     stats_group<T><<<K * a.nb_stats, 256, 0, s>>>(ga, a.nb_stats);   // (each evaluation's last block: knots)
     cudaError_t e = cudaSuccess;
-    if (a.nfwd > 0 && (e = launch(ks.row_fwd_g, nrt, a.thr_rowf, rowf_smem<T>(a)))) return e;
+    if (a.nfwd > 0 && (e = launch(ks.row_fwd_g, nrt, a.thr_rowf, rowf_smem<T>(a), a.any2))) return e;
     if (a.ncol > 0 &&
-        (e = launch(ks.pen_fwd_g, (int)pencil_tiles(a, a.ncol), a.thr_p1, pencil_smem_bytes<T>(a.n1, a.TW1))))
+        (e = launch(ks.pen_fwd_g, (int)pencil_tiles(a, a.ncol), a.thr_p1, pen_smem(a), a.any1)))
         return e;
     if (ks.recip.k) {
         if (!maps) return cudaErrorInvalidValue;
@@ -56,13 +57,13 @@ cudaError_t launch_group(const EvalArgs<T> &a, const EvalArgs<T> *ga, int K, con
                              args, ks.recip.smem, s);
     } else {
         e = launch(a.mgp_tab ? ks.axis0_mgp_g : ks.axis0_g, a.nb_ax0, a.thr_ax0,
-                   axis0_smem_bytes<T>(a.n0, a.TW0, a.ax0_scr));
+                   ax0_smem(a), a.any0);
     }
     if (e) return e;
     if (a.ncol_inv > 0 &&
-        (e = launch(ks.pen_inv_g, (int)pencil_tiles(a, a.ncol_inv), a.thr_p1, pencil_smem_bytes<T>(a.n1, a.TW1))))
+        (e = launch(ks.pen_inv_g, (int)pencil_tiles(a, a.ncol_inv), a.thr_p1, pen_smem(a), a.any1)))
         return e;
-    if ((e = launch(ks.row_inv_g, nrt, a.thr_rowi, rowi_smem<T>(a)))) return e;
+    if ((e = launch(ks.row_inv_g, nrt, a.thr_rowi, rowi_smem<T>(a), a.any2))) return e;
     finalize_group<T><<<K * 5, 256, 0, s>>>(ga, 5);
     return cudaGetLastError();
 }

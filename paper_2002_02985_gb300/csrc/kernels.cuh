@@ -1087,13 +1087,22 @@ __device__ __forceinline__ void row_inv_body(const EvalArgs<T> &a, const int bid
 template <typename T, int N, int G, int NT, int MAXR, int MINB>
 struct RowPolicy2 {
     typedef typename Vec2<T>::type C;
+    static constexpr bool ct = true;
     static constexpr int N_ = N, G_ = G, NT_ = NT, LD = (G % 2) ? G : G + 1;
     // each of the two buffers (the batch and the out-of-place transform's scratch) holds
     // N x LD elements and, when used as staging, G pairs of half-spectrum rows
     static constexpr int SCR = (N * LD > G * (N + 2)) ? N * LD : G * (N + 2);
     static constexpr int E = (N + NT - 1) / NT;      // elements (pairs of points) per thread
     static constexpr int min_blocks = MINB;
-    template <int DIR> __device__ static C *fft(C *x, C *y, const C *tw) {
+    __device__ static constexpr int n(const EvalArgs<T> &) { return N; }
+    __device__ static constexpr int Gn(const EvalArgs<T> &) { return G; }
+    __device__ static constexpr int Ld(const EvalArgs<T> &) { return LD; }
+    __device__ static constexpr int Scr(const EvalArgs<T> &) { return SCR; }
+    __device__ static constexpr int Nt() { return NT; }
+    // index / (n/2 + 1) and index / (n + 2) of the half-spectrum loops
+    __device__ static constexpr int slot(const EvalArgs<T> &, int idx) { return idx / (N / 2 + 1); }
+    __device__ static constexpr int slot2(const EvalArgs<T> &, int idx) { return idx / (2 * (N / 2 + 1)); }
+    template <int DIR> __device__ static C *fft(C *x, C *y, const EvalArgs<T> &, const C *tw) {
         return ct::fft_oop<DIR, N, G, LD, NT, MAXR>(x, y, tw);
     }
 };
@@ -1101,11 +1110,12 @@ struct RowPolicy2 {
 template <typename T, class Q>
 __device__ __forceinline__ void row_fwd2_body(const EvalArgs<T> &a, const int bid, const int nblk) {
     typedef typename Vec2<T>::type C;
-    constexpr int n = Q::N_, G = Q::G_, LD = Q::LD, NT = Q::NT_, E = Q::E, n2h = n / 2 + 1;
+    constexpr int E = Q::E;
+    const int n = Q::n(a), G = Q::Gn(a), LD = Q::Ld(a), NT = Q::Nt(), n2h = n / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tw = (C *)smem_raw;
-    C *buf = tw + n;                 // the channel batch, formed here
-    C *scr = buf + Q::SCR;           // scratch of the out-of-place transform
+    C *buf = tw + (Q::ct ? n : 0);                 // the channel batch, formed here
+    C *scr = buf + Q::Scr(a);           // scratch of the out-of-place transform
     __shared__ T sk[OFDFT_MAX_KNOTS], sdk[OFDFT_MAX_KNOTS];
     __shared__ int sch[kMaxChan], skpos;
     const long long R = (long long)a.n0 * a.n1;
@@ -1122,7 +1132,8 @@ __device__ __forceinline__ void row_fwd2_body(const EvalArgs<T> &a, const int bi
 #pragma unroll
         for (int s = 0; s < 2; s++) xr[q][s] = (e < n && (s == 0 || has1)) ? a.rho[(row0 + s) * n + e] : (T)0;
     }
-    for (int i = threadIdx.x; i < n; i += NT) tw[i] = a.tw2[i];
+    if constexpr (Q::ct)
+        for (int i = threadIdx.x; i < n; i += NT) tw[i] = a.tw2[i];
     if (lwt)
         for (int i = threadIdx.x; i < M; i += NT) {
             sk[i] = a.knots_t[i];
@@ -1183,18 +1194,30 @@ __device__ __forceinline__ void row_fwd2_body(const EvalArgs<T> &a, const int bi
             const int e = threadIdx.x + q * NT;
             if (e < n) {
                 C *row = buf + e * LD;
-#pragma unroll
-                for (int s = 0; s < G; s++) {
-                    const int ci = g0 + s;
-                    C v = cmake<C>((T)0, (T)0);
-                    if (ci < kpos && ci < nf) {
-                        const int ch = sch[ci];
-                        if (ch == CH_HPP) v = cmake<C>(vh[q][0], vh[q][1]);
-                        else if (ch == CH_VW) v = cmake<C>(vv[q][0], vv[q][1]);
-                        else if (ch == CH_NL) v = cmake<C>(vb[q][0], vb[q][1]);
-                        else v = cmake<C>(fa[q][0], fa[q][1]);          // WT: rho^alpha
+                if constexpr (!Q::ct) {
+                    const int sem = kpos - g0 < 0 ? 0 : (kpos - g0 < gact ? kpos - g0 : gact);
+                    for (int s = 0; s < sem; s++) {
+                        const int ch = sch[g0 + s];
+                        row[s] = ch == CH_HPP  ? cmake<C>(vh[q][0], vh[q][1])
+                                 : ch == CH_VW ? cmake<C>(vv[q][0], vv[q][1])
+                                 : ch == CH_NL ? cmake<C>(vb[q][0], vb[q][1])
+                                               : cmake<C>(fa[q][0], fa[q][1]);   // WT: rho^alpha
                     }
-                    row[s] = v;
+                    for (int s = sem; s < G; s++) row[s] = cmake<C>((T)0, (T)0);
+                } else {
+#pragma unroll
+                    for (int s = 0; s < G; s++) {
+                        const int ci = g0 + s;
+                        C v = cmake<C>((T)0, (T)0);
+                        if (ci < kpos && ci < nf) {
+                            const int ch = sch[ci];
+                            if (ch == CH_HPP) v = cmake<C>(vh[q][0], vh[q][1]);
+                            else if (ch == CH_VW) v = cmake<C>(vv[q][0], vv[q][1]);
+                            else if (ch == CH_NL) v = cmake<C>(vb[q][0], vb[q][1]);
+                            else v = cmake<C>(fa[q][0], fa[q][1]);          // WT: rho^alpha
+                        }
+                        row[s] = v;
+                    }
                 }
                 if (kpos < nf) {
 #pragma unroll
@@ -1207,13 +1230,13 @@ __device__ __forceinline__ void row_fwd2_body(const EvalArgs<T> &a, const int bi
             }
         }
         __syncthreads();
-        const C *Z = Q::template fft<-1>(buf, scr, tw);
+        const C *Z = Q::template fft<-1>(buf, scr, a, tw);
         // unpack X_2p[k] = (Z_k + conj Z_{n-k})/2, X_2p+1[k] = (Z_k - conj Z_{n-k})/(2i)
         // (plain stores: staging for bulk stores measured slower here)
         for (int idx = threadIdx.x; idx < gact * n2h; idx += NT) {
-            const int s = idx / n2h, k = idx - s * n2h;
+            const int s = Q::slot(a, idx), k = idx - s * n2h;
             const C A = Z[k * LD + s];
-            const C Bv = Z[((n - k) % n) * LD + s];
+            const C Bv = Z[(k ? n - k : 0) * LD + s];
             C *out = a.chan + (size_t)sch[g0 + s] * a.NH + row0 * n2h + k;
             out[0] = cmake<C>((T)0.5 * (A.x + Bv.x), (T)0.5 * (A.y - Bv.y));
             if (has1) out[n2h] = cmake<C>((T)0.5 * (A.y + Bv.y), (T)0.5 * (Bv.x - A.x));
@@ -1225,11 +1248,12 @@ __device__ __forceinline__ void row_fwd2_body(const EvalArgs<T> &a, const int bi
 template <typename T, class Q>
 __device__ __forceinline__ void row_inv2_body(const EvalArgs<T> &a, const int bid, const int nblk) {
     typedef typename Vec2<T>::type C;
-    constexpr int n = Q::N_, G = Q::G_, LD = Q::LD, NT = Q::NT_, E = Q::E, n2h = n / 2 + 1;
+    constexpr int E = Q::E;
+    const int n = Q::n(a), G = Q::Gn(a), LD = Q::Ld(a), NT = Q::Nt(), n2h = n / 2 + 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *tw = (C *)smem_raw;
-    C *buf = tw + n;                 // the packed channel batch
-    C *scr = buf + Q::SCR;           // scratch of the out-of-place transform; stages the raw rows
+    C *buf = tw + (Q::ct ? n : 0);                 // the packed channel batch
+    C *scr = buf + Q::Scr(a);           // scratch of the out-of-place transform; stages the raw rows
     __shared__ double sd[32];
     __shared__ __align__(8) uint64_t mbar;
     __shared__ int s_ok;
@@ -1266,7 +1290,8 @@ __device__ __forceinline__ void row_inv2_body(const EvalArgs<T> &a, const int bi
 #pragma unroll
         for (int s = 0; s < 2; s++) xr[q][s] = (e < n && (s == 0 || has1)) ? a.rho[(row0 + s) * n + e] : (T)0;
     }
-    for (int i = threadIdx.x; i < n; i += NT) tw[i] = a.tw2[i];
+    if constexpr (Q::ct)
+        for (int i = threadIdx.x; i < n; i += NT) tw[i] = a.tw2[i];
     if (lwt)
         for (int i = threadIdx.x; i < M; i += NT) {
             sk[i] = a.knots_t[i];
@@ -1376,7 +1401,7 @@ __device__ __forceinline__ void row_inv2_body(const EvalArgs<T> &a, const int bi
             phase ^= 1u;
         } else {
             for (int idx = threadIdx.x; idx < gact * 2 * n2h; idx += NT) {
-                const int s = idx / (2 * n2h), j = idx - s * 2 * n2h;
+                const int s = Q::slot2(a, idx), j = idx - s * 2 * n2h;
                 const bool ok = j < n2h || has1;
                 cp_async<sizeof(C)>(scr + idx, a.chan + (size_t)sch[g0 + s] * a.NH + (ok ? row0 * n2h + j : 0), ok);
             }
@@ -1386,7 +1411,7 @@ __device__ __forceinline__ void row_inv2_body(const EvalArgs<T> &a, const int bi
         }
         // pack each pair of half-spectrum rows into one full complex spectrum
         for (int idx = threadIdx.x; idx < gact * n2h; idx += NT) {
-            const int s = idx / n2h, k = idx - s * n2h;
+            const int s = Q::slot(a, idx), k = idx - s * n2h;
             const C X0 = scr[2 * s * n2h + k];
             const C X1 = scr[(2 * s + 1) * n2h + k];
             if (k == 0 || 2 * k == n) {
@@ -1397,7 +1422,7 @@ __device__ __forceinline__ void row_inv2_body(const EvalArgs<T> &a, const int bi
             }
         }
         __syncthreads();
-        const C *Z = Q::template fft<+1>(buf, scr, tw);
+        const C *Z = Q::template fft<+1>(buf, scr, a, tw);
 #pragma unroll
         for (int q = 0; q < E; q++) {
             const int e = threadIdx.x + q * NT;
