@@ -191,7 +191,10 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     pencil_any_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
     int bid;
     const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
-    pencil_any_body<T, DIR>(ar, bid);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int f = DIR > 0 ? ar.fin : 0;
+    if (f && bid == 0) energies_block(ar, (double *)smem_raw);
+    else pencil_any_body<T, DIR>(ar, bid - f);
 }
 
 // ---------------------------------------------------------------- reciprocal-space pass

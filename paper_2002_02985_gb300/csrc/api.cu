@@ -200,6 +200,9 @@ int fail(ofdft_grid *g, int code, const char *what, cudaError_t e = cudaSuccess)
     } while (0)
 
 static_assert(E_NUM == OFDFT_N_ENERGIES, "energy slots");
+constexpr long long kFormTableMax = 32LL << 20;   // doubles of the kept form-factor tables
+constexpr int kEnergySlot = 24;      // the energies' place behind the scalar slots (one copy fetches both)
+static_assert(S_FIN + 5 <= kEnergySlot, "scalar slots");
 
 // every device allocation of a grid goes through here: the optional cap of
 // ofdft_set_option(OFDFT_OPTION_ALLOC_CAP) is checked first (out of memory past it)
@@ -459,7 +462,7 @@ template <typename T> int ensure_ws(ofdft_grid *g, int nslots) {
         }
         CK(gmalloc(g, &w.scal, 64 * sizeof(double)), "cudaMalloc scalars");
         CK(cudaMemset(w.scal, 0, 64 * sizeof(double)), "memset");
-        CK(gmalloc(g, &w.energies, 8 * sizeof(double)), "cudaMalloc energies");
+        w.energies = w.scal + kEnergySlot;
         CK(gmalloc(g, &w.knots_d, OFDFT_MAX_KNOTS * sizeof(double)), "cudaMalloc knots");
         CK(gmalloc(g, &w.knots_t, OFDFT_MAX_KNOTS * sizeof(T)), "cudaMalloc knots");
         CK(gmalloc(g, &w.invdk_t, OFDFT_MAX_KNOTS * sizeof(T)), "cudaMalloc knots");
@@ -490,7 +493,6 @@ template <typename T> void free_ws(Workspace<T> &w) {
     for (int a = 0; a < 3; a++) cudaFree(w.tw[a]);
     cudaFree(w.vext);
     cudaFree(w.scal);
-    cudaFree(w.energies);
     cudaFree(w.knots_d);
     cudaFree(w.knots_t);
     cudaFree(w.invdk_t);
@@ -785,6 +787,12 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
     return OFDFT_OK;
 }
 
+// blocks of the stats kernel: a thread reads four points at a time, and a small grid makes no
+// more blocks than it has work for (their partials are summed by one block)
+int stats_blocks(const ofdft_grid *g) {
+    return (int)std::min<long long>(2 * g->nsm, (g->N + 1023) / 1024);
+}
+
 // the any-length plans of an evaluation or a plain transform (its rows are not any-length)
 template <typename T> void any_args_of(const ofdft_grid *g, const Workspace<T> &w, EvalArgs<T> &a) {
     a.any0 = w.any0;
@@ -890,7 +898,8 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     a.part_row = w.part_row;
     a.energies = E_dev_out ? E_dev_out : w.energies;
     a.ticket = w.ticket;
-    a.nb_stats = 2 * g->nsm;
+    a.nb_stats = stats_blocks(g);
+    a.clear_flags = 1;
     a.nb_ax0 = w.ks.recip.k ? w.recip_grid : w.tile_nb_ax0;
     a.nb_row = (int)((((long long)g->n[0] * g->n[1] + 1) / 2 + w.Brow - 1) / w.Brow);   // the row kernels' grid
     a.p0 = g->plan[0];
@@ -958,6 +967,8 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
             }
         }
     }
+    // the energies ride on the inverse pencils unless E_NL is a real-space sum
+    a.fin = a.ncol_inv > 0 && !(lwt && !exact);
     if (w.any2) choose_any_rows<T>(w, a);
     if (w.ks.recip.k && (w.maps_chan != w.chan || w.maps_vext != w.vext || w.maps_nslots != w.nslots ||
                          w.maps_tw != w.ks.recip.tw)) {
@@ -986,9 +997,6 @@ template <typename T> int upload_knots(ofdft_grid *g, const EvalArgs<T> &a, cons
 // Enqueue one evaluation with filled arguments on g->stream.
 template <typename T> int eval_launch(ofdft_grid *g, const EvalArgs<T> &a, const ofdft_functional *f) {
     Workspace<T> &w = ws<T>(g);
-    // clears the bad-density flag, the WT kF (recomputed) and the device-wait counters
-    static_assert(S_TIMEOUT == S_BAD + 2 && S_FATAL == S_BAD + 3, "flag slots");
-    CK(cudaMemsetAsync(a.scal + S_BAD, 0, 4 * sizeof(double), g->stream), "memset flags");
     if (int rc = upload_knots<T>(g, a, f)) return rc;
     ProfHook hook{prof_record, g};
     CK(launch_eval<T>(a, w.ks, g->stream, g->prof_on ? &hook : nullptr, w.ks.recip.k ? &w.maps : nullptr),
@@ -1020,13 +1028,12 @@ int eval_sync(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     int rc = enqueue_eval<T>(g, rho, f, V, nullptr);
     if (rc) return rc;
     Workspace<T> &w = ws<T>(g);
-    CK(cudaMemcpyAsync(g->h_pinned, w.energies, E_NUM * sizeof(double), cudaMemcpyDeviceToHost, g->stream), "copy E");
-    CK(cudaMemcpyAsync(g->h_pinned + 8, w.scal, S_NSCAL * sizeof(double), cudaMemcpyDeviceToHost, g->stream),
-       "copy scalars");
+    CK(cudaMemcpyAsync(g->h_pinned, w.scal, (kEnergySlot + E_NUM) * sizeof(double), cudaMemcpyDeviceToHost, g->stream),
+       "copy scalars and energies");
     CK(cudaStreamSynchronize(g->stream), "stream synchronize");
-    if ((rc = wait_status(g, g->h_pinned + 8))) return rc;
-    if (g->h_pinned[8 + S_BAD] != 0.0) return fail(g, OFDFT_ERR_BAD_DENSITY, "density has NaN/Inf or negative values");
-    if (E_out) std::memcpy(E_out, g->h_pinned, E_NUM * sizeof(double));
+    if ((rc = wait_status(g, g->h_pinned))) return rc;
+    if (g->h_pinned[S_BAD] != 0.0) return fail(g, OFDFT_ERR_BAD_DENSITY, "density has NaN/Inf or negative values");
+    if (E_out) std::memcpy(E_out, g->h_pinned + kEnergySlot, E_NUM * sizeof(double));
     return OFDFT_OK;
 }
 
@@ -1042,7 +1049,7 @@ template <typename T> EvalArgs<T> plain_args(ofdft_grid *g, Workspace<T> &w, con
     a.scal = w.scal; a.knots_d = w.knots_d; a.knots_t = w.knots_t; a.invdk_t = w.invdk_t;
     a.part_stats = w.part_stats; a.part_minmax = w.part_minmax; a.energies = w.energies; a.ticket = w.ticket;
     a.part_ax0 = w.part_ax0; a.part_row = w.part_row;
-    a.nb_stats = 2 * g->nsm; a.nb_ax0 = w.nb_ax0; a.nb_row = w.nb_row;
+    a.nb_stats = stats_blocks(g); a.nb_ax0 = w.nb_ax0; a.nb_row = w.nb_row;
     a.p0 = g->plan[0]; a.p1 = g->plan[1]; a.p2 = g->plan[2];
     a.tw0 = w.tw[0]; a.tw1 = w.tw[1]; a.tw2 = w.tw[2];
     a.Brow = w.Brow_p; a.thr_rowf = w.thr_rowf_p; a.thr_rowi = w.thr_rowi_p;
@@ -2202,7 +2209,7 @@ template <typename T> std::vector<unsigned char> launch_signature(const LaunchSe
     const int v[] = {a.n0,       a.n1,       a.n2,    a.nb_stats, a.nb_ax0, a.nb_row, a.Brow,     a.thr_rowf,
                      a.thr_rowi, a.TW1,      a.thr_p1, tile[0],   tile[1],  tile[2],  a.grid_p1,  a.row2_G,
                      a.nfwd,     a.ncol,     a.ncol_inv, a.exact_sums, a.mgp_tab != nullptr,
-                     a.any0,     a.any1,     a.any2,  a.lg0,      a.lg1,    a.any_G[0], a.any_G[1]};
+                     a.any0,     a.any1,     a.any2,  a.lg0,      a.lg1,    a.any_G[0], a.any_G[1], a.fin};
     append_bytes(k, v);
     return k;
 }
@@ -2246,7 +2253,7 @@ int make_plan(ofdft_grid *g0, int n, ofdft_grid *const *grids, const std::vector
     for (int gi = 0; gi < ng; gi++) {
         const EvalArgs<T> &a = args[p.order[p.gbeg[gi]]];
         const int K = p.gbeg[gi + 1] - p.gbeg[gi];
-        p.launches += (K > 1 ? 1 : 0) + 4 + (a.nfwd > 0) + (a.ncol > 0) + (a.ncol_inv > 0);
+        p.launches += 3 + (a.fin ? 0 : 1) + (a.nfwd > 0) + (a.ncol > 0) + (a.ncol_inv > 0);
         const bool recip = ws<T>(grids[p.order[p.gbeg[gi]]]).ks.recip.k != nullptr;
         std::snprintf(buf, sizeof(buf), "%s %dx%dx%d x%d%s", gi ? "," : "", a.n0, a.n1, a.n2, K,
                       K > 1 ? (recip ? " (grouped, persistent recip)" : " (grouped)") : "");

@@ -9,10 +9,10 @@
 //   axis0     FFT along n0, the reciprocal-space products (Hartree, PP, vW,
 //             per-knot kernels K_j(G), s2 and s3), FP64 energy partials, and
 //             the inverse FFT along n0
-//   pencil    inverse complex FFT along n1
+//   pencil    inverse complex FFT along n1; its first block makes the FP64 energies in a fixed order
 //   row_inv   complex-to-real FFT along n2 fused with the s4 spline blend and
 //             the assembly of V; FP64 partial of E_NL
-//   finalize  1 block: FP64 energies in a fixed order
+//   finalize  the energies instead, where E_NL is a real-space sum or nothing is transformed
 #pragma once
 
 #include <vector>
@@ -98,6 +98,8 @@ template <typename T> struct EvalArgs {
     int any0, any1, any2, lg0, lg1, any_G[2];
     AnyPlan q0, q0i, q1, q2;
     unsigned magic_n2h, magic_2n2h, magic_G[2];
+    int clear_flags;                     // an evaluation (its stats kernel sets the flags), not a plain transform
+    int fin;                             // the inverse n1 pencils' launch has a block 0 that makes the energies
     C *rhohat_out;                       // if set: the normalised rho_hat (Hartree/PP channel) for the forces
     int nfwd, fwd_ch[kMaxChan];          // channels formed by row_fwd (slot ids)
     int ncol, col_ch[kMaxChan];          // channels transformed forward along n1
@@ -130,8 +132,10 @@ template <typename T> __host__ __device__ inline size_t row_fwd_smem_bytes(int n
 }
 template <typename T> __host__ __device__ inline size_t pencil_smem_bytes(int n, int TW) {
     typedef typename Vec2<T>::type C;
-    // twiddles + two tile buffers (prefetch ping-pong) + the transform's scratch
-    return (size_t)n * sizeof(C) + 3 * (size_t)n * TW * sizeof(C);
+    // twiddles + two tile buffers (prefetch ping-pong) + the transform's scratch (at least the
+    // 1 KB of the block that makes the energies)
+    const size_t b = (size_t)n * sizeof(C) + 3 * (size_t)n * TW * sizeof(C);
+    return b > 1024 ? b : 1024;
 }
 
 // Whether the size-specialised reciprocal-space kernel for n0 = n transforms out of place
@@ -172,7 +176,8 @@ template <typename T> __host__ __device__ inline size_t rowi_smem(const EvalArgs
 // any-length pencils: one tile per exchange (three passes: two); the any-length
 // reciprocal-space pass: two load buffers and the exchange tile
 template <typename T> inline size_t any_pencil_smem(const AnyPlan &q, int lg) {
-    return ((size_t)(q.np > 2 ? 2 : 1) * q.n << lg) * 2 * sizeof(T);
+    const size_t b = ((size_t)(q.np > 2 ? 2 : 1) * q.n << lg) * 2 * sizeof(T);
+    return b > 1024 ? b : 1024;
 }
 template <typename T> inline size_t any_axis0_smem(int n, int lg) { return ((size_t)3 * n << lg) * 2 * sizeof(T); }
 template <typename T> inline size_t pen_smem(const EvalArgs<T> &a) {

@@ -111,8 +111,7 @@ cudaError_t launch_eval(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t 
     mark(K_AXIS0, 1);
     if (a.ncol_inv > 0) {
         mark(K_PENCIL_INV, 0);
-        e = launch(ks.pen_inv, dim3(pencil_tiles(a, a.ncol_inv)), a.thr_p1, pen_smem(a),
-                   a, s);
+        e = launch(ks.pen_inv, dim3(pencil_tiles(a, a.ncol_inv) + a.fin), a.thr_p1, pen_smem(a), a, s);
         if (e) return e;
         mark(K_PENCIL_INV, 1);
     }
@@ -120,9 +119,11 @@ cudaError_t launch_eval(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t 
     e = launch(ks.row_inv, dim3(nrt), a.thr_rowi, rowi_smem<T>(a), a, s);
     if (e) return e;
     mark(K_ROW_INV, 1);
-    mark(K_FINALIZE, 0);
-    finalize_kernel<T><<<5, 256, 0, s>>>(a);
-    mark(K_FINALIZE, 1);
+    if (!a.fin) {
+        mark(K_FINALIZE, 0);
+        finalize_kernel<T><<<5, 256, 0, s>>>(a);
+        mark(K_FINALIZE, 1);
+    }
     return cudaGetLastError();
 }
 

@@ -22,13 +22,6 @@ template <typename T> bool grouped_ok(const LaunchSet &ks, const EvalArgs<T> &a)
     return (a.mgp_tab ? ks.axis0_mgp_g : ks.axis0_g) != nullptr;
 }
 
-// Clears the per-evaluation flags (bad density, the WT kF, the device-wait counters): the
-// grouped form of the single evaluation's flag memset.
-template <typename T> __global__ void group_clear_kernel(const EvalArgs<T> *__restrict__ ga, int K) {
-    const int k = threadIdx.x >> 2, i = threadIdx.x & 3;
-    if (k < K) ga[k].scal[S_BAD + i] = 0.0;
-}
-
 template <typename T>
 cudaError_t launch_group(const EvalArgs<T> &a, const EvalArgs<T> *ga, int K, const LaunchSet &ks, cudaStream_t s,
                          const RecipMaps *maps) {
@@ -40,7 +33,6 @@ cudaError_t launch_group(const EvalArgs<T> &a, const EvalArgs<T> *ga, int K, con
         void *args[] = {(void *)&a, (void *)&ga, (void *)&bps};
         return cudaLaunchKernel(k, dim3((unsigned)(K * bps)), dim3(nt), any ? args : args + 1, smem, s);
     };
-    group_clear_kernel<T><<<1, 4 * kGroupMax, 0, s>>>(ga, K);
     stats_group<T><<<K * a.nb_stats, 256, 0, s>>>(ga, a.nb_stats);   // (each evaluation's last block: knots)
     cudaError_t e = cudaSuccess;
     if (a.nfwd > 0 && (e = launch(ks.row_fwd_g, nrt, a.thr_rowf, rowf_smem<T>(a), a.any2))) return e;
@@ -61,10 +53,10 @@ cudaError_t launch_group(const EvalArgs<T> &a, const EvalArgs<T> *ga, int K, con
     }
     if (e) return e;
     if (a.ncol_inv > 0 &&
-        (e = launch(ks.pen_inv_g, (int)pencil_tiles(a, a.ncol_inv), a.thr_p1, pen_smem(a), a.any1)))
+        (e = launch(ks.pen_inv_g, (int)pencil_tiles(a, a.ncol_inv) + a.fin, a.thr_p1, pen_smem(a), a.any1)))
         return e;
     if ((e = launch(ks.row_inv_g, nrt, a.thr_rowi, rowi_smem<T>(a), a.any2))) return e;
-    finalize_group<T><<<K * 5, 256, 0, s>>>(ga, 5);
+    if (!a.fin) finalize_group<T><<<K * 5, 256, 0, s>>>(ga, 5);
     return cudaGetLastError();
 }
 

@@ -286,55 +286,101 @@ __device__ __forceinline__ bool in_knot_range(const EvalArgs<T> &a, T xf, T kf, 
 
 // ======================================================================= knots (s1)
 // FP64 reduction of the stats partials (read through L2: they were written by
-// other blocks of the same launch), the mean density, E_TF, and the M knots
-// between kF(min rho) and kF(max rho).  Called by the last stats block.
-template <typename T>
-__device__ __forceinline__ void knots_from_partials(const EvalArgs<T> &a, double *sd, T *st) {
+// other blocks of the same launch), the mean density, E_TF, the flags, and the M knots
+// between kF(min rho) and kF(max rho).  Called by the last stats block (256 threads).
+//
+// GB300 issues about two FP64 operations per clock per SM, so this serial tail is bound by
+// the latency of its FP64 chains.  They run side by side in different warps: warp 0 takes the
+// two cube roots, warp 1 the logarithm (of the density ratio: ln(kmax/kmin) is a third of it,
+// so it does not wait for the roots) and the M exponentials, warps 2 to 4 one sum each.
+// (one chain after the other took 11 us of the kernel's 27 at 128^3)
+template <typename T> __device__ __forceinline__ void knots_from_partials(const EvalArgs<T> &a) {
     __shared__ double kn[OFDFT_MAX_KNOTS];
-    __shared__ double smm[2];
-    double s_rho = 0.0, s_tf = 0.0, s_xc = 0.0;
+    __shared__ T wmn[8], wmx[8];
+    __shared__ double kend[2];
+    __shared__ int any_bad;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int M = a.M;
+    const bool lwt = (a.terms & 4u) && a.kernel == 0 && M >= 2;
+    if (threadIdx.x == 0) any_bad = 0;
+    // warps 2..4: the terms of one sum each, requested before the extrema are awaited
+    double sum = 0.0;
+    if (warp >= 2 && warp < 5)
+        for (int b = lane; b < a.nb_stats; b += 32) sum += __ldcg(a.part_stats + 3 * b + (warp - 2));
     T mn = (T)3.0e38, mx = (T)-3.0e38;
+    int bad = 0;
     for (int b = threadIdx.x; b < a.nb_stats; b += blockDim.x) {
-        s_rho += __ldcg(a.part_stats + 3 * b);
-        s_tf += __ldcg(a.part_stats + 3 * b + 1);
-        s_xc += __ldcg(a.part_stats + 3 * b + 2);
         const T x = __ldcg(a.part_minmax + 2 * b), y = __ldcg(a.part_minmax + 2 * b + 1);
+        if (!(x == x)) bad = 1;                       // (a block that saw a bad value leaves NaN)
         mn = x < mn ? x : mn;
         mx = y > mx ? y : mx;
     }
-    double r[3] = {s_rho, s_tf, s_xc};
-    block_sum_n<3>(r, sd);
-    s_rho = r[0];
-    s_tf = r[1];
-    s_xc = r[2];
-    mn = block_min(mn, st);
-    mx = block_max(mx, st);
-    const double fl = (double)a.floor_;
-    if (threadIdx.x == 0) {
-        a.scal[S_SUM_RHO] = s_rho;
-        a.scal[S_SUM_TF] = s_tf;
-        a.scal[S_RHO_MIN] = (double)mn;
-        a.scal[S_RHO_MAX] = (double)mx;
-        const double mean = s_rho / (double)a.N;
-        a.scal[S_RHO_MEAN] = mean;
-        a.scal[S_KF_WT] = cbrt(kThreePi2 * (mean > fl ? mean : fl));
-        a.energies[E_TF] = (a.terms & 1u) ? kCTF * s_tf * a.dV : 0.0;
-        a.energies[E_XC] = (a.terms & 32u) ? s_xc * a.dV : 0.0;
-        smm[0] = (double)mn;
-        smm[1] = (double)mx;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const T x = __shfl_xor_sync(0xffffffffu, mn, o), y = __shfl_xor_sync(0xffffffffu, mx, o);
+        mn = x < mn ? x : mn;
+        mx = y > mx ? y : mx;
+    }
+    if (lane == 0) {
+        wmn[warp] = mn;
+        wmx[warp] = mx;
     }
     __syncthreads();
-    if (!((a.terms & 4u) && a.kernel == 0 && a.M >= 2)) return;
+    if (bad) any_bad = 1;
+#pragma unroll
+    for (int w = 0; w < 8; w++) {
+        mn = wmn[w] < mn ? wmn[w] : mn;
+        mx = wmx[w] > mx ? wmx[w] : mx;
+    }
+    const double fl = (double)a.floor_;
+    const double xmin = (double)mn > fl ? (double)mn : fl, xmax = (double)mx > fl ? (double)mx : fl;
+    if (warp == 0) {
+        if (lane < 2) kend[lane] = cbrt(kThreePi2 * (lane ? xmax : xmin));
+        if (lane == 2) {
+            a.scal[S_RHO_MIN] = (double)mn;
+            a.scal[S_RHO_MAX] = (double)mx;
+        }
+    } else if (warp == 1) {
+        if (lwt && !a.frozen && a.knot_spacing == 0) {
+            const double l = log(xmax / xmin) * (1.0 / 3.0) / (double)(M - 1);
+            for (int m = lane; m < M; m += 32) kn[m] = exp((double)m * l);
+        }
+    } else if (warp < 5) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0 && warp == 2) {
+            const double mean = sum / (double)a.N;
+            a.scal[S_SUM_RHO] = sum;
+            a.scal[S_RHO_MEAN] = mean;
+            if ((a.terms & 4u) && a.kernel != 0) a.scal[S_KF_WT] = cbrt(kThreePi2 * (mean > fl ? mean : fl));
+        } else if (lane == 0 && warp == 3) {
+            a.scal[S_SUM_TF] = sum;
+            a.energies[E_TF] = (a.terms & 1u) ? kCTF * sum * a.dV : 0.0;
+        } else if (lane == 0) {
+            a.energies[E_XC] = (a.terms & 32u) ? sum * a.dV : 0.0;
+        }
+    }
+    __syncthreads();
+    // the flags of the evaluation start here; a plain transform only reports bad values
+    if (threadIdx.x == 32 * 7) {
+        if (a.clear_flags) {
+            a.scal[S_BAD] = any_bad ? 1.0 : 0.0;
+            a.scal[S_TIMEOUT] = 0.0;
+            a.scal[S_FATAL] = 0.0;
+        } else if (any_bad) {
+            a.scal[S_BAD] = 1.0;
+        }
+    }
+    if (!lwt) return;
     // s1: one thread per knot, in FP64
-    const int M = a.M, m = threadIdx.x;
+    const int m = threadIdx.x;
     if (m < M) {
+        const double kmin = kend[0], kmax = kend[1];
         double k;
         if (!a.frozen) {
-            const double kmin = cbrt(kThreePi2 * (smm[0] > fl ? smm[0] : fl));
-            const double kmax = cbrt(kThreePi2 * (smm[1] > fl ? smm[1] : fl));
             if (m == 0) k = kmin;
             else if (m == M - 1) k = kmax;
-            else if (a.knot_spacing == 0) k = kmin * exp((double)m * (log(kmax / kmin) / (double)(M - 1)));
+            else if (a.knot_spacing == 0) k = kmin * kn[m];
             else k = kmin + (double)m * ((kmax - kmin) / (double)(M - 1));
             a.knots_d[m] = k;
         } else {
@@ -353,8 +399,9 @@ __device__ __forceinline__ void knots_from_partials(const EvalArgs<T> &a, double
 // ======================================================================= stats (s1 input)
 template <typename T, bool XS>
 __device__ __forceinline__ void stats_body(const EvalArgs<T> &a, const int bid, const int nblk) {
-    __shared__ double sd[3 * 32];
-    __shared__ T st[32];
+    __shared__ double sd[3][8];
+    __shared__ T smn[8], smx[8];
+    __shared__ int sbad[8];
     double s_rho = 0.0, s_tf = 0.0, s_xc = 0.0;
     T mn = (T)3.0e38, mx = (T)-3.0e38;
     int bad = 0;
@@ -423,28 +470,70 @@ __device__ __forceinline__ void stats_body(const EvalArgs<T> &a, const int bid, 
             s_xc += (double)x16;
         }
     }
+    // one exchange for the block's five results: warp sums (FP32 in the FP32-mixed path, as the
+    // terms), then lane k of warp 0 combines the warps' k-th result in FP64
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double r[3] = {s_rho, s_tf, s_xc};
-    if constexpr (sizeof(T) == 4 && !XS) block_sum_n_f32warp<3>(r, sd);
-    else block_sum_n<3>(r, sd);
-    if (threadIdx.x == 0)
-        for (int k = 0; k < 3; k++) a.part_stats[3 * bid + k] = r[k];
-    mn = block_min(mn, st);
-    if (threadIdx.x == 0) a.part_minmax[2 * bid] = mn;
-    mx = block_max(mx, st);
-    if (threadIdx.x == 0) a.part_minmax[2 * bid + 1] = mx;
-    bad = __syncthreads_or(bad);
-    if (threadIdx.x == 0 && bad) a.scal[S_BAD] = 1.0;
-    // the last block to finish reduces every block's partials and makes the knots (thread 0
-    // wrote this block's partials and flag, so only it orders them before the ticket)
+    if constexpr (sizeof(T) == 4 && !XS) {
+        float f[3] = {(float)s_rho, (float)s_tf, (float)s_xc};
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 3; k++) f[k] += __shfl_down_sync(0xffffffffu, f[k], o);
+#pragma unroll
+        for (int k = 0; k < 3; k++) r[k] = (double)f[k];
+    } else {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 3; k++) r[k] += __shfl_down_sync(0xffffffffu, r[k], o);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const T x = __shfl_down_sync(0xffffffffu, mn, o), y = __shfl_down_sync(0xffffffffu, mx, o);
+        mn = x < mn ? x : mn;
+        mx = y > mx ? y : mx;
+    }
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) {
+#pragma unroll
+        for (int k = 0; k < 3; k++) sd[k][warp] = r[k];
+        smn[warp] = mn;
+        smx[warp] = mx;
+        sbad[warp] = bad;
+    }
+    __syncthreads();
+    // the last block to finish reduces every block's partials and makes the knots
     __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        last = atomicAdd(a.ticket, 1u) == nblk - 1;
+    if (warp == 0) {
+        if (lane < 3) {
+            double t = 0.0;
+#pragma unroll
+            for (int w = 0; w < 8; w++) t += sd[lane][w];
+            a.part_stats[3 * bid + lane] = t;
+        } else if (lane == 3) {
+            int bb = 0;
+#pragma unroll
+            for (int w = 0; w < 8; w++) {
+                mn = smn[w] < mn ? smn[w] : mn;
+                bb |= sbad[w];
+            }
+            a.part_minmax[2 * bid] = bb ? (T)NAN : mn;
+        } else if (lane == 4) {
+#pragma unroll
+            for (int w = 0; w < 8; w++) mx = smx[w] > mx ? smx[w] : mx;
+            a.part_minmax[2 * bid + 1] = mx;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();
+            last = atomicAdd(a.ticket, 1u) == nblk - 1;
+        }
     }
     __syncthreads();
     if (!last) return;
     __threadfence();
-    knots_from_partials(a, sd, st);
+    knots_from_partials(a);
     if (threadIdx.x == 0) *a.ticket = 0u;           // ready for the next evaluation
 }
 
@@ -1522,6 +1611,36 @@ __device__ __forceinline__ void finalize_body(const EvalArgs<T> &a, const int bi
     *a.ticket = 0u;                                   // ready for the next evaluation
 }
 
+// The energies by one extra block of the inverse n1 pencils (block 0, so that it starts with
+// the first ones): the reciprocal-space partials are complete by then, and nothing later adds to
+// the energies unless E_NL is a real-space sum (interpolated LWT: the finalize kernel above).
+// A kernel of its own cost 8 to 10 us of every evaluation; here it hides behind the pencils.
+// (its scratch is the pencils' dynamic shared memory, at least 1 KB: a static array would take
+// from the tiles' share of the SM)
+template <typename T> __device__ __noinline__ void energies_block(const EvalArgs<T> &a, double *sd) {
+    double r[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < a.nb_ax0; b += blockDim.x) {
+        const double2 x = reinterpret_cast<const double2 *>(a.part_ax0)[2 * b];
+        const double2 y = reinterpret_cast<const double2 *>(a.part_ax0)[2 * b + 1];
+        r[0] += x.x;
+        r[1] += x.y;
+        r[2] += y.x;
+        r[3] += y.y;
+    }
+    block_sum_n<4>(r, sd);
+    if (threadIdx.x) return;
+    double *E = a.energies;
+    const double vw = (a.terms & 2u) ? 0.5 * a.omega * r[1] : 0.0;
+    const double h = (a.terms & 8u) ? 2.0 * kPi * a.omega * r[0] : 0.0;
+    const double p = (a.terms & 16u) ? a.omega * (r[2] + a.scal[S_RHO_MEAN] * (double)a.vext[0].x) : 0.0;
+    const double n = (a.terms & 4u) ? a.omega * r[3] : 0.0;
+    E[E_VW] = vw;
+    E[E_H] = h;
+    E[E_PP] = p;
+    E[E_NL] = n;
+    E[E_TOT] = E[E_TF] + vw + n + h + p + E[E_XC];
+}
+
 // ======================================================================= kernel wrappers
 // Single evaluation: the arguments in the kernel's parameter space, block b = blockIdx.x.
 template <typename T, bool XS = false>
@@ -1538,7 +1657,10 @@ __global__ void __launch_bounds__(P::max_threads, P::min_blocks) row_fwd_kernel(
 }
 template <typename T, int DIR, class P>
 __global__ void __launch_bounds__(P::max_threads, P::min_blocks) pencil1_kernel(EvalArgs<T> a) {
-    pencil1_body<T, DIR, P>(a, blockIdx.x, gridDim.x);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int f = DIR > 0 ? a.fin : 0;
+    if (f && blockIdx.x == 0) energies_block(a, (double *)smem_raw);
+    else pencil1_body<T, DIR, P>(a, (int)blockIdx.x - f, (int)gridDim.x - f);
 }
 // MGP: the knots' kernels of Eq. MGP from the correction table (a separate instantiation,
 // so that the Wang-Teter form carries no trace of it)
@@ -1586,7 +1708,10 @@ template <typename T, int DIR, class P>
 __global__ void __launch_bounds__(P::max_threads, P::min_blocks) pencil1_group(const EvalArgs<T> *__restrict__ ga,
                                                                                 int bps) {
     OFDFT_GROUP_INDEX;
-    pencil1_body<T, DIR, P>(ga[gk], gb, bps);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int f = DIR > 0 ? ga[gk].fin : 0;
+    if (f && gb == 0) energies_block(ga[gk], (double *)smem_raw);
+    else pencil1_body<T, DIR, P>(ga[gk], gb - f, bps - f);
 }
 template <typename T, class P, bool MGP = false>
 __global__ void __launch_bounds__(P::max_threads, P::min_blocks_ax0) axis0_group(const EvalArgs<T> *__restrict__ ga,
