@@ -133,6 +133,9 @@ struct ofdft_grid {
     float *gf = nullptr;         // per-species form-factor tables of the FP32-mixed force kernel
     long long gf_len = 0;
     bool gf_fresh = false;       // the tables match the current ions (species, Z, rc)
+    double *vf = nullptr;        // per-species v_s(|G|) / Omega in FP64 for the FP32 V_ext(G)
+    long long vf_len = 0;
+    bool vf_fresh = false;
     int *d_sp_ions = nullptr;    // the ions grouped by species (device), the groups' offsets (host)
     std::vector<int> sp_off;
     // smooth PME (ofdft_set_ions_pme): order > 0 selects it for V_ext(G) and forces
@@ -548,7 +551,24 @@ template <typename T> int ensure_vext(ofdft_grid *g) {
     }
     IonArgs a = ion_args(g);
     cudaError_t e;
-    if (sizeof(T) == 4) e = launch_vext(a, nullptr, (float2 *)w.vext, g->stream, g->ph32);
+    if (sizeof(T) == 4) {
+        // the species' form factors in FP64, kept while Z and rc stay (up to 256 MB)
+        const long long len = (long long)g->n_species * g->NH;
+        if (len <= kFormTableMax) {
+            if (g->vf_len < len) {
+                cudaFree(g->vf);
+                g->vf = nullptr;
+                g->vf_len = 0;
+                CK(gmalloc(g, &g->vf, (size_t)len * sizeof(double)), "cudaMalloc form factors");
+                g->vf_len = len;
+                g->vf_fresh = false;
+            }
+            if (!g->vf_fresh) CK(launch_form_tables(a, g->vf, g->stream), "form factors");
+            g->vf_fresh = true;
+        }
+        e = launch_vext(a, nullptr, (float2 *)w.vext, g->stream, g->ph32, g->d_sp_ions, g->sp_off.data(),
+                        len <= kFormTableMax ? g->vf : nullptr);
+    }
     else e = launch_vext(a, (double2 *)w.vext, nullptr, g->stream);
     CK(e, "structure factor kernel");
     fresh = true;
@@ -2746,6 +2766,7 @@ int ofdft_grid_destroy(ofdft_grid *g) {
     free_ws(g->w64);
     cudaFree(g->ph);
     cudaFree(g->ph32);
+    cudaFree(g->vf);
     cudaFree(g->gf);
     cudaFree(g->d_sp_ions);
     cudaFree(g->fpart);
@@ -2806,7 +2827,7 @@ int store_ions(ofdft_grid *g, const ofdft_ions *ions, const ofdft_species *sp) {
     // the force tables depend on the species' Z and rc only (not on positions)
     if (g->n_species != sp->n_species || !std::equal(g->Z.begin(), g->Z.end(), sp->Z) ||
         !std::equal(g->rc.begin(), g->rc.end(), sp->rc))
-        g->gf_fresh = false;
+        g->gf_fresh = g->vf_fresh = false;
     g->n_species = sp->n_species;
     g->pos.assign(ions->pos, ions->pos + 3 * (size_t)n);
     g->species.assign(ions->species, ions->species + n);
@@ -2842,27 +2863,9 @@ int ofdft_set_ions(ofdft_grid *g, const ofdft_ions *ions, const ofdft_species *s
         CK(gmalloc(g, &g->ph32, (size_t)n * (g->n[0] + g->n[1] + g->n2h) * sizeof(float2)), "cudaMalloc phases");
     }
     // per-axis phase tables e^{-2 pi i m_a f_a}, f = R . inv(cell) (fractional)
-    const int na[3] = {g->n[0], g->n[1], g->n2h};
-    std::vector<double2> ph((size_t)n * (na[0] + na[1] + na[2]));
-    size_t off = 0;
-    for (int ax = 0; ax < 3; ax++) {
-        for (int I = 0; I < n; I++) {
-            const double *R = &g->pos[3 * (size_t)I];
-            // fractional coordinate along a_ax: R . b_ax
-            const double fr = R[0] * g->recip[3 * ax] + R[1] * g->recip[3 * ax + 1] + R[2] * g->recip[3 * ax + 2];
-            for (int k = 0; k < na[ax]; k++) {
-                const int nn = g->n[ax];
-                const double m = (ax == 2) ? k : ((k <= nn / 2) ? k : k - nn);
-                double t = m * fr;
-                t -= std::floor(t);
-                const double ang = -2.0 * kPi * t;
-                ph[off + (size_t)I * na[ax] + k] = make_double2(std::cos(ang), std::sin(ang));
-            }
-        }
-        off += (size_t)n * na[ax];
-    }
-    CK(cudaMemcpy(g->ph, ph.data(), ph.size() * sizeof(double2), cudaMemcpyHostToDevice), "upload phases");
-    CK(launch_round_phases(g->ph, g->ph32, (long long)ph.size(), g->stream), "round phases");
+    if (!g->d_pos) CK(gmalloc(g, &g->d_pos, 3 * (size_t)n * sizeof(double)), "cudaMalloc positions");
+    CK(cudaMemcpy(g->d_pos, g->pos.data(), 3 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice), "upload positions");
+    CK(launch_phases(g->n, g->n2h, n, g->recip, g->d_pos, g->ph, g->ph32, g->stream), "phase tables");
     return OFDFT_OK;
 }
 

@@ -19,11 +19,16 @@ struct IonArgs {
     int charge_ff = 0;               // 1: form factor Z_s instead of v_s (Ewald: S_Z(G) and its forces)
 };
 
-// vext64 != null: FP64 build; otherwise the FP32 copy from FP32 phase products
-// (ph32 = FP32 copy of the phase tables) with FP64 accumulation of 8-ion groups
+// vext64 != null: FP64 build; otherwise the FP32 build from the FP32 phase tables ph32 over the
+// ions grouped by species (sp_ions, HOST offsets sp_off); vf = the FP64 tables of
+// launch_form_tables ([n_species][NH]: v_s(|G|) / Omega), or null to evaluate them in place
 cudaError_t launch_vext(const IonArgs &a, double2 *vext64, float2 *vext32, cudaStream_t s,
-                        const float2 *ph32 = nullptr);
-cudaError_t launch_round_phases(const double2 *in, float2 *out, long long n, cudaStream_t s);
+                        const float2 *ph32 = nullptr, const int *sp_ions = nullptr, const int *sp_off = nullptr,
+                        const double *vf = nullptr);
+cudaError_t launch_form_tables(const IonArgs &a, double *vf, cudaStream_t st);
+// the ions' phase tables (FP64 and FP32) from their Cartesian positions in device memory
+cudaError_t launch_phases(const int *n, int n2h, int n_ions, const double *recip, const double *pos, double2 *ph,
+                          float2 *ph32, cudaStream_t s);
 // FP32-mixed forces (separable form): gf = the per-species tables of launch_force_tables
 // ([n_species][NH] floats: -w v_s(|G|)); sp_ions = the ions grouped by species, sp_off (HOST)
 // the groups' offsets; partials [n_ions][nrb][3] (the S_a sums per row-tile block), then

@@ -53,61 +53,198 @@ __global__ void __launch_bounds__(256) vext_kernel(IonArgs a, double2 *v64, floa
     if (v32) v32[e] = make_float2((float)acc.x, (float)acc.y);
 }
 
-// FP32-mixed variant: the per-ion phase products e^{-iG.R} = P0 P1 P2 are formed
-// in FP32 from the FP64 tables rounded once; groups of 8 ions are summed in
-// FP32 and the groups in FP64 (GB300's FP64 rate is a small fraction of FP32's).
-__global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 *ph32, float2 *v32) {
+// v_s(|G|) / Omega of species s in FP64, once per set of species (positions do not enter)
+__global__ void __launch_bounds__(256) form_table_kernel(IonArgs a, double *vf, int s) {
     const long long NH = (long long)a.n0 * a.n1 * a.n2h;
     const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (e >= NH) return;
     double gx, gy, gz;
     int k0, k1, k2;
     gvec_of(a, e, gx, gy, gz, k0, k1, k2);
-    const double q2 = gx * gx + gy * gy + gz * gz;
-    const float2 *P0 = ph32, *P1 = ph32 + (size_t)a.n_ions * a.n0, *P2 = P1 + (size_t)a.n_ions * a.n1;
-    double ax = 0.0, ay = 0.0;
-    for (int s = 0; s < a.n_species; s++) {
-        double Sx = 0.0, Sy = 0.0;
-        float gxs = 0.f, gys = 0.f;
-        int cnt = 0;
-        for (int I = 0; I < a.n_ions; I++) {
-            if (a.species[I] != s) continue;
-            const float2 p0 = P0[(size_t)I * a.n0 + k0], p1 = P1[(size_t)I * a.n1 + k1], p2 = P2[(size_t)I * a.n2h + k2];
-            const float rx = p0.x * p1.x - p0.y * p1.y, ry = p0.x * p1.y + p0.y * p1.x;
-            gxs += rx * p2.x - ry * p2.y;
-            gys += rx * p2.y + ry * p2.x;
-            if (++cnt == 8) {
-                Sx += (double)gxs;
-                Sy += (double)gys;
-                gxs = gys = 0.f;
-                cnt = 0;
-            }
-        }
-        Sx += (double)gxs;
-        Sy += (double)gys;
-        const double v = pp_form(q2, a.Z[s], a.rc[s]) / a.omega;
-        ax += v * Sx;
-        ay += v * Sy;
-    }
-    v32[e] = make_float2((float)ax, (float)ay);
+    vf[e] = pp_form(gx * gx + gy * gy + gz * gz, a.Z[s], a.rc[s]) / a.omega;
 }
-
-cudaError_t launch_vext(const IonArgs &a, double2 *vext64, float2 *vext32, cudaStream_t s, const float2 *ph32) {
+cudaError_t launch_form_tables(const IonArgs &a, double *vf, cudaStream_t st) {
     const long long NH = (long long)a.n0 * a.n1 * a.n2h;
-    if (ph32 && vext32 && !vext64)
-        vext_fast_kernel<<<(unsigned)((NH + 255) / 256), 256, 0, s>>>(a, ph32, vext32);
-    else
-        vext_kernel<<<(unsigned)((NH + 255) / 256), 256, 0, s>>>(a, vext64, vext32);
+    for (int s = 0; s < a.n_species; s++)
+        form_table_kernel<<<(unsigned)((NH + 255) / 256), 256, 0, st>>>(a, vf + (size_t)s * NH, s);
     return cudaGetLastError();
 }
 
-// FP32 copy of the FP64 phase tables
-__global__ void round_phases_kernel(const double2 *in, float2 *out, long long n) {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = make_float2((float)in[i].x, (float)in[i].y);
+// FP32-mixed variant: S_s(G) is the complex product [rows (k0, k1) x ions] x [ions x k2] of
+// P01 = P0(k0) P1(k1) and P2(k2), formed in FP32 from the FP64 tables rounded once; groups of 8
+// ions are summed in FP32 and the groups as FP32 pairs (hi + lo, exact two-sums: about 48 bits,
+// without GB300's slow FP64 adds), the form factor and the sum over species in FP64.
+//
+// Block: kVR rows x kVK values of k2; the ions come kVI at a time through shared memory.  A thread
+// owns 4 rows x 4 k2, as two packed pairs of k2, so an ion costs 4 shared 16-byte reads for 32
+// packed FMAs.  One thread per G (three gathers of the tables per ion, FP64 group sums and the
+// form factor's exponential at every G) took 0.6 ms for 500 ions at 96^3.
+constexpr int kVR = 64, kVK = 64, kVI = 32;
+__device__ __forceinline__ void pair_add(float2 &hi, float2 &lo, float2 x) {
+    // two-sum of hi + x, component by component (Knuth): the rounding error goes into lo
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 s = __fadd2_rn(hi, x);
+    const float2 bb = __ffma2_rn(hi, m1, s);
+    const float2 e1 = __ffma2_rn(__ffma2_rn(bb, m1, s), m1, hi);
+    const float2 e2 = __ffma2_rn(bb, m1, x);
+    lo = __fadd2_rn(lo, __fadd2_rn(e1, e2));
+    hi = s;
 }
-cudaError_t launch_round_phases(const double2 *in, float2 *out, long long n, cudaStream_t s) {
-    round_phases_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(in, out, n);
+__global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 *ph32, const int *sp_ions, int s0,
+                                                        int s1, int s, const double *vf, float2 *v32, bool first) {
+    __shared__ __align__(16) float2 p01[kVI][kVR];
+    __shared__ __align__(16) float4 p2s[kVI][kVK / 2];        // P2 of k2 pairs: (re, re', im, im')
+    const int rows = a.n0 * a.n1, n2h = a.n2h;
+    const int r0 = blockIdx.x * kVR, kc = blockIdx.y * kVK;
+    const int tk = threadIdx.x & 15, tr = threadIdx.x >> 4;
+    const float2 *P0 = ph32, *P1 = ph32 + (size_t)a.n_ions * a.n0, *P2 = P1 + (size_t)a.n_ions * a.n1;
+    const float2 zero = make_float2(0.f, 0.f);
+    float2 hi[4][2][2], lo[4][2][2];                          // [row][k2 pair][re, im]
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+#pragma unroll
+        for (int p = 0; p < 2; p++) hi[j][p][0] = hi[j][p][1] = lo[j][p][0] = lo[j][p][1] = zero;
+    for (int i0 = s0; i0 < s1; i0 += kVI) {
+        __syncthreads();
+        for (int idx = threadIdx.x; idx < kVI * kVR; idx += 256) {
+            const int i = idx / kVR, r = idx - i * kVR;
+            float2 c = zero;
+            if (i0 + i < s1 && r0 + r < rows) {
+                const int I = sp_ions[i0 + i], k0 = (r0 + r) / a.n1, k1 = r0 + r - k0 * a.n1;
+                const float2 x = P0[(size_t)I * a.n0 + k0], y = P1[(size_t)I * a.n1 + k1];
+                c = make_float2(x.x * y.x - x.y * y.y, x.x * y.y + x.y * y.x);
+            }
+            p01[i][r] = c;
+        }
+        for (int idx = threadIdx.x; idx < kVI * (kVK / 2); idx += 256) {
+            const int i = idx / (kVK / 2), k = idx - i * (kVK / 2);
+            float2 u = zero, w = zero;
+            if (i0 + i < s1) {
+                const float2 *q = P2 + (size_t)sp_ions[i0 + i] * n2h;
+                if (kc + 2 * k < n2h) u = q[kc + 2 * k];
+                if (kc + 2 * k + 1 < n2h) w = q[kc + 2 * k + 1];
+            }
+            p2s[i][k] = make_float4(u.x, w.x, u.y, w.y);
+        }
+        __syncthreads();
+        const int ni = min(kVI, s1 - i0);
+        for (int g = 0; g < ni; g += 8) {
+            float2 acc[4][2][2];
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+#pragma unroll
+                for (int p = 0; p < 2; p++) acc[j][p][0] = acc[j][p][1] = zero;
+#pragma unroll 4
+            for (int i = g; i < g + 8; i++) {                 // (ions past the list are zeros)
+                const float4 c01 = *reinterpret_cast<const float4 *>(&p01[i][4 * tr]);
+                const float4 c23 = *reinterpret_cast<const float4 *>(&p01[i][4 * tr + 2]);
+                const float4 qa = p2s[i][2 * tk], qb = p2s[i][2 * tk + 1];
+                const float cr[4] = {c01.x, c01.z, c23.x, c23.z}, ci[4] = {c01.y, c01.w, c23.y, c23.w};
+                const float2 Qr[2] = {make_float2(qa.x, qa.y), make_float2(qb.x, qb.y)};
+                const float2 Qi[2] = {make_float2(qa.z, qa.w), make_float2(qb.z, qb.w)};
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const float2 ar = make_float2(cr[j], cr[j]), ai = make_float2(ci[j], ci[j]);
+                    const float2 mi = make_float2(-ci[j], -ci[j]);
+#pragma unroll
+                    for (int p = 0; p < 2; p++) {
+                        acc[j][p][0] = __ffma2_rn(mi, Qi[p], __ffma2_rn(ar, Qr[p], acc[j][p][0]));
+                        acc[j][p][1] = __ffma2_rn(ai, Qr[p], __ffma2_rn(ar, Qi[p], acc[j][p][1]));
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+#pragma unroll
+                for (int p = 0; p < 2; p++)
+#pragma unroll
+                    for (int d = 0; d < 2; d++) pair_add(hi[j][p][d], lo[j][p][d], acc[j][p][d]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const int r = r0 + 4 * tr + j;
+        if (r >= rows) continue;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int k = kc + 4 * tk + q, p = q >> 1;
+            if (k >= n2h) continue;
+            const long long e = (long long)r * n2h + k;
+            double v;
+            if (vf) {
+                v = vf[e];
+            } else {
+                double gx, gy, gz;
+                int k0, k1, k2;
+                gvec_of(a, e, gx, gy, gz, k0, k1, k2);
+                v = pp_form(gx * gx + gy * gy + gz * gz, a.Z[s], a.rc[s]) / a.omega;
+            }
+            const double sr = (q & 1) ? (double)hi[j][p][0].y + (double)lo[j][p][0].y
+                                      : (double)hi[j][p][0].x + (double)lo[j][p][0].x;
+            const double si = (q & 1) ? (double)hi[j][p][1].y + (double)lo[j][p][1].y
+                                      : (double)hi[j][p][1].x + (double)lo[j][p][1].x;
+            float2 o = make_float2((float)(v * sr), (float)(v * si));
+            if (!first) {
+                const float2 old = v32[e];
+                o = make_float2((float)(v * sr + (double)old.x), (float)(v * si + (double)old.y));
+            }
+            v32[e] = o;
+        }
+    }
+}
+
+cudaError_t launch_vext(const IonArgs &a, double2 *vext64, float2 *vext32, cudaStream_t s, const float2 *ph32,
+                        const int *sp_ions, const int *sp_off, const double *vf) {
+    const long long NH = (long long)a.n0 * a.n1 * a.n2h;
+    if (ph32 && vext32 && !vext64) {
+        const dim3 grid((unsigned)((a.n0 * a.n1 + kVR - 1) / kVR), (unsigned)((a.n2h + kVK - 1) / kVK));
+        for (int t = 0; t < a.n_species; t++)
+            vext_fast_kernel<<<grid, 256, 0, s>>>(a, ph32, sp_ions, sp_off[t], sp_off[t + 1], t,
+                                                  vf ? vf + (size_t)t * NH : nullptr, vext32, t == 0);
+    } else {
+        vext_kernel<<<(unsigned)((NH + 255) / 256), 256, 0, s>>>(a, vext64, vext32);
+    }
+    return cudaGetLastError();
+}
+
+// phase tables of the ions: P_a(k) = e^{-2 pi i m_a(k) f_a}, f_a = R . (row a of recip), in FP64 and
+// rounded to FP32 ([n_ions][n0], then [n_ions][n1], then [n_ions][n2h]); on the host their sines and
+// cosines were the largest part of a change of ions
+struct PhaseArgs {
+    int n[3], len[3], n_ions;
+    double recip[9];
+};
+__global__ void __launch_bounds__(256) phase_kernel(PhaseArgs a, const double *pos, double2 *ph, float2 *ph32) {
+    const int ax = blockIdx.y;
+    const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const int len = a.len[ax], nn = a.n[ax];
+    if (idx >= (long long)a.n_ions * len) return;
+    const int I = (int)(idx / len), k = (int)(idx - (long long)I * len);
+    const double fr = pos[3 * (size_t)I] * a.recip[3 * ax] + pos[3 * (size_t)I + 1] * a.recip[3 * ax + 1] +
+                      pos[3 * (size_t)I + 2] * a.recip[3 * ax + 2];
+    const double m = (ax == 2 || k <= nn / 2) ? k : k - nn;
+    double t = m * fr;
+    t -= floor(t);
+    double sn, cs;
+    sincospi(-2.0 * t, &sn, &cs);
+    long long off = 0;
+    for (int b = 0; b < ax; b++) off += (long long)a.n_ions * a.len[b];
+    ph[off + idx] = make_double2(cs, sn);
+    ph32[off + idx] = make_float2((float)cs, (float)sn);
+}
+cudaError_t launch_phases(const int *n, int n2h, int n_ions, const double *recip, const double *pos, double2 *ph,
+                          float2 *ph32, cudaStream_t s) {
+    PhaseArgs a;
+    int longest = 0;
+    for (int k = 0; k < 3; k++) {
+        a.n[k] = n[k];
+        a.len[k] = k == 2 ? n2h : n[k];
+        longest = a.len[k] > longest ? a.len[k] : longest;
+    }
+    a.n_ions = n_ions;
+    for (int k = 0; k < 9; k++) a.recip[k] = recip[k];
+    const dim3 grid((unsigned)(((long long)n_ions * longest + 255) / 256), 3);
+    phase_kernel<<<grid, 256, 0, s>>>(a, pos, ph, ph32);
     return cudaGetLastError();
 }
 
@@ -343,17 +480,22 @@ cudaError_t launch_forces_sep(const IonArgs &a, const float2 *rhohat, const floa
     return cudaSuccess;
 }
 
-// F_I = sum_a b_a S_a(I), S_a(I) = the partials [n_ions][nrb][3] summed over the row tiles in order
-__global__ void reduce_force_sep_kernel(IonArgs a, const double *part, int nrb, double *F) {
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
+// F_I = sum_a b_a S_a(I), S_a(I) = the partials [n_ions][nrb][3]: one warp per ion, its lanes over
+// the row tiles and a fixed shuffle tree (a thread per ion waited for nrb dependent loads)
+__global__ void __launch_bounds__(128) reduce_force_sep_kernel(IonArgs a, const double *part, int nrb, double *F) {
+    const int I = (blockIdx.x * 128 + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (I >= a.n_ions) return;
     double S[3] = {0.0, 0.0, 0.0};
-    for (int c = 0; c < nrb; c++)
+    for (int c = lane; c < nrb; c += 32)
         for (int k = 0; k < 3; k++) S[k] += part[((size_t)I * nrb + c) * 3 + k];
-    for (int d = 0; d < 3; d++) F[3 * I + d] = S[0] * a.bvec[d] + S[1] * a.bvec[3 + d] + S[2] * a.bvec[6 + d];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 3; k++) S[k] += __shfl_xor_sync(0xffffffffu, S[k], o);
+    if (lane < 3) F[3 * I + lane] = S[0] * a.bvec[lane] + S[1] * a.bvec[3 + lane] + S[2] * a.bvec[6 + lane];
 }
 cudaError_t launch_reduce_force_sep(const IonArgs &a, const double *part, int nrb, double *F, cudaStream_t s) {
-    reduce_force_sep_kernel<<<(a.n_ions + 127) / 128, 128, 0, s>>>(a, part, nrb, F);
+    reduce_force_sep_kernel<<<(a.n_ions + 3) / 4, 128, 0, s>>>(a, part, nrb, F);
     return cudaGetLastError();
 }
 
