@@ -83,7 +83,7 @@ template <typename T> const void *any_row_kernel(int E, bool inverse) {
     return inverse ? (const void *)row_inv_any_kernel<T, 4> : (const void *)row_fwd_any_kernel<T, 4>;
 }
 
-template <typename T> void any_candidates(int role, int n, std::vector<KernelCand> &out) {
+template <typename T> void any_candidates(int role, int n, long long cols, int nsm, std::vector<KernelCand> &out) {
     KernelCand c;
     c.any = 1;
     auto add = [&](const void *k1, const void *k2, int B, int nt, const char *kind) {
@@ -122,8 +122,10 @@ template <typename T> void any_candidates(int role, int n, std::vector<KernelCan
             const void *k = any_axis0_kernel<T>(RL, false), *km = any_axis0_kernel<T>(RL, true);
             if (!k || n % RL || any_plan(n, RL).np < 2 || made >= 3) continue;
             const int tmax = sizeof(T) == 4 ? (RL >= 12 ? 256 : 512) : 256;
-            // 16 columns where the block and its tiles leave room for two blocks per SM, else 8, else 4
+            // 16 columns where the block and its tiles leave room for two blocks per SM and the
+            // grid has a tile for every SM, else 8, else 4
             for (int lg : {4, 3, 2}) {
+                if (lg > 2 && (cols >> lg) < nsm) continue;
                 const int nt = ((n / RL << lg) + 31) / 32 * 32;
                 if (nt > tmax || any_axis0_smem<T>(n, lg) > (lg == 4 ? 100 : 200) * 1024) continue;
                 c.RL = RL;
@@ -139,7 +141,7 @@ template <typename T> void any_candidates(int role, int n, std::vector<KernelCan
 
 #define INST(T)                                                              \
     template const void *any_row_kernel<T>(int, bool);                       \
-    template void any_candidates<T>(int, int, std::vector<KernelCand> &);
+    template void any_candidates<T>(int, int, long long, int, std::vector<KernelCand> &);
 INST(float)
 INST(double)
 

@@ -285,7 +285,7 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
             const T m0 = (T)(k0 <= n / 2 ? k0 : k0 - n);
             const T gx = cv[0] + m0 * bx, gy = cv[1] + m0 * by, gz = cv[2] + m0 * bz;
             // (threads past the last frequency carry zeros: any |G| that keeps their kernel finite)
-            gn[r] = act ? dsqrt(gx * gx + gy * gy + gz * gz) : (T)1e3;
+            gn[r] = g_state(act ? gx * gx + gy * gy + gz * gz : (T)1e6);
             gmin = gn[r] < gmin ? gn[r] : gmin;
         }
     }
@@ -326,13 +326,14 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
         if (kind == OP_WT || kind == OP_EX || kind == OP_IP) {
             // the kernel of this knot (WT: of the mean density's kF) at the thread's |G|
             const T hk = kind == OP_WT ? (T)(0.5 / a.scal[S_KF_WT]) : (T)0.5 / sk[op.m];
+            const T ihk2 = (T)1 / (hk * hk);
             Part<T, false> fN;
             auto knot = [&](auto large) {
 #pragma unroll
                 for (int r = 0; r < RL; r++) {
                     T K;
                     if constexpr (decltype(large)::value) K = kernel_value_large(gn[r] * hk);
-                    else K = kernel_value<T, MGP>(a, gn[r] * hk);
+                    else K = kernel_of_state<T, MGP>(a, gn[r], hk, ihk2);
                     if (kind == OP_EX) {
                         // E_NL += Omega sum_G w Re(conj(FFT[h_k rho^alpha]) K_k FFT[rho^beta])
                         const C Sm = cscale(v[r], invN);
@@ -357,7 +358,7 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
 #pragma unroll
             for (int r = 0; r < RL; r++) {
                 const C X0 = cscale(v[r], invN);
-                const T g2 = gn[r] * gn[r];
+                const T g2 = g2_of(gn[r]);
                 const size_t e = (size_t)(t + r * m) * PL + col;
                 if (a.rhohat_out && ok && act) a.rhohat_out[e] = X0;
                 C out = cmake<C>((T)0, (T)0), vx = out;
@@ -384,7 +385,7 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
 #pragma unroll
             for (int r = 0; r < RL; r++) {
                 const C X0 = cscale(v[r], invN);
-                const T g2 = gn[r] * gn[r];
+                const T g2 = g2_of(gn[r]);
                 fV.add(cw * g2 * (X0.x * X0.x + X0.y * X0.y));
                 v[r] = cscale(X0, g2);
             }

@@ -383,9 +383,9 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
         }
         // any-length kernels: the default where nothing is compiled for the length
         if (g->kernel_choice == OFDFT_KERNELS_AUTO) {
-            any_candidates<T>(ROLE_ROW2, g->n[2], w.cand[TUNE_ROWS]);
-            any_candidates<T>(ROLE_PENCIL, g->n[1], w.cand[TUNE_PENCIL]);
-            any_candidates<T>(ROLE_AXIS0, g->n[0], w.cand[TUNE_AXIS0]);
+            any_candidates<T>(ROLE_ROW2, g->n[2], P, g->nsm, w.cand[TUNE_ROWS]);
+            any_candidates<T>(ROLE_PENCIL, g->n[1], P, g->nsm, w.cand[TUNE_PENCIL]);
+            any_candidates<T>(ROLE_AXIS0, g->n[0], P, g->nsm, w.cand[TUNE_AXIS0]);
             for (int E : {1, 2, 4}) {
                 cudaError_t e = allow_max_dynamic_smem(any_row_kernel<T>(E, false));
                 if (e == cudaSuccess) e = allow_max_dynamic_smem(any_row_kernel<T>(E, true));

@@ -241,8 +241,9 @@ struct KernelCand {
 // The compiled configurations of a role for axis length n (empty: only the runtime-size
 // kernels exist), the default first.  ROLE_AXIS0 lists the persistent kernels first.
 template <typename T> void kernel_candidates(int role, int n, std::vector<KernelCand> &out);
-// the any-length configurations of a role for axis length n (any.cu), appended to out
-template <typename T> void any_candidates(int role, int n, std::vector<KernelCand> &out);
+// the any-length configurations of a role for axis length n (any.cu), appended to out (cols: the
+// columns of the reciprocal-space pass, nsm: multiprocessors)
+template <typename T> void any_candidates(int role, int n, long long cols, int nsm, std::vector<KernelCand> &out);
 // the any-length plan of n (last: the radix of the last pass, 0 = free); np = 0 if there is none
 AnyPlan any_plan(int n, int last = 0);
 AnyPlan any_reversed(const AnyPlan &q);

@@ -68,16 +68,9 @@ struct CtPolicy {
 // Lindhard-derived WT kernel (Sec. 2.3, the G_NL definition below Eq. MGP):
 //   G_NL(eta) = 1/F(eta) - 3 eta^2 - 1,
 //   F(eta)    = 1/2 + (1 - eta^2)/(4 eta) ln|(1+eta)/(1-eta)|.
-// Below eta = 1/2 and above eta = 2 the exact series of F in y = eta^2
-// (resp. x = 1/eta^2) are summed, with the numerator 1 - (1 + 3 eta^2) F
-// expanded term by term so that nothing cancels (a_m = 1/(4 m^2 - 1)):
-//   eta < 1/2:  F = 1 - sum_m a_m y^m,   num = -(8/3) y + sum_{m>=2} (a_m + 3 a_{m-1}) y^m
-//   eta > 2  :  F = sum_m a_m x^m,       num = -sum_{m>=1} (a_m + 3 a_{m+1}) x^m
-// and G_NL = num / F.  The loops are unrolled, so every coefficient folds to
-// a constant.  (These series serve the FP64 kernels; the FP32-mixed kernels use the
-// polynomial forms of gnl_fit.cuh in the same two ranges.)
-template <typename T> struct GnlTerms { static constexpr int value = 10; };
-template <> struct GnlTerms<double> { static constexpr int value = 28; };
+// G_NL is analytic in y = eta^2 below eta = 1 and in x = 1/eta^2 above it; below eta = 1/2 it is
+// y S(y) and above eta = 2 it is L(x), S and L the polynomials of gnl_fit.cuh (error below the
+// rounding of the precision they serve; neither cancels, as the closed form does there).
 
 // Divisions and the logarithm of the kernel: in the FP32-mixed path the fast
 // intrinsics (at most 2 ulp for these operand ranges, against the few ulp the
@@ -97,53 +90,19 @@ template <typename T> __host__ __device__ __forceinline__ T gnl_mid(T eta) {
     return gdiv((T)1, F) - (T)3 * eta * eta - (T)1;
 }
 
-// (host and device: the FP64 form also builds the MGP correction table).  The FP32-mixed
-// kernels take G_NL below eta = 1/2 and above eta = 2 from the degree-6 polynomials of
-// gnl_fit.cuh (y S(y) and L(1/eta^2), within 2e-10 of the closed form: below FP32 rounding,
-// in 7 fused multiply-adds instead of two 10-term series and a division).
-template <typename T> __host__ __device__ __forceinline__ T gnl(T eta) {
-#ifdef __CUDA_ARCH__
-    if constexpr (sizeof(T) == 4) {
-        // both polynomials and the select carry no branch, so that the evaluations of a
-        // thread's several G vectors interleave; only 1/2 <= eta <= 2 branches
-        const float y = eta * eta;
-        const float gs = y * gnl_small_s(y), gl = gnl_large_l(gdiv(1.0f, y));
-        float g = eta < 0.5f ? gs : gl;
-        if (eta >= 0.5f && eta <= 2.0f) g = gnl_mid(eta);
-        return g;
-    } else
-#endif
-    {
-        constexpr int nt = GnlTerms<T>::value;
-        // both series are sums sum_{m=1}^{nt} c_m z^m, evaluated by Horner's rule with fused
-        // multiply-adds: p = c_nt, p = p z + c_m (m = nt-1..1), sum = p z
-        if (eta < (T)0.5) {
-            const T y = eta * eta;
-            T pF = (T)(1.0 / (4.0 * nt * nt - 1.0));
-            T pN = (T)(1.0 / (4.0 * nt * nt - 1.0) + 3.0 / (4.0 * (nt - 1) * (nt - 1) - 1.0));
-#pragma unroll
-            for (int m = nt - 1; m >= 1; m--) {
-                const double am = 1.0 / (4.0 * m * m - 1.0);
-                const double lo = (m >= 2) ? am + 3.0 / (4.0 * (m - 1) * (m - 1) - 1.0) : -8.0 / 3.0;
-                pF = pF * y + (T)am;
-                pN = pN * y + (T)lo;
-            }
-            return gdiv(pN * y, (T)1 - pF * y);
-        } else if (eta > (T)2) {
-            const T x = gdiv((T)1, eta * eta);
-            T pF = (T)(1.0 / (4.0 * nt * nt - 1.0));
-            T pN = (T)(1.0 / (4.0 * nt * nt - 1.0) + 3.0 / (4.0 * (nt + 1) * (nt + 1) - 1.0));
-#pragma unroll
-            for (int m = nt - 1; m >= 1; m--) {
-                const double am = 1.0 / (4.0 * m * m - 1.0);
-                const double hi = am + 3.0 / (4.0 * (m + 1) * (m + 1) - 1.0);
-                pF = pF * x + (T)am;
-                pN = pN * x + (T)hi;
-            }
-            return -gdiv(pN, pF);          // the common factor x of both sums cancels
-        }
-        return gnl_mid(eta);
-    }
+// G_NL from eta, y = eta^2 and x = 1/eta^2: both polynomials and the select carry no branch, so
+// that the evaluations of a thread's several G vectors interleave; only 1/2 <= eta <= 2 branches.
+// (In FP64 the polynomials of degree 12 replace two 28-term series and a division per value:
+// GB300 does two FP64 operations per clock per SM.)
+template <typename T> __device__ __forceinline__ T gnl_of(T eta, T y, T x) {
+    const T gs = y * gnl_small_s(y), gl = gnl_large_l(x);
+    T g = eta < (T)0.5 ? gs : gl;
+    if (eta >= (T)0.5 && eta <= (T)2) g = gnl_mid(eta);
+    return g;
+}
+template <typename T> __device__ __forceinline__ T gnl(T eta) {
+    const T y = eta * eta;
+    return gnl_of(eta, y, gdiv((T)1, y));
 }
 
 // MGP correction J_y(eta) by linear interpolation in u = eta / (1 + eta) of the table a.mgp_tab
@@ -161,6 +120,23 @@ template <typename T, bool MGP> __device__ __forceinline__ T kernel_value(const 
     T G = gnl(eta);
     if constexpr (MGP) G = a.mgp_1mx * G + a.mgp_3xy * mgp_j(a.mgp_tab, a.mgp_n, eta);
     return (T)kCWT * G;
+}
+
+// The per-G state from which the any-length reciprocal-space kernel takes eta at every knot: |G| in
+// FP32; in FP64 1/G^2, so that the large-eta form needs no division per knot (its eta comes from a
+// square root only in the rare closed-form range)
+template <typename T> __device__ __forceinline__ T g_state(T g2) { return sizeof(T) == 4 ? dsqrt(g2) : (T)1 / g2; }
+template <typename T> __device__ __forceinline__ T g2_of(T s) { return sizeof(T) == 4 ? s * s : (T)1 / s; }
+template <typename T, bool MGP> __device__ __forceinline__ T kernel_of_state(const EvalArgs<T> &a, T s, T hk, T ihk2) {
+    if constexpr (sizeof(T) == 4 || MGP) {
+        const T g = sizeof(T) == 4 ? s : dsqrt((T)1 / s);
+        return kernel_value<T, MGP>(a, g * hk);
+    } else {
+        const T x = s * ihk2;                    // 1/eta^2 (infinite at G = 0)
+        if (x < (T)0.25) return (T)kCWT * gnl_large_l(x);
+        const T y = (T)1 / x;
+        return (T)kCWT * gnl_of(dsqrt(y), y, (T)0);
+    }
 }
 
 // The FP32 kernel at eta > 2, exactly as kernel_value<float, false> gives it there, for a warp
