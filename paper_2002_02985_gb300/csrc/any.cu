@@ -77,6 +77,16 @@ AnyPlan any_reversed(const AnyPlan &q) {
 // the reciprocal-space kernels (any_ax0.cu): null where RL is not compiled for T
 template <typename T> const void *any_axis0_kernel(int RL, bool mgp);
 
+// the compile-time plans (any_ct*.cu)
+bool any_ct_axis0_1(int, AnyCt &);
+bool any_ct_axis0_2(int, AnyCt &);
+bool any_ct_axis0_3(int, AnyCt &);
+bool any_ct_axis0_4(int, AnyCt &);
+bool any_ct_rows_1(int, AnyCt &);
+bool any_ct_rows_2(int, AnyCt &);
+bool any_ct_rows_3(int, AnyCt &);
+bool any_ct_rows_4(int, AnyCt &);
+
 template <typename T> const void *any_row_kernel(int E, bool inverse) {
     if (E <= 1) return inverse ? (const void *)row_inv_any_kernel<T, 1> : (const void *)row_fwd_any_kernel<T, 1>;
     if (E <= 2) return inverse ? (const void *)row_inv_any_kernel<T, 2> : (const void *)row_fwd_any_kernel<T, 2>;
@@ -107,17 +117,30 @@ template <typename T> void any_candidates(int role, int n, long long cols, int n
     if (role == ROLE_ROW2 && q.np >= 1) {
         c.batched = true;
         int last = 0;
+        AnyCt ct;
+        if (sizeof(T) == 4 && (any_ct_rows_1(n, ct) || any_ct_rows_2(n, ct) || any_ct_rows_3(n, ct) || any_ct_rows_4(n, ct)))
+            c.any = 2;
         // the channel group fills half or a third of an SM's shared memory per block
         for (int kb : {40, 76}) {
             const int G = std::min(34, (int)(kb * 1024 / (2 * (size_t)(n + 2) * 2 * sizeof(T))));
             if (G < 1 || G == last) continue;
             last = G;
             c.batched = true;
-            add(any_row_kernel<T>(1, false), any_row_kernel<T>(1, true), G, 320, "anyrows");
+            add(c.any == 2 ? ct.k : any_row_kernel<T>(1, false), c.any == 2 ? ct.k2 : any_row_kernel<T>(1, true), G, 320,
+                c.any == 2 ? "ctrows" : "anyrows");
         }
     }
     if (role == ROLE_AXIS0) {
         int made = 0;
+        AnyCt ct;
+        if (sizeof(T) == 4 && (any_ct_axis0_1(n, ct) || any_ct_axis0_2(n, ct) || any_ct_axis0_3(n, ct) || any_ct_axis0_4(n, ct))) {
+            c.any = 2;
+            c.RL = ct.RL;
+            add(ct.k, ct.k2, 1 << ct.lg, ct.nt, "ctrecip");
+            c.any = 1;
+            // the run-time kernels only where the compiled tiles leave SMs without one
+            if ((cols >> ct.lg) >= nsm) return;
+        }
         for (int RL : {16, 15, 12, 10, 9, 8, 5, 4}) {
             const void *k = any_axis0_kernel<T>(RL, false), *km = any_axis0_kernel<T>(RL, true);
             if (!k || n % RL || any_plan(n, RL).np < 2 || made >= 3) continue;

@@ -92,12 +92,12 @@ template <typename C> struct AnyGlobal {
     __device__ __forceinline__ bool ok() const { return valid; }
 };
 template <int DIR, int R, typename C, class Dec, class Src, class Dst>
-__device__ __forceinline__ void any_pass_r(const AnyPass &p, int total, const C *__restrict__ tw, Dec dec, Src src,
-                                           Dst dst) {
+__device__ __forceinline__ void any_pass_r(const AnyPass p, int total, int nthr, const C *__restrict__ tw, Dec dec,
+                                           Src src, Dst dst) {
     const int ns = p.ns, nb = p.nb, stride = p.stride, magic = p.magic;
     const int istep = nb * src.ld, ostep = ns * dst.ld;
 #pragma unroll 1
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < total; idx += nthr) {
         int b, j;
         dec(idx, b, j);
         C v[R];
@@ -126,19 +126,26 @@ __device__ __forceinline__ void any_pass_r(const AnyPass &p, int total, const C 
 template <int DIR, typename C, class Dec, class Src, class Dst>
 __device__ __forceinline__ void any_pass(const AnyPass &p, int total, const C *__restrict__ tw, Dec dec, Src src,
                                          Dst dst) {
+    const int nthr = blockDim.x;
     switch (p.R) {
-        case 16: any_pass_r<DIR, 16>(p, total, tw, dec, src, dst); break;
-        case 15: any_pass_r<DIR, 15>(p, total, tw, dec, src, dst); break;
-        case 12: any_pass_r<DIR, 12>(p, total, tw, dec, src, dst); break;
-        case 10: any_pass_r<DIR, 10>(p, total, tw, dec, src, dst); break;
-        case 9: any_pass_r<DIR, 9>(p, total, tw, dec, src, dst); break;
-        case 8: any_pass_r<DIR, 8>(p, total, tw, dec, src, dst); break;
-        case 6: any_pass_r<DIR, 6>(p, total, tw, dec, src, dst); break;
-        case 5: any_pass_r<DIR, 5>(p, total, tw, dec, src, dst); break;
-        case 4: any_pass_r<DIR, 4>(p, total, tw, dec, src, dst); break;
-        case 3: any_pass_r<DIR, 3>(p, total, tw, dec, src, dst); break;
-        default: any_pass_r<DIR, 2>(p, total, tw, dec, src, dst); break;
+        case 16: any_pass_r<DIR, 16>(p, total, nthr, tw, dec, src, dst); break;
+        case 15: any_pass_r<DIR, 15>(p, total, nthr, tw, dec, src, dst); break;
+        case 12: any_pass_r<DIR, 12>(p, total, nthr, tw, dec, src, dst); break;
+        case 10: any_pass_r<DIR, 10>(p, total, nthr, tw, dec, src, dst); break;
+        case 9: any_pass_r<DIR, 9>(p, total, nthr, tw, dec, src, dst); break;
+        case 8: any_pass_r<DIR, 8>(p, total, nthr, tw, dec, src, dst); break;
+        case 6: any_pass_r<DIR, 6>(p, total, nthr, tw, dec, src, dst); break;
+        case 5: any_pass_r<DIR, 5>(p, total, nthr, tw, dec, src, dst); break;
+        case 4: any_pass_r<DIR, 4>(p, total, nthr, tw, dec, src, dst); break;
+        case 3: any_pass_r<DIR, 3>(p, total, nthr, tw, dec, src, dst); break;
+        default: any_pass_r<DIR, 2>(p, total, nthr, tw, dec, src, dst); break;
     }
+}
+
+// Plans known at compile time: radices R1 R2 R3 (R3 = 1: two passes).  The same pass code with
+// every bound, stride and twiddle step folded to a constant.
+constexpr AnyPass any_const_pass(int n, int R, int ns) {
+    return AnyPass{R, ns, n / R, n / (ns * R), ((1 << 20) + ns - 1) / ns};
 }
 
 // arguments of a block: the launch's own (one evaluation) or entry gk of a batch's list
@@ -205,8 +212,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
 // The next channel's tile arrives by cp.async while the current one is worked on; the last
 // inverse pass stores straight to global memory.  rho^beta hat, the term-2 accumulator and
 // |G| stay in registers for the whole tile.
-template <typename T, int RL, bool MGP>
+// R1 = 0: the plan and the tile width of the launch; R1 > 0: n0 = R1 R2 RL (R2 = 1: two passes)
+// and 2^LG columns, fixed at compile time.
+template <typename T, int RL, bool MGP, int R1 = 0, int R2 = 1, int LG = 0>
 __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int bid) {
+    constexpr bool CT = R1 > 0;
+    constexpr int NC = CT ? R1 * R2 * RL : 1;
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double sd[4 * 32];
@@ -215,7 +226,8 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
     __shared__ RecipOp ops[kMaxChan + 2];
     __shared__ int s_nload, s_nops;
     const AnyPlan &q = a.q0, &qi = a.q0i;
-    const int n = q.n, lg = a.lg0, TW = 1 << lg, np = q.np, m = n / RL, n2h = a.n2h;
+    const int n = CT ? NC : q.n, lg = CT ? LG : a.lg0, TW = 1 << lg, np = CT ? (R2 > 1 ? 3 : 2) : q.np;
+    const int m = n / RL, n2h = a.n2h, nthr = CT ? ((NC / RL << LG) + 31) / 32 * 32 : blockDim.x;
     const int PL = a.n1 * n2h;
     C *const L0 = (C *)smem_raw, *const L1 = L0 + (n << lg), *const X = L1 + (n << lg);
     const C *const tw = a.tw0;
@@ -252,13 +264,13 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
         s_nops = no;
     }
     if (nl && lwt)
-        for (int i = threadIdx.x; i < a.M; i += blockDim.x) sk[i] = a.knots_t[i];
+        for (int i = threadIdx.x; i < a.M; i += nthr) sk[i] = a.knots_t[i];
     __syncthreads();
     const int nload = s_nload, nops = s_nops;
     const C *const gcol = a.chan + (ok ? col : 0);
     auto prefetch = [&](C *dst, int ch) {
         const C *src = gcol + (size_t)ch * a.NH;
-        const int step = blockDim.x >> lg;
+        const int step = nthr >> lg;
         for (int i = t; i < n; i += step) cp_async<sizeof(C)>(dst + (i << lg) + w, src + (size_t)i * PL, ok);
         cp_async_commit();
     };
@@ -307,11 +319,15 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
             issued++;
             if (issued < nload) prefetch(nxt, order[issued]);
             // forward transform; v[r] ends at frequency t + r m
-            any_pass<-1>(q.p[0], q.p[0].nb << lg, tw, dec, sh(cur), sh(X));
+            if constexpr (CT)
+                any_pass_r<-1, R1>(any_const_pass(NC, R1, 1), NC / R1 << LG, nthr, tw, dec, sh(cur), sh(X));
+            else any_pass<-1>(q.p[0], q.p[0].nb << lg, tw, dec, sh(cur), sh(X));
             __syncthreads();
             C *S = X;
             if (np > 2) {
-                any_pass<-1>(q.p[1], q.p[1].nb << lg, tw, dec, sh(X), sh(cur));
+                if constexpr (CT && R2 > 1)
+                    any_pass_r<-1, R2>(any_const_pass(NC, R2, R1), NC / R2 << LG, nthr, tw, dec, sh(X), sh(cur));
+                else if constexpr (!CT) any_pass<-1>(q.p[1], q.p[1].nb << lg, tw, dec, sh(X), sh(cur));
                 __syncthreads();
                 S = cur;
             }
@@ -409,12 +425,17 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
         __syncthreads();
         C *S = D;
         if (np > 2) {
-            any_pass<+1>(qi.p[1], qi.p[1].nb << lg, tw, dec, sh(D), sh(cur));
+            if constexpr (CT && R2 > 1)
+                any_pass_r<+1, R2>(any_const_pass(NC, R2, RL), NC / R2 << LG, nthr, tw, dec, sh(D), sh(cur));
+            else if constexpr (!CT) any_pass<+1>(qi.p[1], qi.p[1].nb << lg, tw, dec, sh(D), sh(cur));
             __syncthreads();
             S = cur;
         }
         C *dst = a.chan + (size_t)op.store * a.NH + (ok ? col : 0);
-        any_pass<+1>(qi.p[np - 1], qi.p[np - 1].nb << lg, tw, dec, sh(S), AnyGlobal<C>{dst, PL, ok});
+        const AnyGlobal<C> G{dst, PL, ok};
+        if constexpr (CT)
+            any_pass_r<+1, R1>(any_const_pass(NC, R1, R2 * RL), NC / R1 << LG, nthr, tw, dec, sh(S), G);
+        else any_pass<+1>(qi.p[np - 1], qi.p[np - 1].nb << lg, tw, dec, sh(S), G);
     }
     double r4[4] = {eH, eV, eP, eN};
     if constexpr (sizeof(T) == 4) block_sum_n_f32warp<4>(r4, sd);
@@ -435,22 +456,39 @@ __global__ void __launch_bounds__(any_ax0_threads<T, RL>(), 1)
     axis0_any_body<T, RL, MGP>(ar, bid);
 }
 
+// compile-time lengths: as many blocks per SM as 128 registers a thread (255 from RL = 12 on) allow
+constexpr int any_ct_threads(int N, int RL, int lg) { return ((N / RL << lg) + 31) / 32 * 32; }
+constexpr int any_ct_blocks(int N, int RL, int lg) {
+    const int b = (RL >= 12 ? 256 : 512) / any_ct_threads(N, RL, lg);
+    return b > 1 ? b : 1;
+}
+template <typename T, int R1, int R2, int RL, int LG, bool MGP>
+__global__ void __launch_bounds__(any_ct_threads(R1 *R2 *RL, RL, LG), any_ct_blocks(R1 *R2 *RL, RL, LG))
+    axis0_ct_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
+    int bid;
+    const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
+    axis0_any_body<T, RL, MGP, R1, R2, LG>(ar, bid);
+}
+
 // ---------------------------------------------------------------- rows
 // Policy of the channel-batched row bodies (kernels.cuh) for any n2: E elements per thread,
 // the channel group and the transform's passes read at run time.
-template <typename T, int E__, bool INV> struct RowAny {
+template <typename T, int E__, bool INV, int R1 = 0, int R2 = 1, int R3 = 1> struct RowAny {
+    static constexpr int NC = R1 * R2 * R3;               // 0: the length of the launch
     typedef typename Vec2<T>::type C;
     static constexpr bool ct = false;
     static constexpr int E = E__, NT_ = E__ == 4 ? 256 : 320;
-    __device__ static int n(const EvalArgs<T> &a) { return a.n2; }
+    __device__ static int n(const EvalArgs<T> &a) { return NC ? NC : a.n2; }
     __device__ static int Gn(const EvalArgs<T> &a) { return a.any_G[INV]; }
     __device__ static int Ld(const EvalArgs<T> &a) { return a.any_G[INV] | 1; }
     __device__ static int Nt() { return blockDim.x; }
     __device__ static int Scr(const EvalArgs<T> &a) {
-        const int x = a.n2 * Ld(a), y = Gn(a) * (a.n2 + 2);
+        const int x = n(a) * Ld(a), y = Gn(a) * (n(a) + 2);
         return x > y ? x : y;
     }
-    __device__ static int slot(const EvalArgs<T> &a, int idx) { return (int)__umulhi((unsigned)idx, a.magic_n2h); }
+    __device__ static int slot(const EvalArgs<T> &a, int idx) {
+        return NC ? idx / (NC / 2 + 1) : (int)__umulhi((unsigned)idx, a.magic_n2h);
+    }
     __device__ static int slot2(const EvalArgs<T> &a, int idx) { return (int)__umulhi((unsigned)idx, a.magic_2n2h); }
     template <int DIR> __device__ static C *fft(C *x, C *y, const EvalArgs<T> &a, const C *) {
         const AnyPlan &q = a.q2;
@@ -461,14 +499,29 @@ template <typename T, int E__, bool INV> struct RowAny {
             j = G > 1 ? (int)__umulhi((unsigned)idx, mg) : idx;
             b = idx - j * G;
         };
-        for (int s = 0; s < q.np; s++) {
-            any_pass<DIR>(q.p[s], q.p[s].nb * G, tw, dec, AnyShared<C>{x, ld}, AnyShared<C>{y, ld});
+        if constexpr (NC > 0) {
+            const int nt = blockDim.x;
+            const AnyShared<C> X{x, ld}, Y{y, ld};
+            any_pass_r<DIR, R1>(any_const_pass(NC, R1, 1), NC / R1 * G, nt, tw, dec, X, Y);
             __syncthreads();
-            C *z = x;
-            x = y;
-            y = z;
+            any_pass_r<DIR, R2>(any_const_pass(NC, R2, R1), NC / R2 * G, nt, tw, dec, Y, X);
+            __syncthreads();
+            if constexpr (R3 > 1) {
+                any_pass_r<DIR, R3>(any_const_pass(NC, R3, R1 * R2), NC / R3 * G, nt, tw, dec, X, Y);
+                __syncthreads();
+                return y;
+            }
+            return x;
+        } else {
+            for (int s = 0; s < q.np; s++) {
+                any_pass<DIR>(q.p[s], q.p[s].nb * G, tw, dec, AnyShared<C>{x, ld}, AnyShared<C>{y, ld});
+                __syncthreads();
+                C *z = x;
+                x = y;
+                y = z;
+            }
+            return x;
         }
-        return x;
     }
 };
 template <typename T, int E>
@@ -484,6 +537,21 @@ __global__ void __launch_bounds__(RowAny<T, E, true>::NT_, sizeof(T) == 4 ? 2 : 
     int bid;
     const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
     row_inv2_body<T, RowAny<T, E, true>>(ar, bid, 0);
+}
+
+template <typename T, int E, int R1, int R2, int R3>
+__global__ void __launch_bounds__(320, 2)
+    row_fwd_ct_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
+    int bid;
+    const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
+    row_fwd2_body<T, RowAny<T, E, false, R1, R2, R3>>(ar, bid, 0);
+}
+template <typename T, int E, int R1, int R2, int R3>
+__global__ void __launch_bounds__(320, 2)
+    row_inv_ct_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
+    int bid;
+    const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
+    row_inv2_body<T, RowAny<T, E, true, R1, R2, R3>>(ar, bid, 0);
 }
 
 }  // namespace ofdft

@@ -1,0 +1,19 @@
+// Any-length rows with compile-time plans (lengths: any_ct.cuh, list 1).
+#include "any_ct.cuh"
+
+namespace ofdft {
+
+bool any_ct_rows_1(int n, AnyCt &c) {
+#define X(A, B, D, W)                                                                                      \
+    if (n == A * B * D) {                                                                                   \
+        constexpr int E = any_ct_E(A * B * D), S2 = B > 1 ? B : D, S3 = B > 1 ? D : 1;                 \
+        c.k = (const void *)row_fwd_ct_kernel<float, E, A, S2, S3>;                                           \
+        c.k2 = (const void *)row_inv_ct_kernel<float, E, A, S2, S3>;                                          \
+        return true;                                                                                           \
+    }
+    OFDFT_ANY_CT_1(X)
+#undef X
+    return false;
+}
+
+}  // namespace ofdft

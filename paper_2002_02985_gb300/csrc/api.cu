@@ -13,6 +13,7 @@
 #include <cudaTypedefs.h>
 
 #include "../../include/ofdft.h"
+#include "any_ct.cuh"
 #include "eval.cuh"
 #include "recip.cuh"
 #include "ewald.cuh"
@@ -296,7 +297,7 @@ template <typename T> int apply_cand(ofdft_grid *g, Workspace<T> &w, int role, c
         w.any0 = c.any;
         if (c.any) {
             for (w.lg0 = 0; (1 << w.lg0) < c.B;) w.lg0++;
-            w.q0 = any_plan(g->n[0], c.RL);
+            w.q0 = any_plan(g->n[0], c.RL);      // (unused by the compiled plans)
             w.q0i = any_reversed(w.q0);
         }
         if (c.recip.k) {
@@ -841,13 +842,21 @@ template <typename T> void choose_any_rows(Workspace<T> &w, EvalArgs<T> &a) {
         const int nch = std::max(1, inv ? a.ninv : a.nfwd), groups = (nch + w.any_Gmax - 1) / w.any_Gmax;
         const int G = (nch + groups - 1) / groups;
         int nt = std::min(320, std::max(64, (nbmax * G + 31) / 32 * 32));
+        if (w.any2 == 2) {
+            const int E = any_ct_E(n);
+            nt = std::max(nt, ((n + E - 1) / E + 31) / 32 * 32);
+        }
         int E = (n + nt - 1) / nt;
-        if (E > 2) {
+        if (w.any2 == 1 && E > 2) {
             E = 4;
             nt = std::min(256, std::max(nt, ((n + 3) / 4 + 31) / 32 * 32));
         }
         a.any_G[inv] = G;
         a.magic_G[inv] = (unsigned)(((1ull << 32) + G - 1) / G);
+        if (w.any2 == 2) {
+            (inv ? a.thr_rowi : a.thr_rowf) = nt;
+            continue;
+        }
         const void *k = any_row_kernel<T>(E, inv != 0);
         if (inv) {
             w.ks.row_inv = w.ks.row_inv_g = k;

@@ -233,7 +233,9 @@ struct KernelCand {
     const void *g1 = nullptr, *g2 = nullptr;   // their grouped forms
     int B = 0, nt = 0;
     bool batched = false;                 // channel-batched row kernels (B = channels per group)
-    int any = 0, RL = 0;                  // any-length kernels (any.cuh): B = tile width or largest channel group
+    // any-length kernels (any.cuh): 1 the plan read at run time, 2 compiled; B = tile width or
+    // largest channel group
+    int any = 0, RL = 0;
     RecipLaunch recip;
     char name[48] = {0};
 };
@@ -244,6 +246,12 @@ template <typename T> void kernel_candidates(int role, int n, std::vector<Kernel
 // the any-length configurations of a role for axis length n (any.cu), appended to out (cols: the
 // columns of the reciprocal-space pass, nsm: multiprocessors)
 template <typename T> void any_candidates(int role, int n, long long cols, int nsm, std::vector<KernelCand> &out);
+// an any-length configuration with a compile-time plan (any_ct.cuh): kernels (Wang-Teter and Eq. MGP
+// forms, or forward and inverse rows), frequencies per thread, log2 of the tile width, block size
+struct AnyCt {
+    const void *k = nullptr, *k2 = nullptr;
+    int RL = 0, lg = 0, nt = 0;
+};
 // the any-length plan of n (last: the radix of the last pass, 0 = free); np = 0 if there is none
 AnyPlan any_plan(int n, int last = 0);
 AnyPlan any_reversed(const AnyPlan &q);
