@@ -18,6 +18,7 @@
 #include "recip.cuh"
 #include "ewald.cuh"
 #include "misc.cuh"
+#include "plain.cuh"
 #include "pme.cuh"
 
 using namespace ofdft;
@@ -91,6 +92,8 @@ template <typename T> struct Workspace {
     int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0;
     AnyPlan q0, q0i;
     int TW0_p = 0, thr_ax0_p = 0;     // the runtime-size n0 transform of plain fields
+    bool plain_any = false;           // the any-length plain transforms (plain.cu) serve this grid
+    PlainArgs<T> pl;
     int row2_G = 0;                   // channel-batched row kernels in use: channels per group
     int ax0_scr = 0;                  // the reciprocal-space kernel transforms out of place
     // plain one-channel transforms (preconditioner, interpolation, TD-OFDFT): the per-channel row
@@ -439,6 +442,13 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
             w.row2_G_p = 0;
             break;
         }
+    std::memset(&w.pl, 0, sizeof(w.pl));
+    w.pl.n0 = g->n[0];
+    w.pl.n1 = g->n[1];
+    w.pl.n2 = g->n[2];
+    w.pl.n2h = g->n2h;
+    for (int i = 0; i < 9; i++) w.pl.b[i] = (T)(2.0 * kPi * g->recip[i]);
+    w.plain_any = g->kernel_choice == OFDFT_KERNELS_AUTO && !generic_only && plain_setup<T>(w.pl, g->nsm);
     cudaError_t e = prepare_kernels(w.ks);
     if (e == cudaSuccess) e = prepare_kernels(w.ks_plain);
     if (e != cudaSuccess) return fail(g, OFDFT_ERR_CUDA, "kernel attributes", e);
@@ -1089,8 +1099,39 @@ template <typename T> EvalArgs<T> plain_args(ofdft_grid *g, Workspace<T> &w, con
     return a;
 }
 
+// the any-length plain transform of slot `slot` with the workspace's buffers
+template <typename T> PlainArgs<T> plain_any_args(Workspace<T> &w, ofdft_grid *g, int slot) {
+    PlainArgs<T> a = w.pl;
+    a.h = w.chan + (size_t)slot * g->NH;
+    a.tw0 = w.tw[0];
+    a.tw2 = w.tw[2];
+    a.scal = w.scal;
+    a.c1 = a.scale = (T)1;
+    return a;
+}
+// the n1 pencils of one slot, in place
+template <typename T> int plain_pencils(ofdft_grid *g, Workspace<T> &w, int slot, bool inverse) {
+    EvalArgs<T> a = plain_args<T>(g, w, nullptr);
+    a.col_ch[0] = slot;
+    a.ncol_inv = 1;
+    a.col_inv_ch[0] = slot;
+    CK(launch_pencils<T>(a, w.ks_plain, inverse, g->stream), "transform along n1");
+    return OFDFT_OK;
+}
+
 // normalised half spectrum (1/N) of a real field into slot CH_HPP (G = 0 is not kept)
 template <typename T> int forward_plain(ofdft_grid *g, Workspace<T> &w, const T *field) {
+    if (w.plain_any) {
+        PlainArgs<T> p = plain_any_args<T>(w, g, CH_HPP);
+        p.u = field;
+        CK(launch_plain_mean<T>(field, g->N, stats_blocks(g), w.part_stats, w.scal, w.ticket, g->stream), "mean");
+        CK(launch_plain_rows<T>(p, false, g->stream), "forward rows");
+        if (int rc = plain_pencils<T>(g, w, CH_HPP, false)) return rc;
+        p.mode = PLAIN_FORWARD;
+        p.scale = (T)(1.0 / (double)g->N);
+        CK(launch_plain_n0<T>(p, g->stream), "forward transform along n0");
+        return OFDFT_OK;
+    }
     EvalArgs<T> a = plain_args<T>(g, w, field);
     CK(launch_forward_rows_cols<T>(a, w.ks_plain, g->stream), "forward transform");
     CK(launch_axis0_fft<T>(w.chan, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0], w.tw[0], w.TW0_p, w.thr_ax0_p,
@@ -1102,6 +1143,15 @@ template <typename T> int forward_plain(ofdft_grid *g, Workspace<T> &w, const T 
 // real field out = sum_G F(G) e^{iG.r} of the half spectrum F in slot `slot` (destroys it)
 template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot, T *out, const T *any_field) {
     typedef typename Vec2<T>::type C;
+    if (w.plain_any) {
+        PlainArgs<T> p = plain_any_args<T>(w, g, slot);
+        p.mode = PLAIN_INVERSE;
+        CK(launch_plain_n0<T>(p, g->stream), "inverse transform along n0");
+        if (int rc = plain_pencils<T>(g, w, slot, true)) return rc;
+        p.out = out;
+        CK(launch_plain_rows<T>(p, true, g->stream), "inverse rows");
+        return OFDFT_OK;
+    }
     EvalArgs<T> a = plain_args<T>(g, w, any_field);
     a.terms = 0;
     a.V = out;
@@ -1114,6 +1164,52 @@ template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot
                            w.tw[0], w.TW0_p, w.thr_ax0_p, 1.0, g->stream, +1),
        "inverse transform along n0");
     CK(launch_inverse_cols_rows<T>(a, w.ks_plain, g->stream), "inverse transform");
+    return OFDFT_OK;
+}
+
+// out = c0 base + c1 (IFFT(f FFT(u)) + v u), f the factor of `mode` (PLAIN_KINETIC, PLAIN_CN or
+// PLAIN_PRECOND with parameters p1, p2; f0 = f(G = 0), applied to the mean); v, base may be null.
+// out is neither u nor base.
+template <typename T>
+int filter_plain(ofdft_grid *g, Workspace<T> &w, const T *u, int mode, double p1, double p2, double f0, T *out,
+                 const T *v = nullptr, const T *base = nullptr, double c0 = 0.0, double c1 = 1.0) {
+    typedef typename Vec2<T>::type C;
+    const long long N = g->N;
+    cudaStream_t s = g->stream;
+    int rc;
+    if (w.plain_any) {
+        PlainArgs<T> p = plain_any_args<T>(w, g, CH_HPP);
+        p.u = u;
+        CK(launch_plain_mean<T>(u, N, stats_blocks(g), w.part_stats, w.scal, w.ticket, s), "mean");
+        CK(launch_plain_rows<T>(p, false, s), "forward rows");
+        if ((rc = plain_pencils<T>(g, w, CH_HPP, false))) return rc;
+        p.mode = mode;
+        p.p1 = (T)p1;
+        p.p2 = (T)p2;
+        p.scale = (T)(1.0 / (double)N);
+        CK(launch_plain_n0<T>(p, s), "filter along n0");
+        if ((rc = plain_pencils<T>(g, w, CH_HPP, true))) return rc;
+        p.out = out;
+        p.madd = (T)f0;
+        p.v = v;
+        p.vu = u;
+        p.base = base;
+        p.c0 = (T)c0;
+        p.c1 = (T)c1;
+        CK(launch_plain_rows<T>(p, true, s), "inverse rows");
+        return OFDFT_OK;
+    }
+    double bv[9];
+    for (int i = 0; i < 9; i++) bv[i] = 2.0 * kPi * g->recip[i];
+    if ((rc = forward_plain<T>(g, w, u))) return rc;
+    if (mode == PLAIN_PRECOND) CK(launch_precond<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, p1, p2, s), "factor");
+    else
+        CK(launch_spectral_factor<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, mode == PLAIN_CN, p1, p2, s), "factor");
+    if ((rc = inverse_plain<T>(g, w, CH_HPP, out, u))) return rc;
+    if (f0 != 0.0) CK(launch_add_scaled_scalar<T>(out, w.scal + S_RHO_MEAN, f0, N, s), "mean");
+    if (v) CK(launch_add_vu<T>(out, v, u, 1.0, 1.0, N, s), "potential");
+    if (base) CK(launch_axpby<T>(out, base, c0, c1, N, s), "axpby");
+    else if (c1 != 1.0) CK(launch_axpby<T>(out, out, c1, 0.0, N, s), "axpby");
     return OFDFT_OK;
 }
 
@@ -1509,8 +1605,8 @@ template <typename T> struct Dev {
     cudaError_t err = cudaSuccess;
     double dot(const T *a, const T *b, const T *c = nullptr) {
         if (err != cudaSuccess) return std::nan("");
-        cudaError_t e = launch_dot<T>(a, b, c, g->N, w->part_misc, 1024, w->part_misc + 2048, g->stream,
-                                      g->exact_sums != 0);
+        cudaError_t e = launch_dot<T>(a, b, c, g->N, w->part_misc, 2 * stats_blocks(g), w->part_misc + 2048, w->ticket,
+                                      g->stream, g->exact_sums != 0);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(g->h_pinned + 40, w->part_misc + 2048, sizeof(double), cudaMemcpyDeviceToHost,
                                 g->stream);
@@ -1576,18 +1672,11 @@ int optimize_impl(ofdft_grid *g, T *psi, const ofdft_functional *f0, double Ne, 
     const bool resid_obj = o.objective == OFDFT_OBJECTIVE_RESIDUAL;
     const double rho_m = Ne / g->omega;
     const double pa = 70.0 / 9.0 * kCTF * std::pow(rho_m, 2.0 / 3.0), pb = 16.0 * kPi * rho_m;
-    double bv[9];
-    for (int i = 0; i < 9; i++) bv[i] = 2.0 * kPi * g->recip[i];
     T *z = tmp;                        // preconditioned gradient (tmp is free until the line search)
     double zg_prev = 0.0;
     auto apply_precond = [&](const T *x, T *out) -> int {
-        // the plain forward transform drops the mean (kept in the scalars); P(0) = 1 adds it back
-        int r = forward_plain<T>(g, w, x);
-        if (r) return r;
-        CK(launch_precond<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, pa, pb, s), "preconditioner");
-        if ((r = inverse_plain<T>(g, w, 0, out, x))) return r;
-        CK(launch_add_scalar<T>(out, w.scal + S_RHO_MEAN, N, s), "preconditioner mean");
-        return OFDFT_OK;
+        // (P(0) = 1 keeps the mean)
+        return filter_plain<T>(g, w, x, PLAIN_PRECOND, pa, pb, 1.0, out);
     };
     double pp = 0.0;                   // <psi, psi> of the current iterate
     auto project = [&](T *v) -> int {  // v -= (<v, psi> / <psi, psi>) psi: the tangent space
@@ -1957,8 +2046,6 @@ int td_impl(ofdft_grid *g, T *pre, T *pim, const T *rho0, const ofdft_functional
     T *x[2] = {pre, pim};
     Dev<T> dv{g, &w};
     cudaStream_t s = g->stream;
-    double bv[9];
-    for (int i = 0; i < 9; i++) bv[i] = 2.0 * kPi * g->recip[i];
     TdCell cell;
     for (int i = 0; i < 9; i++) cell.a[i] = g->cell[i];
     ofdft_functional f = *f0;
@@ -1984,28 +2071,16 @@ int td_impl(ofdft_grid *g, T *pre, T *pim, const T *rho0, const ofdft_functional
         return e;
     };
     auto apply_h = [&](const T *u, const T *v, T *out) -> int {   // out = K u + v u
-        int e = forward_plain<T>(g, w, u);
-        if (e) return e;
-        CK(launch_spectral_factor<C>((C *)w.chan, n0, n1, n2, bv, 0, 0.0, 0.0, s), "kinetic");
-        if ((e = inverse_plain<T>(g, w, 0, out, u))) return e;
-        CK(launch_add_vu<T>(out, v, u, 1.0, 1.0, N, s), "potential");
-        return OFDFT_OK;
+        return filter_plain<T>(g, w, u, PLAIN_KINETIC, 0.0, 0.0, 0.0, out, v);
     };
     auto apply_a = [&](const T *u, const T *v, T *out) -> int {   // out = (1 + tau^2 H^2) u
-        int e = apply_h(u, v, h1);
-        if (e || (e = apply_h(h1, v, out))) return e;
-        CK(launch_axpby<T>(out, u, 1.0, tau * tau, N, s), "axpby");
-        return OFDFT_OK;
+        if (int e = apply_h(u, v, h1)) return e;
+        return filter_plain<T>(g, w, h1, PLAIN_KINETIC, 0.0, 0.0, 0.0, out, v, u, 1.0, tau * tau);
     };
     double vbar = 0.0;
     auto apply_m = [&](const T *u, T *out) -> int {              // out = M u
-        int e = forward_plain<T>(g, w, u);
-        if (e) return e;
-        CK(launch_spectral_factor<C>((C *)w.chan, n0, n1, n2, bv, 1, tau, vbar, s), "preconditioner");
-        if ((e = inverse_plain<T>(g, w, 0, out, u))) return e;
         const double a0 = tau * vbar;
-        CK(launch_add_scaled_scalar<T>(out, w.scal + S_RHO_MEAN, 1.0 / (1.0 + a0 * a0), N, s), "mean");
-        return OFDFT_OK;
+        return filter_plain<T>(g, w, u, PLAIN_CN, tau, vbar, 1.0 / (1.0 + a0 * a0), out);
     };
     // x <- psi(t + dt) for the Hamiltonian with potential v, x holding the initial guess
     // (x_is_psi: the guess is psi(t) itself, whose residual follows from the right-hand side)

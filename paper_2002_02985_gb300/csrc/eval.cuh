@@ -283,6 +283,8 @@ template <typename T> cudaError_t launch_group(const EvalArgs<T> &a, const EvalA
 template <typename T> cudaError_t launch_collect(const EvalArgs<T> *ga, int n, double *out, cudaStream_t s);
 // inverse pencil along n1 + C2R rows of the channels in a.col_inv_ch / a.inv_ch (CONS_ADD), V = result
 template <typename T> cudaError_t launch_inverse_cols_rows(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t s);
+// the n1 pencils alone (channels a.col_ch or a.col_inv_ch)
+template <typename T> cudaError_t launch_pencils(const EvalArgs<T> &a, const LaunchSet &ks, bool inverse, cudaStream_t s);
 // stats + knots + row_fwd + forward pencil along n1 only (the channels of a.fwd_ch / a.col_ch)
 template <typename T> cudaError_t launch_forward_rows_cols(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t s);
 // Table of the MGP correction J_y(eta) = 2 int_0^1 r^(6y-1) G_NL(eta/r^2) dr at eta = u/(1-u),

@@ -140,6 +140,12 @@ template <typename T> cudaError_t launch_forward_rows_cols(const EvalArgs<T> &a,
 }
 
 template <typename T>
+cudaError_t launch_pencils(const EvalArgs<T> &a, const LaunchSet &ks, bool inverse, cudaStream_t s) {
+    return launch(inverse ? ks.pen_inv : ks.pen_fwd, dim3(pencil_tiles(a, inverse ? a.ncol_inv : a.ncol)), a.thr_p1,
+                  pen_smem(a), a, s);
+}
+
+template <typename T>
 cudaError_t launch_inverse_cols_rows(const EvalArgs<T> &a, const LaunchSet &ks, cudaStream_t s) {
     const long long R = (long long)a.n0 * a.n1;
     const long long pairs = (R + 1) / 2;
@@ -219,6 +225,7 @@ template <typename T> cudaError_t launch_mgp_table(T *tab, int n, double y, cons
     template LaunchSet generic_kernels<T>(bool);                                                             \
     template cudaError_t launch_eval<T>(const EvalArgs<T> &, const LaunchSet &, cudaStream_t, const ProfHook *,   \
                                         const RecipMaps *);                                                  \
+    template cudaError_t launch_pencils<T>(const EvalArgs<T> &, const LaunchSet &, bool, cudaStream_t);        \
     template cudaError_t launch_forward_rows_cols<T>(const EvalArgs<T> &, const LaunchSet &, cudaStream_t); \
     template cudaError_t launch_inverse_cols_rows<T>(const EvalArgs<T> &, const LaunchSet &, cudaStream_t);
 INST(float)

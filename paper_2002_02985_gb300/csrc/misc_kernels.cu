@@ -628,8 +628,9 @@ template cudaError_t launch_axis0_fft<double>(double2 *, int, long long, const F
 // ---------------------------------------------------------------- optimiser vectors
 template <typename T>
 __global__ void __launch_bounds__(256) dot_kernel(const T *a, const T *b, const T *c, long long N, double *part,
-                                                  bool exact) {
+                                                  double *out, unsigned *ticket, bool exact) {
     __shared__ double sd[32];
+    __shared__ bool last;
     double acc = 0.0;
     const long long stride = (long long)gridDim.x * blockDim.x;
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -653,22 +654,29 @@ __global__ void __launch_bounds__(256) dot_kernel(const T *a, const T *b, const 
         }
     }
     acc = block_sum(acc, sd);
-    if (threadIdx.x == 0) part[blockIdx.x] = acc;
-}
-
-__global__ void __launch_bounds__(256) sum_partials_kernel(const double *part, int n, double *out) {
-    __shared__ double sd[32];
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) acc += part[i];
+    // the last block to finish adds the blocks' partials in order (a launch of its own took 5 us of
+    // the 14 a product costs at 128^3)
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = acc;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    acc = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) acc += __ldcg(part + k);
     acc = block_sum(acc, sd);
-    if (threadIdx.x == 0) *out = acc;
+    if (threadIdx.x == 0) {
+        *out = acc;
+        *ticket = 0u;
+    }
 }
 
 template <typename T>
 cudaError_t launch_dot(const T *a, const T *b, const T *c, long long N, double *partials, int nblk, double *out,
-                       cudaStream_t s, bool exact) {
-    dot_kernel<T><<<nblk, 256, 0, s>>>(a, b, c, N, partials, exact);
-    sum_partials_kernel<<<1, 256, 0, s>>>(partials, nblk, out);
+                       unsigned *ticket, cudaStream_t s, bool exact) {
+    dot_kernel<T><<<nblk, 256, 0, s>>>(a, b, c, N, partials, out, ticket, exact);
     return cudaGetLastError();
 }
 
@@ -1060,7 +1068,7 @@ cudaError_t launch_dipole(const T *re, const T *im, const T *rho0, int n0, int n
                                        double, long long, cudaStream_t);                                     \
     template cudaError_t launch_add_scalar<T>(T *, const double *, long long, cudaStream_t);                  \
     template cudaError_t launch_dot<T>(const T *, const T *, const T *, long long, double *, int, double *,    \
-                                       cudaStream_t, bool);                                                  \
+                                       unsigned *, cudaStream_t, bool);                                                \
     template cudaError_t launch_axpby<T>(T *, const T *, double, double, long long, cudaStream_t);           \
     template cudaError_t launch_rotate<T>(T *, T *, const T *, const T *, double, double, long long,         \
                                           cudaStream_t);                                                     \

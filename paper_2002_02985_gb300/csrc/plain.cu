@@ -1,0 +1,262 @@
+// Plain one-field transforms for any length (any.cuh): the optimiser's preconditioner, TD-OFDFT's
+// Hamiltonian, forces, PME and interpolation transform a single real field at a time.
+//
+// A filter out = IFFT(f(G) FFT(u)) is six launches: the mean, the rows (R2C), the n1 pencils, the
+// n0 pass (forward, factor and inverse in one launch, the column never leaving shared memory), the
+// n1 pencils back, and the rows back with the caller's pointwise epilogue fused into their stores.
+// (the chain it replaces -- stats, per-channel rows, n0 transform, factor kernel, n0 transform,
+// rows, potential kernel -- took 133 us at 128^3, most of it in launches of 8 to 35 us that move
+// 17 MB each)
+#include "any.cuh"
+#include "plain.cuh"
+
+namespace ofdft {
+
+// ---------------------------------------------------------------- mean
+// scal[S_RHO_MEAN] = sum of u / N (FP32: runs of 16 summed in FP32, the runs in FP64)
+template <typename T>
+__global__ void __launch_bounds__(256) plain_mean_kernel(const T *u, long long N, double *part, double *scal,
+                                                         unsigned *ticket) {
+    __shared__ double sd[32];
+    __shared__ bool last;
+    double acc = 0.0;
+    const long long stride = (long long)gridDim.x * 256;
+    long long i = blockIdx.x * 256LL + threadIdx.x;
+    while (i < N) {
+        T s = 0;
+#pragma unroll
+        for (int k = 0; k < 16; k++, i += stride) {
+            if (sizeof(T) == 8) acc += i < N ? (double)u[i] : 0.0;
+            else s += i < N ? u[i] : (T)0;
+        }
+        if (sizeof(T) == 4) acc += (double)s;
+    }
+    acc = block_sum(acc, sd);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = acc;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    acc = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += 256) acc += __ldcg(part + b);
+    acc = block_sum(acc, sd);
+    if (threadIdx.x == 0) {
+        scal[S_SUM_RHO] = acc;
+        scal[S_RHO_MEAN] = acc / (double)N;
+        *ticket = 0u;
+    }
+}
+
+// ---------------------------------------------------------------- rows
+// 2^lgB pairs of rows per block, a pair packed as z = x_2p + i x_2p+1 (element e of pair b at
+// buf[e (2^lgB + 1) + b]: the odd stride keeps both the transposing copies and the passes free of
+// bank conflicts)
+template <typename T> __device__ __forceinline__ typename Vec2<T>::type *plain_passes(const PlainArgs<T> &a, int dir,
+                                                                                      typename Vec2<T>::type *x,
+                                                                                      typename Vec2<T>::type *y) {
+    typedef typename Vec2<T>::type C;
+    const int lg = a.lgB, ld = (1 << lg) + 1;
+    auto dec = [&](int idx, int &b, int &j) {
+        b = idx & ((1 << lg) - 1);
+        j = idx >> lg;
+    };
+    for (int s = 0; s < a.q2.np; s++) {
+        const AnyShared<C> X{x, ld}, Y{y, ld};
+        if (dir < 0) any_pass<-1>(a.q2.p[s], a.q2.p[s].nb << lg, a.tw2, dec, X, Y);
+        else any_pass<+1>(a.q2.p[s], a.q2.p[s].nb << lg, a.tw2, dec, X, Y);
+        __syncthreads();
+        C *z = x;
+        x = y;
+        y = z;
+    }
+    return x;
+}
+
+template <typename T> __global__ void __launch_bounds__(256, 2) plain_rows_fwd(const __grid_constant__ PlainArgs<T> a) {
+    typedef typename Vec2<T>::type C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
+    C *const buf = (C *)smem_raw, *const scr = buf + n * ld;
+    const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1);
+    const T mean = (T)a.scal[S_RHO_MEAN];
+    for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += 256) {
+        const int rr = (int)__umulhi((unsigned)idx, a.magic_n), e = idx - rr * n;
+        const T x = row0 + rr < R ? a.u[(size_t)(row0 + rr) * n + e] - mean : (T)0;
+        ((T *)(buf + e * ld + (rr >> 1)))[rr & 1] = x;
+    }
+    __syncthreads();
+    const C *Z = plain_passes<T>(a, -1, buf, scr);
+    for (int idx = threadIdx.x; idx < n2h << lg; idx += 256) {
+        const int b = (int)__umulhi((unsigned)idx, a.magic_n2h), k = idx - b * n2h;
+        const C A = Z[k * ld + b], Bv = Z[(k ? n - k : 0) * ld + b];
+        const int r0 = row0 + 2 * b;
+        C *out = a.h + (size_t)r0 * n2h + k;
+        if (r0 < R) out[0] = cmake<C>((T)0.5 * (A.x + Bv.x), (T)0.5 * (A.y - Bv.y));
+        if (r0 + 1 < R) out[n2h] = cmake<C>((T)0.5 * (A.y + Bv.y), (T)0.5 * (Bv.x - A.x));
+    }
+}
+
+// out = c0 base + c1 (y + madd mean + v u), y the inverse transform (null pointers: left out)
+template <typename T> __global__ void __launch_bounds__(256, 2) plain_rows_inv(const __grid_constant__ PlainArgs<T> a) {
+    typedef typename Vec2<T>::type C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
+    C *const buf = (C *)smem_raw, *const scr = buf + n * ld;
+    const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1);
+    for (int idx = threadIdx.x; idx < n2h << lg; idx += 256) {
+        const int b = (int)__umulhi((unsigned)idx, a.magic_n2h), k = idx - b * n2h;
+        const int r0 = row0 + 2 * b;
+        const C zero = cmake<C>((T)0, (T)0);
+        const C *in = a.h + (size_t)r0 * n2h + k;
+        const C X0 = r0 < R ? in[0] : zero, X1 = r0 + 1 < R ? in[n2h] : zero;
+        if (k == 0 || 2 * k == n) {
+            buf[k * ld + b] = cmake<C>(X0.x, X1.x);
+        } else {
+            buf[k * ld + b] = cmake<C>(X0.x - X1.y, X0.y + X1.x);
+            buf[(n - k) * ld + b] = cmake<C>(X0.x + X1.y, X1.x - X0.y);
+        }
+    }
+    __syncthreads();
+    const C *Z = plain_passes<T>(a, +1, buf, scr);
+    const T shift = a.madd != (T)0 ? a.madd * (T)a.scal[S_RHO_MEAN] : (T)0;
+    for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += 256) {
+        const int rr = (int)__umulhi((unsigned)idx, a.magic_n), e = idx - rr * n;
+        if (row0 + rr >= R) break;
+        const size_t i = (size_t)(row0 + rr) * n + e;
+        T y = ((const T *)(Z + e * ld + (rr >> 1)))[rr & 1] + shift;
+        if (a.v) y += a.v[i] * a.vu[i];
+        a.out[i] = a.base ? a.c0 * a.base[i] + a.c1 * y : a.c1 * y;
+    }
+}
+
+// ---------------------------------------------------------------- n0
+template <typename T> __device__ __forceinline__ T plain_factor(const PlainArgs<T> &a, T g2) {
+    if (a.mode == PLAIN_KINETIC) return (T)0.5 * g2;
+    if (a.mode == PLAIN_CN) {
+        const T x = a.p1 * ((T)0.5 * g2 + a.p2);
+        return (T)1 / ((T)1 + x * x);
+    }
+    return g2 > (T)0 ? a.p1 * g2 / (g2 * g2 + a.p1 * g2 + a.p2) : (T)1;       // PLAIN_PRECOND
+}
+template <typename T> __global__ void __launch_bounds__(256, 2) plain_n0(const __grid_constant__ PlainArgs<T> a) {
+    typedef typename Vec2<T>::type C;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const AnyPlan &q = a.q0;
+    const int n = q.n, lg = a.lg0, TW = 1 << lg, np = q.np, n2h = a.n2h, PL = a.n1 * n2h;
+    C *X = (C *)smem_raw, *Y = X + (n << lg);
+    const int w = threadIdx.x & (TW - 1), col = (blockIdx.x << lg) + w;
+    const bool ok = col < PL;
+    const AnyGlobal<C> G{a.h + (ok ? col : 0), PL, ok};
+    auto dec = [&](int idx, int &b, int &j) {
+        b = w;
+        j = idx >> lg;
+    };
+    auto sh = [&](C *S) { return AnyShared<C>{S, TW}; };
+    auto swap = [&]() {
+        C *z = X;
+        X = Y;
+        Y = z;
+    };
+    if (a.mode != PLAIN_INVERSE) {
+        any_pass<-1>(q.p[0], q.p[0].nb << lg, a.tw0, dec, G, sh(X));
+        __syncthreads();
+        for (int s = 1; s < np; s++) {
+            any_pass<-1>(q.p[s], q.p[s].nb << lg, a.tw0, dec, sh(X), sh(Y));
+            __syncthreads();
+            swap();
+        }
+        const int step = 256 >> lg;
+        if (a.mode == PLAIN_FORWARD) {
+            if (ok)
+                for (int i = threadIdx.x >> lg; i < n; i += step) G.g[(size_t)i * PL] = cscale(X[(i << lg) + w], a.scale);
+            return;
+        }
+        const int k1 = ok ? col / n2h : 0, k2 = ok ? col - k1 * n2h : 0;
+        const T m1 = (T)(k1 <= a.n1 / 2 ? k1 : k1 - a.n1), m2 = (T)k2;
+        const T cx = m1 * a.b[3] + m2 * a.b[6], cy = m1 * a.b[4] + m2 * a.b[7], cz = m1 * a.b[5] + m2 * a.b[8];
+        for (int i = threadIdx.x >> lg; i < n; i += step) {
+            const T m0 = (T)(i <= n / 2 ? i : i - n);
+            const T gx = m0 * a.b[0] + cx, gy = m0 * a.b[1] + cy, gz = m0 * a.b[2] + cz;
+            C *x = X + (i << lg) + w;
+            *x = cscale(*x, a.scale * plain_factor(a, gx * gx + gy * gy + gz * gz));
+        }
+        __syncthreads();
+        for (int s = 0; s + 1 < np; s++) {
+            any_pass<+1>(q.p[s], q.p[s].nb << lg, a.tw0, dec, sh(X), sh(Y));
+            __syncthreads();
+            swap();
+        }
+    } else {
+        any_pass<+1>(q.p[0], q.p[0].nb << lg, a.tw0, dec, G, sh(X));
+        __syncthreads();
+        for (int s = 1; s + 1 < np; s++) {
+            any_pass<+1>(q.p[s], q.p[s].nb << lg, a.tw0, dec, sh(X), sh(Y));
+            __syncthreads();
+            swap();
+        }
+    }
+    any_pass<+1>(q.p[np - 1], q.p[np - 1].nb << lg, a.tw0, dec, sh(X), G);
+}
+
+// ---------------------------------------------------------------- launches
+template <typename T> static cudaError_t prepare_once() {
+    static const cudaError_t e = []() {
+        cudaError_t r = allow_max_dynamic_smem(plain_rows_fwd<T>);
+        if (r == cudaSuccess) r = allow_max_dynamic_smem(plain_rows_inv<T>);
+        if (r == cudaSuccess) r = allow_max_dynamic_smem(plain_n0<T>);
+        return r;
+    }();
+    return e;
+}
+
+template <typename T> bool plain_setup(PlainArgs<T> &a, int nsm) {
+    a.q0 = any_plan(a.n0);
+    a.q2 = any_plan(a.n2);
+    if (a.q0.np < 2 || a.q2.np < 1) return false;
+    const size_t cb = 2 * sizeof(T);
+    // rows: up to 16 pairs per block in at most 72 KB, fewer while the grid has no two blocks per SM
+    const long long R = (long long)a.n0 * a.n1;
+    for (a.lgB = 4; a.lgB > 1; a.lgB--)
+        if (2 * cb * a.n2 * ((1 << a.lgB) + 1) <= 72 * 1024 && (R >> (a.lgB + 1)) >= 2 * nsm) break;
+    if (2 * cb * a.n2 * ((1 << a.lgB) + 1) > 200 * 1024) return false;
+    // n0: 16 columns in at most 72 KB, fewer while the grid has no tile per SM
+    const long long PL = (long long)a.n1 * a.n2h;
+    for (a.lg0 = 4; a.lg0 > 2; a.lg0--)
+        if (2 * cb * ((size_t)a.n0 << a.lg0) <= 72 * 1024 && (PL >> a.lg0) >= nsm) break;
+    if (2 * cb * ((size_t)a.n0 << a.lg0) > 200 * 1024) return false;
+    a.magic_n = (unsigned)(((1ull << 32) + a.n2 - 1) / a.n2);
+    a.magic_n2h = (unsigned)(((1ull << 32) + a.n2h - 1) / a.n2h);
+    return prepare_once<T>() == cudaSuccess;
+}
+template <typename T>
+cudaError_t launch_plain_mean(const T *u, long long N, int nblk, double *part, double *scal, unsigned *ticket,
+                              cudaStream_t s) {
+    plain_mean_kernel<T><<<nblk, 256, 0, s>>>(u, N, part, scal, ticket);
+    return cudaGetLastError();
+}
+template <typename T> cudaError_t launch_plain_rows(const PlainArgs<T> &a, bool inverse, cudaStream_t s) {
+    const long long R = (long long)a.n0 * a.n1;
+    const unsigned nb = (unsigned)((R + (2 << a.lgB) - 1) >> (a.lgB + 1));
+    const size_t sm = 2 * 2 * sizeof(T) * (size_t)a.n2 * ((1 << a.lgB) + 1);
+    if (inverse) plain_rows_inv<T><<<nb, 256, sm, s>>>(a);
+    else plain_rows_fwd<T><<<nb, 256, sm, s>>>(a);
+    return cudaGetLastError();
+}
+template <typename T> cudaError_t launch_plain_n0(const PlainArgs<T> &a, cudaStream_t s) {
+    const long long PL = (long long)a.n1 * a.n2h;
+    const unsigned nb = (unsigned)((PL + (1 << a.lg0) - 1) >> a.lg0);
+    plain_n0<T><<<nb, 256, 2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s>>>(a);
+    return cudaGetLastError();
+}
+#define INST(T)                                                                                                     \
+    template bool plain_setup<T>(PlainArgs<T> &, int);                                                              \
+    template cudaError_t launch_plain_mean<T>(const T *, long long, int, double *, double *, unsigned *, cudaStream_t); \
+    template cudaError_t launch_plain_rows<T>(const PlainArgs<T> &, bool, cudaStream_t);                            \
+    template cudaError_t launch_plain_n0<T>(const PlainArgs<T> &, cudaStream_t);
+INST(float)
+INST(double)
+
+}  // namespace ofdft
