@@ -75,11 +75,13 @@ cudaError_t launch_form_tables(const IonArgs &a, double *vf, cudaStream_t st) {
 // ions are summed in FP32 and the groups as FP32 pairs (hi + lo, exact two-sums: about 48 bits,
 // without GB300's slow FP64 adds), the form factor and the sum over species in FP64.
 //
-// Block: kVR rows x kVK values of k2; the ions come kVI at a time through shared memory.  A thread
-// owns 4 rows x 4 k2, as two packed pairs of k2, so an ion costs 4 shared 16-byte reads for 32
-// packed FMAs.  One thread per G (three gathers of the tables per ion, FP64 group sums and the
-// form factor's exponential at every G) took 0.6 ms for 500 ions at 96^3.
-constexpr int kVR = 64, kVK = 64, kVI = 32;
+// Block: kVR rows x kVK values of k2; the ions come kVI at a time through shared memory, the next
+// kVI loaded into registers while the current ones are multiplied (the index and table gathers
+// are two dependent loads).  A thread owns 2 rows x 4 k2, as two packed pairs of k2, so an ion
+// costs 3 shared 16-byte reads for 16 packed FMAs.  500 ions at 96^3: 0.6 ms with one thread per
+// G (three gathers of the tables per ion, FP64 group sums, the form factor's exponential at every
+// G); 0.2 ms with 64-row tiles and loads between the barriers (144 blocks, one per SM).
+constexpr int kVR = 32, kVK = 64, kVI = 32;
 __device__ __forceinline__ void pair_add(float2 &hi, float2 &lo, float2 x) {
     // two-sum of hi + x, component by component (Knuth): the rounding error goes into lo
     const float2 m1 = make_float2(-1.f, -1.f);
@@ -99,51 +101,60 @@ __global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 
     const int tk = threadIdx.x & 15, tr = threadIdx.x >> 4;
     const float2 *P0 = ph32, *P1 = ph32 + (size_t)a.n_ions * a.n0, *P2 = P1 + (size_t)a.n_ions * a.n1;
     const float2 zero = make_float2(0.f, 0.f);
-    float2 hi[4][2][2], lo[4][2][2];                          // [row][k2 pair][re, im]
+    float2 hi[2][2][2], lo[2][2][2];                          // [row][k2 pair][re, im]
 #pragma unroll
-    for (int j = 0; j < 4; j++)
+    for (int j = 0; j < 2; j++)
 #pragma unroll
         for (int p = 0; p < 2; p++) hi[j][p][0] = hi[j][p][1] = lo[j][p][0] = lo[j][p][1] = zero;
+    // what this thread stages: ions i = it + 8 u (u < 4) of one row and of one pair of k2
+    const int il = threadIdx.x & 31, it = threadIdx.x >> 5;
+    const int row = r0 + il, k0 = row < rows ? row / a.n1 : 0, k1 = row < rows ? row - k0 * a.n1 : 0;
+    const int ka = kc + 2 * il, kb = ka + 1;
+    float2 x[4], y[4], u[4], w[4];
+    auto load = [&](int i0) {
+#pragma unroll
+        for (int v = 0; v < 4; v++) {
+            const int i = i0 + it + 8 * v;
+            x[v] = y[v] = u[v] = w[v] = zero;
+            if (i < s1) {
+                const int I = sp_ions[i];
+                if (row < rows) {
+                    x[v] = P0[(size_t)I * a.n0 + k0];
+                    y[v] = P1[(size_t)I * a.n1 + k1];
+                }
+                const float2 *q = P2 + (size_t)I * n2h;
+                if (ka < n2h) u[v] = q[ka];
+                if (kb < n2h) w[v] = q[kb];
+            }
+        }
+    };
+    load(s0);
     for (int i0 = s0; i0 < s1; i0 += kVI) {
         __syncthreads();
-        for (int idx = threadIdx.x; idx < kVI * kVR; idx += 256) {
-            const int i = idx / kVR, r = idx - i * kVR;
-            float2 c = zero;
-            if (i0 + i < s1 && r0 + r < rows) {
-                const int I = sp_ions[i0 + i], k0 = (r0 + r) / a.n1, k1 = r0 + r - k0 * a.n1;
-                const float2 x = P0[(size_t)I * a.n0 + k0], y = P1[(size_t)I * a.n1 + k1];
-                c = make_float2(x.x * y.x - x.y * y.y, x.x * y.y + x.y * y.x);
-            }
-            p01[i][r] = c;
-        }
-        for (int idx = threadIdx.x; idx < kVI * (kVK / 2); idx += 256) {
-            const int i = idx / (kVK / 2), k = idx - i * (kVK / 2);
-            float2 u = zero, w = zero;
-            if (i0 + i < s1) {
-                const float2 *q = P2 + (size_t)sp_ions[i0 + i] * n2h;
-                if (kc + 2 * k < n2h) u = q[kc + 2 * k];
-                if (kc + 2 * k + 1 < n2h) w = q[kc + 2 * k + 1];
-            }
-            p2s[i][k] = make_float4(u.x, w.x, u.y, w.y);
+#pragma unroll
+        for (int v = 0; v < 4; v++) {
+            p01[it + 8 * v][il] =
+                make_float2(x[v].x * y[v].x - x[v].y * y[v].y, x[v].x * y[v].y + x[v].y * y[v].x);
+            p2s[it + 8 * v][il] = make_float4(u[v].x, w[v].x, u[v].y, w[v].y);
         }
         __syncthreads();
+        if (i0 + kVI < s1) load(i0 + kVI);
         const int ni = min(kVI, s1 - i0);
         for (int g = 0; g < ni; g += 8) {
-            float2 acc[4][2][2];
+            float2 acc[2][2][2];
 #pragma unroll
-            for (int j = 0; j < 4; j++)
+            for (int j = 0; j < 2; j++)
 #pragma unroll
                 for (int p = 0; p < 2; p++) acc[j][p][0] = acc[j][p][1] = zero;
-#pragma unroll 4
+#pragma unroll
             for (int i = g; i < g + 8; i++) {                 // (ions past the list are zeros)
-                const float4 c01 = *reinterpret_cast<const float4 *>(&p01[i][4 * tr]);
-                const float4 c23 = *reinterpret_cast<const float4 *>(&p01[i][4 * tr + 2]);
+                const float4 c01 = *reinterpret_cast<const float4 *>(&p01[i][2 * tr]);
                 const float4 qa = p2s[i][2 * tk], qb = p2s[i][2 * tk + 1];
-                const float cr[4] = {c01.x, c01.z, c23.x, c23.z}, ci[4] = {c01.y, c01.w, c23.y, c23.w};
+                const float cr[2] = {c01.x, c01.z}, ci[2] = {c01.y, c01.w};
                 const float2 Qr[2] = {make_float2(qa.x, qa.y), make_float2(qb.x, qb.y)};
                 const float2 Qi[2] = {make_float2(qa.z, qa.w), make_float2(qb.z, qb.w)};
 #pragma unroll
-                for (int j = 0; j < 4; j++) {
+                for (int j = 0; j < 2; j++) {
                     const float2 ar = make_float2(cr[j], cr[j]), ai = make_float2(ci[j], ci[j]);
                     const float2 mi = make_float2(-ci[j], -ci[j]);
 #pragma unroll
@@ -154,7 +165,7 @@ __global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 
                 }
             }
 #pragma unroll
-            for (int j = 0; j < 4; j++)
+            for (int j = 0; j < 2; j++)
 #pragma unroll
                 for (int p = 0; p < 2; p++)
 #pragma unroll
@@ -162,8 +173,8 @@ __global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 
         }
     }
 #pragma unroll
-    for (int j = 0; j < 4; j++) {
-        const int r = r0 + 4 * tr + j;
+    for (int j = 0; j < 2; j++) {
+        const int r = r0 + 2 * tr + j;
         if (r >= rows) continue;
 #pragma unroll
         for (int q = 0; q < 4; q++) {
