@@ -19,8 +19,3 @@
 #define OFDFT_ANY_CT_4(X) \
     X(6, 6, 8, 3) X(6, 5, 10, 3) X(8, 4, 10, 3) X(6, 6, 9, 3) X(9, 5, 8, 3) X(15, 5, 5, 3) X(8, 6, 8, 3) \
     X(10, 5, 8, 3) X(9, 5, 9, 3) X(8, 6, 9, 3) X(10, 5, 9, 3) X(10, 6, 8, 3) X(9, 6, 9, 3) X(10, 5, 10, 3) X(8, 8, 8, 3)
-
-namespace ofdft {
-// elements per thread of the compile-time rows
-constexpr int any_ct_E(int n) { return n <= 160 ? 1 : 2; }
-}  // namespace ofdft

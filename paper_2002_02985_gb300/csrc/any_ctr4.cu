@@ -6,9 +6,9 @@ namespace ofdft {
 bool any_ct_rows_4(int n, AnyCt &c) {
 #define X(A, B, D, W)                                                                                      \
     if (n == A * B * D) {                                                                                   \
-        constexpr int E = any_ct_E(A * B * D), S2 = B > 1 ? B : D, S3 = B > 1 ? D : 1;                 \
-        c.k = (const void *)row_fwd_ct_kernel<float, E, A, S2, S3>;                                           \
-        c.k2 = (const void *)row_inv_ct_kernel<float, E, A, S2, S3>;                                          \
+        constexpr int S2 = B > 1 ? B : D, S3 = B > 1 ? D : 1;                 \
+        c.k = (const void *)row_fwd_ct_kernel<float, A, S2, S3>;                                           \
+        c.k2 = (const void *)row_inv_ct_kernel<float, A, S2, S3>;                                          \
         return true;                                                                                           \
     }
     OFDFT_ANY_CT_4(X)

@@ -90,7 +90,7 @@ template <typename T> struct Workspace {
     int grid_p1 = 0;
     // any-length kernels in use per role, their tile widths (log2), plans, largest row group
     int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0;
-    AnyPlan q0, q0i;
+    AnyPlan q0, q0i, q1, q2;
     int TW0_p = 0, thr_ax0_p = 0;     // the runtime-size n0 transform of plain fields
     bool plain_any = false;           // the any-length plain transforms (plain.cu) serve this grid
     PlainArgs<T> pl;
@@ -361,6 +361,8 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
         w.Brow_p = w.Brow;
         w.thr_rowf_p = w.thr_rowi_p = w.thr_rowf;
         w.any0 = w.any1 = w.any2 = 0;
+        w.q1 = any_plan(g->n[1]);
+        w.q2 = any_plan(g->n[2]);
         w.ks_plain = w.ks;
         w.ks.recip = RecipLaunch();
     }
@@ -835,7 +837,7 @@ template <typename T> void any_args_of(const ofdft_grid *g, const Workspace<T> &
     }
     if (w.any1) {
         a.lg1 = w.lg1;
-        a.q1 = any_plan(g->n[1]);
+        a.q1 = w.q1;
     }
 }
 
@@ -843,18 +845,21 @@ template <typename T> void any_args_of(const ofdft_grid *g, const Workspace<T> &
 // a thread per butterfly of the widest pass, and the kernel for the points a thread then owns.
 template <typename T> void choose_any_rows(Workspace<T> &w, EvalArgs<T> &a) {
     const int n = a.n2, n2h = a.n2h;
-    a.q2 = any_plan(n);
+    a.q2 = w.q2;
     a.magic_n2h = (unsigned)(((1ull << 32) + n2h - 1) / n2h);
     a.magic_2n2h = (unsigned)(((1ull << 32) + 2 * n2h - 1) / (2 * n2h));
-    int nbmax = 1;
-    for (int i = 0; i < a.q2.np; i++) nbmax = std::max(nbmax, a.q2.p[i].nb);
+    int nbmax = 1, nbmin = n;
+    for (int i = 0; i < a.q2.np; i++) {
+        nbmax = std::max(nbmax, a.q2.p[i].nb);
+        nbmin = std::min(nbmin, a.q2.p[i].nb);
+    }
     for (int inv = 0; inv < 2; inv++) {
         const int nch = std::max(1, inv ? a.ninv : a.nfwd), groups = (nch + w.any_Gmax - 1) / w.any_Gmax;
         const int G = (nch + groups - 1) / groups;
         int nt = std::min(320, std::max(64, (nbmax * G + 31) / 32 * 32));
         if (w.any2 == 2) {
-            const int E = any_ct_E(n);
-            nt = std::max(nt, ((n + E - 1) / E + 31) / 32 * 32);
+            const int E = any_ct_E(n), need = ((n + E - 1) / E + 31) / 32 * 32;
+            nt = std::max(std::min((nbmin * G + 31) / 32 * 32, any_ct_row_threads(n)), std::max(need, 64));
         }
         int E = (n + nt - 1) / nt;
         if (w.any2 == 1 && E > 2) {
