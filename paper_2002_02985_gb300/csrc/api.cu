@@ -1173,7 +1173,8 @@ template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot
 }
 
 // out = c0 base + c1 (IFFT(f FFT(u)) + v u), f the factor of `mode` (PLAIN_KINETIC, PLAIN_CN or
-// PLAIN_PRECOND with parameters p1, p2; f0 = f(G = 0), applied to the mean); v, base may be null.
+// PLAIN_PRECOND with parameters p1, p2; f0 = f(G = 0), applied to what the forward rows subtract);
+// v, base may be null.
 // out is neither u nor base.
 template <typename T>
 int filter_plain(ofdft_grid *g, Workspace<T> &w, const T *u, int mode, double p1, double p2, double f0, T *out,
@@ -1185,7 +1186,7 @@ int filter_plain(ofdft_grid *g, Workspace<T> &w, const T *u, int mode, double p1
     if (w.plain_any) {
         PlainArgs<T> p = plain_any_args<T>(w, g, CH_HPP);
         p.u = u;
-        CK(launch_plain_mean<T>(u, N, stats_blocks(g), w.part_stats, w.scal, w.ticket, s), "mean");
+        p.sampled = 1;
         CK(launch_plain_rows<T>(p, false, s), "forward rows");
         if ((rc = plain_pencils<T>(g, w, CH_HPP, false))) return rc;
         p.mode = mode;

@@ -1,9 +1,9 @@
 // Plain one-field transforms for any length (any.cuh): the optimiser's preconditioner, TD-OFDFT's
 // Hamiltonian, forces, PME and interpolation transform a single real field at a time.
 //
-// A filter out = IFFT(f(G) FFT(u)) is six launches: the mean, the rows (R2C), the n1 pencils, the
-// n0 pass (forward, factor and inverse in one launch, the column never leaving shared memory), the
-// n1 pencils back, and the rows back with the caller's pointwise epilogue fused into their stores.
+// A filter out = IFFT(f(G) FFT(u)) is five launches: the rows (R2C), the n1 pencils, the n0 pass
+// (forward, factor and inverse in one launch, the column never leaving shared memory), the n1
+// pencils back, and the rows back with the caller's pointwise epilogue fused into their stores.
 // (the chain it replaces -- stats, per-channel rows, n0 transform, factor kernel, n0 transform,
 // rows, potential kernel -- took 133 us at 128^3, most of it in launches of 8 to 35 us that move
 // 17 MB each)
@@ -11,6 +11,9 @@
 #include "plain.cuh"
 
 namespace ofdft {
+
+// 128 threads: a block's 16 transforms of 128 points are 128 radix-16 butterflies
+constexpr int kPlainThreads = 128;
 
 // ---------------------------------------------------------------- mean
 // scal[S_RHO_MEAN] = sum of u / N (FP32: runs of 16 summed in FP32, the runs in FP64)
@@ -51,6 +54,13 @@ __global__ void __launch_bounds__(256) plain_mean_kernel(const T *u, long long N
 }
 
 // ---------------------------------------------------------------- rows
+__device__ __forceinline__ void store4(float *p, const float v[4]) {
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void store4(double *p, const double v[4]) {
+    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+}
 // 2^lgB pairs of rows per block, a pair packed as z = x_2p + i x_2p+1 (element e of pair b at
 // buf[e (2^lgB + 1) + b]: the odd stride keeps both the transposing copies and the passes free of
 // bank conflicts)
@@ -75,21 +85,61 @@ template <typename T> __device__ __forceinline__ typename Vec2<T>::type *plain_p
     return x;
 }
 
-template <typename T> __global__ void __launch_bounds__(256, 2) plain_rows_fwd(const __grid_constant__ PlainArgs<T> a) {
+// What the rows subtract before the transform.  A transform alone takes the mean.  A filter only
+// needs a constant near it, so that the FP32 passes do not carry a large G = 0 term: the mean of
+// 1024 samples spread over the field, which every block takes for itself (the same loads in the
+// same order, so the same value) instead of waiting for a pass over the whole field; block 0
+// leaves it for the inverse rows.
+template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<T> &a) {
+    if (!a.sampled) return (T)a.scal[S_RHO_MEAN];
+    __shared__ T ws[kPlainThreads / 32];
+    const long long N = (long long)a.n0 * a.n1 * a.n2, step = N / 1024 > 0 ? N / 1024 : 1;
+    T s = 0;
+#pragma unroll
+    for (int k = 0; k < 1024 / kPlainThreads; k++) {
+        long long i = (threadIdx.x + k * kPlainThreads) * step;
+        if (i >= N) i %= N;                                   // (fields of fewer than 1024 points)
+        s += a.u[i];
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
+    __syncthreads();
+    s = 0;
+#pragma unroll
+    for (int k = 0; k < kPlainThreads / 32; k++) s += ws[k];
+    s *= (T)(1.0 / 1024.0);
+    if (blockIdx.x == 0 && threadIdx.x == 0) const_cast<double *>(a.scal)[S_RHO_MEAN] = (double)s;
+    return s;
+}
+template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_rows_fwd(const __grid_constant__ PlainArgs<T> a) {
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
     C *const buf = (C *)smem_raw, *const scr = buf + n * ld;
     const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1);
-    const T mean = (T)a.scal[S_RHO_MEAN];
-    for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += 256) {
-        const int rr = (int)__umulhi((unsigned)idx, a.magic_n), e = idx - rr * n;
-        const T x = row0 + rr < R ? a.u[(size_t)(row0 + rr) * n + e] - mean : (T)0;
-        ((T *)(buf + e * ld + (rr >> 1)))[rr & 1] = x;
+    const T mean = plain_offset(a);
+    if (a.vec) {
+        // four consecutive points of a row per thread and step, several steps in flight
+        const int n4 = n >> 2;
+#pragma unroll 4
+        for (int idx = threadIdx.x; idx < (n4 << (lg + 1)); idx += kPlainThreads) {
+            const int rr = (int)__umulhi((unsigned)idx, a.magic_n4), e = 4 * (idx - rr * n4);
+            T x[4] = {mean, mean, mean, mean};
+            if (row0 + rr < R) load4(a.u + (size_t)(row0 + rr) * n + e, x);
+#pragma unroll
+            for (int q = 0; q < 4; q++) ((T *)(buf + (e + q) * ld + (rr >> 1)))[rr & 1] = x[q] - mean;
+        }
+    } else {
+        for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += kPlainThreads) {
+            const int rr = (int)__umulhi((unsigned)idx, a.magic_n), e = idx - rr * n;
+            const T x = row0 + rr < R ? a.u[(size_t)(row0 + rr) * n + e] - mean : (T)0;
+            ((T *)(buf + e * ld + (rr >> 1)))[rr & 1] = x;
+        }
     }
     __syncthreads();
     const C *Z = plain_passes<T>(a, -1, buf, scr);
-    for (int idx = threadIdx.x; idx < n2h << lg; idx += 256) {
+    for (int idx = threadIdx.x; idx < n2h << lg; idx += kPlainThreads) {
         const int b = (int)__umulhi((unsigned)idx, a.magic_n2h), k = idx - b * n2h;
         const C A = Z[k * ld + b], Bv = Z[(k ? n - k : 0) * ld + b];
         const int r0 = row0 + 2 * b;
@@ -99,14 +149,16 @@ template <typename T> __global__ void __launch_bounds__(256, 2) plain_rows_fwd(c
     }
 }
 
-// out = c0 base + c1 (y + madd mean + v u), y the inverse transform (null pointers: left out)
-template <typename T> __global__ void __launch_bounds__(256, 2) plain_rows_inv(const __grid_constant__ PlainArgs<T> a) {
+// out = c0 base + c1 (y + madd mean + v u), y the inverse transform (null pointers: left out); out
+// overlaps none of the inputs
+template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_rows_inv(const __grid_constant__ PlainArgs<T> a) {
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
     C *const buf = (C *)smem_raw, *const scr = buf + n * ld;
     const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1);
-    for (int idx = threadIdx.x; idx < n2h << lg; idx += 256) {
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < n2h << lg; idx += kPlainThreads) {
         const int b = (int)__umulhi((unsigned)idx, a.magic_n2h), k = idx - b * n2h;
         const int r0 = row0 + 2 * b;
         const C zero = cmake<C>((T)0, (T)0);
@@ -122,7 +174,32 @@ template <typename T> __global__ void __launch_bounds__(256, 2) plain_rows_inv(c
     __syncthreads();
     const C *Z = plain_passes<T>(a, +1, buf, scr);
     const T shift = a.madd != (T)0 ? a.madd * (T)a.scal[S_RHO_MEAN] : (T)0;
-    for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += 256) {
+    if (a.vec) {
+        const int n4 = n >> 2;
+        const T *const __restrict__ pv = a.v, *const __restrict__ pu = a.vu, *const __restrict__ pb = a.base;
+        T *const __restrict__ po = a.out;
+#pragma unroll 4
+        for (int idx = threadIdx.x; idx < (n4 << (lg + 1)); idx += kPlainThreads) {
+            const int rr = (int)__umulhi((unsigned)idx, a.magic_n4), e = 4 * (idx - rr * n4);
+            if (row0 + rr < R) {
+                const size_t i = (size_t)(row0 + rr) * n + e;
+                T v[4] = {0, 0, 0, 0}, u[4] = {0, 0, 0, 0}, b[4] = {0, 0, 0, 0};
+                if (pv) {
+                    load4(pv + i, v);
+                    load4(pu + i, u);
+                }
+                if (pb) load4(pb + i, b);
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const T y = ((const T *)(Z + (e + q) * ld + (rr >> 1)))[rr & 1] + shift + v[q] * u[q];
+                    v[q] = pb ? a.c0 * b[q] + a.c1 * y : a.c1 * y;
+                }
+                store4(po + i, v);
+            }
+        }
+        return;
+    }
+    for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += kPlainThreads) {
         const int rr = (int)__umulhi((unsigned)idx, a.magic_n), e = idx - rr * n;
         if (row0 + rr >= R) break;
         const size_t i = (size_t)(row0 + rr) * n + e;
@@ -141,7 +218,7 @@ template <typename T> __device__ __forceinline__ T plain_factor(const PlainArgs<
     }
     return g2 > (T)0 ? a.p1 * g2 / (g2 * g2 + a.p1 * g2 + a.p2) : (T)1;       // PLAIN_PRECOND
 }
-template <typename T> __global__ void __launch_bounds__(256, 2) plain_n0(const __grid_constant__ PlainArgs<T> a) {
+template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_n0(const __grid_constant__ PlainArgs<T> a) {
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AnyPlan &q = a.q0;
@@ -168,7 +245,7 @@ template <typename T> __global__ void __launch_bounds__(256, 2) plain_n0(const _
             __syncthreads();
             swap();
         }
-        const int step = 256 >> lg;
+        const int step = kPlainThreads >> lg;
         if (a.mode == PLAIN_FORWARD) {
             if (ok)
                 for (int i = threadIdx.x >> lg; i < n; i += step) G.g[(size_t)i * PL] = cscale(X[(i << lg) + w], a.scale);
@@ -228,6 +305,7 @@ template <typename T> bool plain_setup(PlainArgs<T> &a, int nsm) {
         if (2 * cb * ((size_t)a.n0 << a.lg0) <= 72 * 1024 && (PL >> a.lg0) >= nsm) break;
     if (2 * cb * ((size_t)a.n0 << a.lg0) > 200 * 1024) return false;
     a.magic_n = (unsigned)(((1ull << 32) + a.n2 - 1) / a.n2);
+    a.magic_n4 = a.n2 >= 8 ? (unsigned)(((1ull << 32) + a.n2 / 4 - 1) / (a.n2 / 4)) : 0;
     a.magic_n2h = (unsigned)(((1ull << 32) + a.n2h - 1) / a.n2h);
     return prepare_once<T>() == cudaSuccess;
 }
@@ -237,18 +315,22 @@ cudaError_t launch_plain_mean(const T *u, long long N, int nblk, double *part, d
     plain_mean_kernel<T><<<nblk, 256, 0, s>>>(u, N, part, scal, ticket);
     return cudaGetLastError();
 }
-template <typename T> cudaError_t launch_plain_rows(const PlainArgs<T> &a, bool inverse, cudaStream_t s) {
+template <typename T> cudaError_t launch_plain_rows(const PlainArgs<T> &a_in, bool inverse, cudaStream_t s) {
+    // 16-byte (FP32) accesses where every row of every field starts on such a boundary
+    PlainArgs<T> a = a_in;
+    const uintptr_t at = (uintptr_t)a.u | (uintptr_t)a.out | (uintptr_t)a.v | (uintptr_t)a.vu | (uintptr_t)a.base;
+    a.vec = a.n2 % 4 == 0 && a.n2 >= 8 && at % 16 == 0;
     const long long R = (long long)a.n0 * a.n1;
     const unsigned nb = (unsigned)((R + (2 << a.lgB) - 1) >> (a.lgB + 1));
     const size_t sm = 2 * 2 * sizeof(T) * (size_t)a.n2 * ((1 << a.lgB) + 1);
-    if (inverse) plain_rows_inv<T><<<nb, 256, sm, s>>>(a);
-    else plain_rows_fwd<T><<<nb, 256, sm, s>>>(a);
+    if (inverse) plain_rows_inv<T><<<nb, kPlainThreads, sm, s>>>(a);
+    else plain_rows_fwd<T><<<nb, kPlainThreads, sm, s>>>(a);
     return cudaGetLastError();
 }
 template <typename T> cudaError_t launch_plain_n0(const PlainArgs<T> &a, cudaStream_t s) {
     const long long PL = (long long)a.n1 * a.n2h;
     const unsigned nb = (unsigned)((PL + (1 << a.lg0) - 1) >> a.lg0);
-    plain_n0<T><<<nb, 256, 2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s>>>(a);
+    plain_n0<T><<<nb, kPlainThreads, 2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s>>>(a);
     return cudaGetLastError();
 }
 #define INST(T)                                                                                                     \

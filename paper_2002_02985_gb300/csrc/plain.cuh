@@ -14,10 +14,12 @@ template <typename T> struct PlainArgs {
     int n0, n1, n2, n2h;
     AnyPlan q0, q2;
     int lgB, lg0, mode;
-    unsigned magic_n, magic_n2h;
+    unsigned magic_n, magic_n2h, magic_n4;
+    int vec;                     // set at the launch: four points per access
     C *h;                        // half spectrum
     const C *tw0, *tw2;
-    const double *scal;          // S_RHO_MEAN of the field
+    const double *scal;          // S_RHO_MEAN: the constant the forward rows subtract
+    int sampled;                 // they take it from a sample of the field (and leave it there)
     const T *u;                  // input field
     T *out;
     const T *v, *vu, *base;      // epilogue out = c0 base + c1 (y + madd mean + v vu)
