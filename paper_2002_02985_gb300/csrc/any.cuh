@@ -196,6 +196,7 @@ __device__ __forceinline__ void pencil_any_body(const EvalArgs<T> &a, const int 
 template <typename T, int DIR>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     pencil_any_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
+    pdl_begin();
     int bid;
     const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -141,8 +141,11 @@ template <typename T> cudaError_t launch_forward_rows_cols(const EvalArgs<T> &a,
 
 template <typename T>
 cudaError_t launch_pencils(const EvalArgs<T> &a, const LaunchSet &ks, bool inverse, cudaStream_t s) {
-    return launch(inverse ? ks.pen_inv : ks.pen_fwd, dim3(pencil_tiles(a, inverse ? a.ncol_inv : a.ncol)), a.thr_p1,
-                  pen_smem(a), a, s);
+    const EvalArgs<T> *ga = nullptr;
+    int bps = 0;
+    void *args[] = {(void *)&a, (void *)&ga, (void *)&bps};
+    return launch_pdl(inverse ? ks.pen_inv : ks.pen_fwd, pencil_tiles(a, inverse ? a.ncol_inv : a.ncol),
+                      (unsigned)a.thr_p1, args, pen_smem(a), s);
 }
 
 template <typename T>

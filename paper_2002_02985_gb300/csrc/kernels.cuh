@@ -1633,6 +1633,7 @@ __global__ void __launch_bounds__(P::max_threads, P::min_blocks) row_fwd_kernel(
 }
 template <typename T, int DIR, class P>
 __global__ void __launch_bounds__(P::max_threads, P::min_blocks) pencil1_kernel(EvalArgs<T> a) {
+    pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int f = DIR > 0 ? a.fin : 0;
     if (f && blockIdx.x == 0) energies_block(a, (double *)smem_raw);

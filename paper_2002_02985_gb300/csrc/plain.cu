@@ -20,6 +20,7 @@ constexpr int kPlainThreads = 128;
 template <typename T>
 __global__ void __launch_bounds__(256) plain_mean_kernel(const T *u, long long N, double *part, double *scal,
                                                          unsigned *ticket) {
+    pdl_begin();
     __shared__ double sd[32];
     __shared__ bool last;
     double acc = 0.0;
@@ -113,6 +114,7 @@ template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<
     return s;
 }
 template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_rows_fwd(const __grid_constant__ PlainArgs<T> a) {
+    pdl_begin();
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
@@ -152,6 +154,7 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
 // out = c0 base + c1 (y + madd mean + v u), y the inverse transform (null pointers: left out); out
 // overlaps none of the inputs
 template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_rows_inv(const __grid_constant__ PlainArgs<T> a) {
+    pdl_begin();
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
@@ -219,6 +222,7 @@ template <typename T> __device__ __forceinline__ T plain_factor(const PlainArgs<
     return g2 > (T)0 ? a.p1 * g2 / (g2 * g2 + a.p1 * g2 + a.p2) : (T)1;       // PLAIN_PRECOND
 }
 template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_n0(const __grid_constant__ PlainArgs<T> a) {
+    pdl_begin();
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const AnyPlan &q = a.q0;
@@ -312,8 +316,8 @@ template <typename T> bool plain_setup(PlainArgs<T> &a, int nsm) {
 template <typename T>
 cudaError_t launch_plain_mean(const T *u, long long N, int nblk, double *part, double *scal, unsigned *ticket,
                               cudaStream_t s) {
-    plain_mean_kernel<T><<<nblk, 256, 0, s>>>(u, N, part, scal, ticket);
-    return cudaGetLastError();
+    void *args[] = {(void *)&u, (void *)&N, (void *)&part, (void *)&scal, (void *)&ticket};
+    return launch_pdl((const void *)plain_mean_kernel<T>, (unsigned)nblk, 256, args, 0, s);
 }
 template <typename T> cudaError_t launch_plain_rows(const PlainArgs<T> &a_in, bool inverse, cudaStream_t s) {
     // 16-byte (FP32) accesses where every row of every field starts on such a boundary
@@ -323,15 +327,15 @@ template <typename T> cudaError_t launch_plain_rows(const PlainArgs<T> &a_in, bo
     const long long R = (long long)a.n0 * a.n1;
     const unsigned nb = (unsigned)((R + (2 << a.lgB) - 1) >> (a.lgB + 1));
     const size_t sm = 2 * 2 * sizeof(T) * (size_t)a.n2 * ((1 << a.lgB) + 1);
-    if (inverse) plain_rows_inv<T><<<nb, kPlainThreads, sm, s>>>(a);
-    else plain_rows_fwd<T><<<nb, kPlainThreads, sm, s>>>(a);
-    return cudaGetLastError();
+    void *args[] = {(void *)&a};
+    return launch_pdl(inverse ? (const void *)plain_rows_inv<T> : (const void *)plain_rows_fwd<T>, nb, kPlainThreads, args,
+                      sm, s);
 }
 template <typename T> cudaError_t launch_plain_n0(const PlainArgs<T> &a, cudaStream_t s) {
     const long long PL = (long long)a.n1 * a.n2h;
     const unsigned nb = (unsigned)((PL + (1 << a.lg0) - 1) >> a.lg0);
-    plain_n0<T><<<nb, kPlainThreads, 2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s>>>(a);
-    return cudaGetLastError();
+    void *args[] = {(void *)&a};
+    return launch_pdl((const void *)plain_n0<T>, nb, kPlainThreads, args, 2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s);
 }
 #define INST(T)                                                                                                     \
     template bool plain_setup<T>(PlainArgs<T> &, int);                                                              \
