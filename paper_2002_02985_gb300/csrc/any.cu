@@ -82,6 +82,10 @@ bool any_ct_axis0_1(int, AnyCt &);
 bool any_ct_axis0_2(int, AnyCt &);
 bool any_ct_axis0_3(int, AnyCt &);
 bool any_ct_axis0_4(int, AnyCt &);
+bool any_ct_pencil_1(int, AnyCt &);
+bool any_ct_pencil_2(int, AnyCt &);
+bool any_ct_pencil_3(int, AnyCt &);
+bool any_ct_pencil_4(int, AnyCt &);
 bool any_ct_rows_1(int, AnyCt &);
 bool any_ct_rows_2(int, AnyCt &);
 bool any_ct_rows_3(int, AnyCt &);
@@ -106,11 +110,20 @@ template <typename T> void any_candidates(int role, int n, long long cols, int n
     };
     const AnyPlan q = any_plan(n);
     if (role == ROLE_PENCIL && q.np >= 2) {
+        AnyCt ct;
+        if (sizeof(T) == 4 && (any_ct_pencil_1(n, ct) || any_ct_pencil_2(n, ct) || any_ct_pencil_3(n, ct) || any_ct_pencil_4(n, ct))) {
+            c.any = 2;
+            add(ct.k, ct.k2, 1 << ct.lg, ct.nt, "ctpencil");
+            return;
+        }
         // 16-column tiles (128-byte rows in FP32) while three blocks fit an SM, else 8
+        int rmax = 1;
+        for (int i = 0; i < q.np; i++) rmax = std::max(rmax, q.p[i].R);
         for (int lg : {4, 3}) {
             if (any_pencil_smem<T>(q, lg) > 74 * 1024 && lg > 3) continue;
             if (any_pencil_smem<T>(q, lg) > 200 * 1024) continue;
-            add((const void *)pencil_any_kernel<T, -1>, (const void *)pencil_any_kernel<T, +1>, 1 << lg, 256, "anypencil");
+            add((const void *)pencil_any_kernel<T, -1>, (const void *)pencil_any_kernel<T, +1>, 1 << lg,
+                any_ct_pencil_threads(n, rmax, lg), "anypencil");
             break;
         }
     }

@@ -161,16 +161,26 @@ __device__ __forceinline__ const EvalArgs<T> &any_args(const EvalArgs<T> &a, con
 }
 
 // ---------------------------------------------------------------- pencils (C2C along n1)
+// block size: a thread per butterfly of the pass with the fewest (at 256 for all lengths half the
+// threads of short or unequal plans had none), 85 registers
+constexpr int any_max3(int a, int b, int c) { return a > b ? (a > c ? a : c) : (b > c ? b : c); }
+constexpr int any_ct_pencil_threads(int n, int rmax, int lg) {
+    const int t = ((n / rmax << lg) + 31) / 32 * 32;
+    return t < 64 ? 64 : (t > 256 ? 256 : t);
+}
 // One tile of 2^lg consecutive columns per block.  The first pass takes its inputs straight
 // from global memory into registers and the last one stores straight from registers (a warp
 // reads and writes whole rows of the tile), so an element crosses shared memory once per
 // exchange and nothing else; many small blocks per SM keep the loads in flight.
-template <typename T, int DIR>
+// (R1 = 0: the launch's plan and tile width; else n1 = R1 R2 R3, R3 = 1 for two passes, and 2^LG columns)
+template <typename T, int DIR, int R1 = 0, int R2 = 1, int R3 = 1, int LG = 0>
 __device__ __forceinline__ void pencil_any_body(const EvalArgs<T> &a, const int bid) {
     typedef typename Vec2<T>::type C;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr bool CT = R1 > 0;
+    constexpr int NC = CT ? R1 * R2 * R3 : 1;
     const AnyPlan &q = a.q1;
-    const int n = q.n, lg = a.lg1, TW = 1 << lg, n2h = a.n2h, np = q.np;
+    const int n = CT ? NC : q.n, lg = CT ? LG : a.lg1, TW = 1 << lg, n2h = a.n2h, np = CT ? (R3 > 1 ? 3 : 2) : q.np;
     C *const X = (C *)smem_raw, *const Y = X + (np > 2 ? (n << lg) : 0);
     const int ncols = a.n0 * n2h;
     const int ntile = (ncols + TW - 1) >> lg;
@@ -185,6 +195,19 @@ __device__ __forceinline__ void pencil_any_body(const EvalArgs<T> &a, const int 
     auto dec = [&](int idx, int &b, int &j) { b = w; j = idx >> lg; };
     const AnyGlobal<C> G{g, n2h, ok};
     const AnyShared<C> SX{X, TW}, SY{Y, TW};
+    if constexpr (CT) {
+        constexpr int NT = any_ct_pencil_threads(NC, any_max3(R1, R2, R3), LG);
+        any_pass_r<DIR, R1>(any_const_pass(NC, R1, 1), NC / R1 << LG, NT, tw, dec, G, SX);
+        __syncthreads();
+        if constexpr (R3 > 1) {
+            any_pass_r<DIR, R2>(any_const_pass(NC, R2, R1), NC / R2 << LG, NT, tw, dec, SX, SY);
+            __syncthreads();
+            any_pass_r<DIR, R3>(any_const_pass(NC, R3, R1 * R2), NC / R3 << LG, NT, tw, dec, SY, G);
+        } else {
+            any_pass_r<DIR, R2>(any_const_pass(NC, R2, R1), NC / R2 << LG, NT, tw, dec, SX, G);
+        }
+        return;
+    }
     any_pass<DIR>(q.p[0], q.p[0].nb << lg, tw, dec, G, SX);
     __syncthreads();
     if (np > 2) {
@@ -203,6 +226,19 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 2)
     const int f = DIR > 0 ? ar.fin : 0;
     if (f && bid == 0) energies_block(ar, (double *)smem_raw);
     else pencil_any_body<T, DIR>(ar, bid - f);
+}
+
+template <typename T, int DIR, int R1, int R2, int R3, int LG>
+__global__ void __launch_bounds__(any_ct_pencil_threads(R1 *R2 *R3, any_max3(R1, R2, R3), LG),
+                                  768 / any_ct_pencil_threads(R1 *R2 *R3, any_max3(R1, R2, R3), LG))
+    pencil_ct_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
+    pdl_begin();
+    int bid;
+    const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int f = DIR > 0 ? ar.fin : 0;
+    if (f && bid == 0) energies_block(ar, (double *)smem_raw);
+    else pencil_any_body<T, DIR, R1, R2, R3, LG>(ar, bid - f);
 }
 
 // ---------------------------------------------------------------- reciprocal-space pass
