@@ -146,30 +146,38 @@ template <typename T> void any_candidates(int role, int n, long long cols, int n
     if (role == ROLE_AXIS0) {
         int made = 0;
         AnyCt ct;
+        // blocks per tile: 1 where the tiles fill the SMs, else up to two blocks per SM
+        auto split = [&](int lg) {
+            const long long tiles = (cols + (1 << lg) - 1) >> lg;
+            return tiles >= nsm ? 1 : (int)std::max(1LL, std::min<long long>(kMaxSplit, 2 * nsm / tiles));
+        };
+        auto put = [&](const void *k, const void *km, int RL, int lg, int nt, const char *kind) {
+            c.RL = RL;
+            c.split = split(lg);
+            add(k, km, 1 << lg, nt, kind);
+            std::snprintf(out.back().name, sizeof(c.name), "%s r%d %dx%d s%d", kind, RL, 1 << lg, nt, c.split);
+            made++;
+        };
         if (sizeof(T) == 4 && (any_ct_axis0_1(n, ct) || any_ct_axis0_2(n, ct) || any_ct_axis0_3(n, ct) || any_ct_axis0_4(n, ct))) {
             c.any = 2;
-            c.RL = ct.RL;
-            add(ct.k, ct.k2, 1 << ct.lg, ct.nt, "ctrecip");
+            put(ct.k, ct.k2, ct.RL, ct.lg, ct.nt, "ctrecip");
             c.any = 1;
             // the run-time kernels only where the compiled tiles leave SMs without one
-            if ((cols >> ct.lg) >= nsm) return;
+            if (c.split == 1) return;
         }
         for (int RL : {16, 15, 12, 10, 9, 8, 5, 4}) {
             const void *k = any_axis0_kernel<T>(RL, false), *km = any_axis0_kernel<T>(RL, true);
-            if (!k || n % RL || any_plan(n, RL).np < 2 || made >= 3) continue;
+            if (!k || n % RL || any_plan(n, RL).np < 2 || made >= 4) continue;
             const int tmax = sizeof(T) == 4 ? (RL >= 12 ? 256 : 512) : 256;
-            // 16 columns where the block and its tiles leave room for two blocks per SM and the
-            // grid has a tile for every SM, else 8, else 4
+            // the widest of 16, 8 or 4 columns that leaves room for two blocks per SM, and the
+            // narrowest as well where the grid has fewer tiles than SMs
+            int widest = -1;
             for (int lg : {4, 3, 2}) {
-                if (lg > 2 && (cols >> lg) < nsm) continue;
                 const int nt = ((n / RL << lg) + 31) / 32 * 32;
                 if (nt > tmax || any_axis0_smem<T>(n, lg) > (lg == 4 ? 100 : 200) * 1024) continue;
-                c.RL = RL;
-                add(k, km, 1 << lg, nt, "anyrecip");
-                std::snprintf(c.name, sizeof(c.name), "anyrecip r%d %dx%d", RL, 1 << lg, nt);
-                std::snprintf(out.back().name, sizeof(c.name), "%s", c.name);
-                made++;
-                break;
+                if (widest >= 0 && !(lg == 2 && (cols >> widest) < nsm)) continue;
+                if (widest < 0) widest = lg;
+                put(k, km, RL, lg, nt, "anyrecip");
             }
         }
     }

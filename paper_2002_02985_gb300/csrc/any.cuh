@@ -249,6 +249,10 @@ __global__ void __launch_bounds__(any_ct_pencil_threads(R1 *R2 *R3, any_max3(R1,
 // The next channel's tile arrives by cp.async while the current one is worked on; the last
 // inverse pass stores straight to global memory.  rho^beta hat, the term-2 accumulator and
 // |G| stay in registers for the whole tile.
+//
+// A grid of few tiles (32^3: 34 of 16 columns) leaves most SMs idle while one block takes the
+// channels in turn, about 2 us each; there up to eight blocks share a tile's channels.
+//
 // R1 = 0: the plan and the tile width of the launch; R1 > 0: n0 = R1 R2 RL (R2 = 1: two passes)
 // and 2^LG columns, fixed at compile time.
 template <typename T, int RL, bool MGP, int R1 = 0, int R2 = 1, int LG = 0>
@@ -272,7 +276,8 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
     const bool nl = a.terms & 4u;
     const int w = threadIdx.x & (TW - 1), t = threadIdx.x >> lg;
     const bool act = t < m;                                  // (the block is rounded up to whole warps)
-    const int col = (bid << lg) + w;
+    const int S = a.ax0_split, tile = S > 1 ? bid / S : bid, sp = bid - tile * S;
+    const int col = (tile << lg) + w;
     const bool ok = col < PL;
     // the channels in load order and the operations of the tile, as in the persistent kernel
     if (threadIdx.x == 0) {
@@ -285,16 +290,21 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
             no++;
             if (fwd) order[nload++] = (short)(kind == OP_RB ? CH_NL : store);
         };
-        if (hp) op(OP_HPP, 1, CH_HPP, 0);
-        if (a.terms & 2u) op(OP_VW, 1, CH_VW, 0);
+        // (a tile shared by S blocks: the channels go round, every block transforms rho^beta for its
+        // knots and leaves its part of term 2 in a slot of its own, summed by the inverse rows)
+        int u = 0;
+        auto mine = [&]() { return S == 1 || u++ % S == sp; };
+        if (hp && mine()) op(OP_HPP, 1, CH_HPP, 0);
+        if ((a.terms & 2u) && mine()) op(OP_VW, 1, CH_VW, 0);
         if (nl) {
             op(OP_RB, 1, -1, 0);
             if (!lwt) {
                 op(OP_WT, 1, CH_KNOT0, 0);
                 op(OP_RR, 0, CH_NL, 0);
             } else {
-                for (int k = 0; k < a.M; k++) op(exact ? OP_EX : OP_IP, exact ? 1 : 0, CH_KNOT0 + k, k);
-                if (exact) op(OP_A, 0, CH_NL, 0);
+                for (int k = 0; k < a.M; k++)
+                    if (mine()) op(exact ? OP_EX : OP_IP, exact ? 1 : 0, CH_KNOT0 + k, k);
+                if (exact) op(OP_A, 0, S > 1 ? a.t2_slot + sp : CH_NL, 0);
             }
         }
         s_nload = nload;

@@ -89,7 +89,7 @@ template <typename T> struct Workspace {
     int Brow = 0, thr_rowf = 0, thr_rowi = 0, TW1 = 0, thr_p1 = 0, TW0 = 0, thr_ax0 = 0, nb_row = 0, nb_ax0 = 0;
     int grid_p1 = 0;
     // any-length kernels in use per role, their tile widths (log2), plans, largest row group
-    int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0;
+    int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0, split = 1;
     AnyPlan q0, q0i, q1, q2;
     int TW0_p = 0, thr_ax0_p = 0;     // the runtime-size n0 transform of plain fields
     bool plain_any = false;           // the any-length plain transforms (plain.cu) serve this grid
@@ -298,6 +298,7 @@ template <typename T> int apply_cand(ofdft_grid *g, Workspace<T> &w, int role, c
     } else {
         const long long P = (long long)g->n[1] * g->n2h;
         w.any0 = c.any;
+        w.split = c.split;
         if (c.any) {
             for (w.lg0 = 0; (1 << w.lg0) < c.B;) w.lg0++;
             w.q0 = any_plan(g->n[0], c.RL);      // (unused by the compiled plans)
@@ -406,7 +407,7 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
     for (const KernelCand &k : w.cand[TUNE_AXIS0])
         w.nb_ax0 = std::max(w.nb_ax0, k.recip.k ? (int)std::min((P + k.recip.tw - 1) / k.recip.tw,
                                                                 (long long)k.recip.per_sm * g->nsm)
-                                                 : (int)((P + k.B - 1) / k.B));
+                                                 : (int)((P + k.B - 1) / k.B) * k.split);
     for (const KernelCand &k : w.cand[TUNE_ROWS]) min_brow = std::min(min_brow, k.batched ? 1 : k.B);
     for (int r = 0; r < TUNE_NROLE; r++) {
         for (const KernelCand &k : w.cand[r]) {
@@ -820,6 +821,16 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
     return OFDFT_OK;
 }
 
+// channel slots of an evaluation: Hartree + ions, vW, rho^beta (and K rho^alpha or the knots), and on
+// grids with fewer column tiles than SMs the term-2 slots of the blocks that share a tile
+int eval_slots(const ofdft_grid *g, const ofdft_functional *f) {
+    if (!(f->terms & OFDFT_TERM_NL)) return 3;
+    if (f->kernel != OFDFT_KERNEL_LWT) return 4;
+    const long long cols = (long long)g->n[1] * g->n2h;
+    const bool shared = f->nl_potential == OFDFT_NLPOT_EXACT && cols / 16 < g->nsm;
+    return 3 + f->n_knots + (shared ? kMaxSplit : 0);
+}
+
 // blocks of the stats kernel: a thread reads four points at a time, and a small grid makes no
 // more blocks than it has work for (their partials are summed by one block)
 int stats_blocks(const ofdft_grid *g) {
@@ -891,8 +902,7 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     const bool nl = f->terms & OFDFT_TERM_NL;
     const bool lwt = nl && f->kernel == OFDFT_KERNEL_LWT;
     const int M = lwt ? f->n_knots : 0;
-    const int nslots = nl ? (lwt ? 3 + M : 4) : 3;
-    int rc = ensure_ws<T>(g, nslots);
+    int rc = ensure_ws<T>(g, eval_slots(g, f));
     if (rc) return rc;
     Workspace<T> &w = ws<T>(g);
     if (f->terms & OFDFT_TERM_PP) {
@@ -944,7 +954,10 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     a.ticket = w.ticket;
     a.nb_stats = stats_blocks(g);
     a.clear_flags = 1;
-    a.nb_ax0 = w.ks.recip.k ? w.recip_grid : w.tile_nb_ax0;
+    // (a tile's channels are shared out by knots: one knot at least for every block)
+    a.ax0_split = lwt && M >= w.split ? w.split : 1;
+    a.t2_slot = CH_KNOT0 + M;
+    a.nb_ax0 = w.ks.recip.k ? w.recip_grid : w.tile_nb_ax0 * a.ax0_split;
     a.nb_row = (int)((((long long)g->n[0] * g->n[1] + 1) / 2 + w.Brow - 1) / w.Brow);   // the row kernels' grid
     a.p0 = g->plan[0];
     a.p1 = g->plan[1];
@@ -994,8 +1007,14 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
         else
             for (int m = 0; m < M; m++) a.col_ch[a.ncol++] = CH_KNOT0 + m;
     }
-    for (int i = 0; i < a.ncol; i++)
-        if (!(lwt && !exact && a.col_ch[i] == CH_NL)) a.col_inv_ch[a.ncol_inv++] = a.col_ch[i];
+    // (term 2 comes back in the rho^beta channel, or in one slot per block that shared a tile)
+    const int nt2 = lwt && exact ? a.ax0_split : 0;
+    for (int i = 0; i < a.ncol; i++) {
+        if (a.col_ch[i] == CH_NL && lwt && (!exact || nt2 > 1)) continue;
+        a.col_inv_ch[a.ncol_inv++] = a.col_ch[i];
+    }
+    if (nt2 > 1)
+        for (int k = 0; k < nt2; k++) a.col_inv_ch[a.ncol_inv++] = a.t2_slot + k;
     if (hpp) { a.inv_ch[a.ninv] = CH_HPP; a.inv_kind[a.ninv++] = CONS_ADD; }
     if (vw) { a.inv_ch[a.ninv] = CH_VW; a.inv_kind[a.ninv++] = CONS_VW; }
     if (nl) {
@@ -1003,7 +1022,10 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
             a.inv_ch[a.ninv] = CH_NL; a.inv_kind[a.ninv++] = CONS_WT_A;
             a.inv_ch[a.ninv] = CH_KNOT0; a.inv_kind[a.ninv++] = CONS_WT_B;
         } else {
-            if (exact) { a.inv_ch[a.ninv] = CH_NL; a.inv_kind[a.ninv++] = CONS_T2; }
+            for (int k = 0; k < nt2; k++) {
+                a.inv_ch[a.ninv] = nt2 > 1 ? a.t2_slot + k : CH_NL;
+                a.inv_kind[a.ninv++] = CONS_T2;
+            }
             for (int m = 0; m < M; m++) {
                 a.inv_ch[a.ninv] = CH_KNOT0 + m;
                 a.inv_kind[a.ninv] = CONS_KNOT;
@@ -2274,9 +2296,7 @@ cudaStream_t *batch_streams() {
 template <typename T>
 int prepare_batch_grid(ofdft_grid *g, const ofdft_functional *f, bool forces, const T *rho) {
     const bool nl = f->terms & OFDFT_TERM_NL;
-    const bool lwt = nl && f->kernel == OFDFT_KERNEL_LWT;
-    const int nslots = nl ? (lwt ? 3 + f->n_knots : 4) : 3;
-    int rc = ensure_ws<T>(g, nslots);
+    int rc = ensure_ws<T>(g, eval_slots(g, f));
     if (rc) return rc;
     if ((f->terms & OFDFT_TERM_PP) && (rc = ensure_vext<T>(g))) return rc;
     if (forces && (rc = ensure_force_buffers<T>(g))) return rc;
@@ -2319,7 +2339,8 @@ template <typename T> std::vector<unsigned char> launch_signature(const LaunchSe
     const int v[] = {a.n0,       a.n1,       a.n2,    a.nb_stats, a.nb_ax0, a.nb_row, a.Brow,     a.thr_rowf,
                      a.thr_rowi, a.TW1,      a.thr_p1, tile[0],   tile[1],  tile[2],  a.grid_p1,  a.row2_G,
                      a.nfwd,     a.ncol,     a.ncol_inv, a.exact_sums, a.mgp_tab != nullptr,
-                     a.any0,     a.any1,     a.any2,  a.lg0,      a.lg1,    a.any_G[0], a.any_G[1], a.fin};
+                     a.any0,     a.any1,     a.any2,  a.lg0,      a.lg1,    a.any_G[0], a.any_G[1], a.fin,
+                     a.ax0_split};
     append_bytes(k, v);
     return k;
 }

@@ -38,7 +38,8 @@ enum {
 // energy slots: total, TF, vW, NL, H, PP, XC
 enum { E_TOT = 0, E_TF = 1, E_VW = 2, E_NL = 3, E_H = 4, E_PP = 5, E_XC = 6, E_NUM = 7 };
 
-constexpr int kMaxChan = 3 + OFDFT_MAX_KNOTS;
+constexpr int kMaxSplit = 8;         // blocks that share one column tile of the n0 pass (small grids)
+constexpr int kMaxChan = 3 + OFDFT_MAX_KNOTS + kMaxSplit;
 constexpr int kGroupMax = 32;        // evaluations per grouped launch (tensor maps in the parameters)
 constexpr int kMaxThreads = 512;     // block size bound of the FFT kernels
 
@@ -97,6 +98,8 @@ template <typename T> struct EvalArgs {
     // the column tiles, channels per row group (forward, inverse), reciprocals of the row indices
     int any0, any1, any2, lg0, lg1, any_G[2];
     AnyPlan q0, q0i, q1, q2;
+    // blocks per column tile of the n0 pass, and the first of their term-2 slots when more than one
+    int ax0_split, t2_slot;
     unsigned magic_n2h, magic_2n2h, magic_G[2];
     int clear_flags;                     // an evaluation (its stats kernel sets the flags), not a plain transform
     int fin;                             // the inverse n1 pencils' launch has a block 0 that makes the energies
@@ -235,7 +238,7 @@ struct KernelCand {
     bool batched = false;                 // channel-batched row kernels (B = channels per group)
     // any-length kernels (any.cuh): 1 the plan read at run time, 2 compiled; B = tile width or
     // largest channel group
-    int any = 0, RL = 0;
+    int any = 0, RL = 0, split = 1;       // (split: blocks per column tile of the n0 pass)
     RecipLaunch recip;
     char name[48] = {0};
 };
