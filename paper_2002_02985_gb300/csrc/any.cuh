@@ -485,7 +485,8 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
         else any_pass<+1>(qi.p[np - 1], qi.p[np - 1].nb << lg, tw, dec, sh(S), G);
     }
     double r4[4] = {eH, eV, eP, eN};
-    if constexpr (sizeof(T) == 4) block_sum_n_f32warp<4>(r4, sd);
+    // (a tile shared by several blocks: FP64 throughout, its few blocks hide the slow adds)
+    if (sizeof(T) == 4 && S == 1) block_sum_n_f32warp<4>(r4, sd);
     else block_sum_n<4>(r4, sd);
     if (threadIdx.x == 0)
         for (int k = 0; k < 4; k++) a.part_ax0[4 * bid + k] = r4[k];
