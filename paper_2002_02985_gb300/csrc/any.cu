@@ -78,10 +78,10 @@ AnyPlan any_reversed(const AnyPlan &q) {
 template <typename T> const void *any_axis0_kernel(int RL, bool mgp);
 
 // the compile-time plans (any_ct*.cu)
-bool any_ct_axis0_1(int, AnyCt &);
-bool any_ct_axis0_2(int, AnyCt &);
-bool any_ct_axis0_3(int, AnyCt &);
-bool any_ct_axis0_4(int, AnyCt &);
+bool any_ct_axis0_1(int, bool, AnyCt &);
+bool any_ct_axis0_2(int, bool, AnyCt &);
+bool any_ct_axis0_3(int, bool, AnyCt &);
+bool any_ct_axis0_4(int, bool, AnyCt &);
 bool any_ct_pencil_1(int, AnyCt &);
 bool any_ct_pencil_2(int, AnyCt &);
 bool any_ct_pencil_3(int, AnyCt &);
@@ -158,12 +158,18 @@ template <typename T> void any_candidates(int role, int n, long long cols, int n
             std::snprintf(out.back().name, sizeof(c.name), "%s r%d %dx%d s%d", kind, RL, 1 << lg, nt, c.split);
             made++;
         };
-        if (sizeof(T) == 4 && (any_ct_axis0_1(n, ct) || any_ct_axis0_2(n, ct) || any_ct_axis0_3(n, ct) || any_ct_axis0_4(n, ct))) {
+        auto compiled = [&](bool narrow) {
+            return any_ct_axis0_1(n, narrow, ct) || any_ct_axis0_2(n, narrow, ct) || any_ct_axis0_3(n, narrow, ct) ||
+                   any_ct_axis0_4(n, narrow, ct);
+        };
+        if (sizeof(T) == 4 && compiled(false)) {
             c.any = 2;
             put(ct.k, ct.k2, ct.RL, ct.lg, ct.nt, "ctrecip");
-            c.any = 1;
             // the run-time kernels only where the compiled tiles leave SMs without one
-            if (c.split == 1) return;
+            const bool enough = c.split == 1;
+            if (compiled(true)) put(ct.k, ct.k2, ct.RL, ct.lg, ct.nt, "ctrecip");
+            c.any = 1;
+            if (enough) return;
         }
         for (int RL : {16, 15, 12, 10, 9, 8, 5, 4}) {
             const void *k = any_axis0_kernel<T>(RL, false), *km = any_axis0_kernel<T>(RL, true);

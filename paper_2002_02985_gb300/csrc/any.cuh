@@ -504,18 +504,44 @@ __global__ void __launch_bounds__(any_ax0_threads<T, RL>(), 1)
     axis0_any_body<T, RL, MGP>(ar, bid);
 }
 
-// compile-time lengths: as many blocks per SM as 128 registers a thread (255 from RL = 12 on) allow
+// compile-time lengths: as many blocks per SM as 128 registers a thread allow, 168 from RL = 12 on
+// (the spectra, the kernel state and term 2 of 12 to 15 frequencies fit without spills) and 255 at 16
 constexpr int any_ct_threads(int N, int RL, int lg) { return ((N / RL << lg) + 31) / 32 * 32; }
 constexpr int any_ct_blocks(int N, int RL, int lg) {
-    const int b = (RL >= 12 ? 256 : 512) / any_ct_threads(N, RL, lg);
+    const int b = (RL >= 16 ? 256 : (RL >= 12 ? 384 : 512)) / any_ct_threads(N, RL, lg);
     return b > 1 ? b : 1;
 }
+// Columns per tile (log2) of the compiled pass.  RL >= 12: 8 columns, so that two or three blocks
+// of 128 threads share an SM and cover one another's barriers (with 16 columns one block of 8 warps
+// issued in 29 % of the cycles; whole evaluations at 180^3 / 192^3 / 240^3 / 256^3: 1.356 / 2.014 /
+// 3.167 / 3.606 -> 1.245 / 1.903 / 2.969 / 3.534 ms).  Smaller RL keep the list's width, and from 72
+// points on the tuner may take 8 columns where that fills the last wave of blocks better (108^3:
+// 0.340 -> 0.299 ms, 100^3: 0.260 -> 0.257, 144^3: 0.689 -> 0.673; 96^3 and 160^3 keep 16).
+constexpr int any_ct_lg(int RL, int W) { return RL >= 12 ? 3 : W; }
+constexpr bool any_ct_narrow(int N, int RL, int W) { return N >= 72 && RL < 12 && W == 4; }
 template <typename T, int R1, int R2, int RL, int LG, bool MGP>
 __global__ void __launch_bounds__(any_ct_threads(R1 *R2 *RL, RL, LG), any_ct_blocks(R1 *R2 *RL, RL, LG))
     axis0_ct_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
     int bid;
     const EvalArgs<T> &ar = any_args(a, ga, bps, bid);
     axis0_any_body<T, RL, MGP, R1, R2, LG>(ar, bid);
+}
+
+// the compiled pass of n0 = R1 R2 RL at its default width, or (narrow) at 8 columns
+template <int R1, int R2, int RL, int W> bool any_ct_axis0_pick(bool narrow, AnyCt &c) {
+    constexpr int N = R1 * R2 * RL;
+    auto put = [&](auto lg) {
+        constexpr int LG = decltype(lg)::value;
+        c.k = (const void *)axis0_ct_kernel<float, R1, R2, RL, LG, false>;
+        c.k2 = (const void *)axis0_ct_kernel<float, R1, R2, RL, LG, true>;
+        c.RL = RL;
+        c.lg = LG;
+        c.nt = any_ct_threads(N, RL, LG);
+        return true;
+    };
+    if (!narrow) return put(std::integral_constant<int, any_ct_lg(RL, W)>{});
+    if constexpr (any_ct_narrow(N, RL, W)) return put(std::integral_constant<int, 3>{});
+    return false;
 }
 
 // ---------------------------------------------------------------- rows

@@ -2,7 +2,8 @@
 // 2^a 3^b 5^c from 24 to 512 that three passes of the compiled radices reach.  X(R1, R2, RL, LG):
 // n = R1 R2 RL, RL the frequencies a thread of the reciprocal-space pass keeps (8 to 10 where
 // the radices allow: 128 registers, two to four blocks per SM), 2^LG columns per tile (16, or 8
-// where the three tiles of 16 would leave room for one block per SM).
+// where the three tiles of 16 would leave room for one block per SM); the reciprocal-space pass
+// takes its width from any_ct_lg, and a second form of 8 columns from any_ct_narrow.
 #pragma once
 
 #include "any.cuh"

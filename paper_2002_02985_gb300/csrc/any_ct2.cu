@@ -3,16 +3,9 @@
 
 namespace ofdft {
 
-bool any_ct_axis0_2(int n, AnyCt &c) {
+bool any_ct_axis0_2(int n, bool narrow, AnyCt &c) {
 #define X(A, B, D, W)                                                             \
-    if (n == A * B * D) {                                                          \
-        c.k = (const void *)axis0_ct_kernel<float, A, B, D, W, false>;            \
-        c.k2 = (const void *)axis0_ct_kernel<float, A, B, D, W, true>;            \
-        c.RL = D;                                                                     \
-        c.lg = W;                                                                     \
-        c.nt = any_ct_threads(A * B * D, D, W);                                  \
-        return true;                                                                  \
-    }
+    if (n == A * B * D) return any_ct_axis0_pick<A, B, D, W>(narrow, c);
     OFDFT_ANY_CT_2(X)
 #undef X
     return false;

@@ -50,6 +50,25 @@ def test_any_length_kernels_match_oracle(role, n):
         assert np.linalg.norm((V - Vo)[m]) / np.linalg.norm(Vo[m]) <= 1e-4, pick
 
 
+@pytest.mark.parametrize("n", (72, 128, 180, 256))
+@pytest.mark.parametrize("cols", [(3, 5), (15, 8)])
+def test_every_reciprocal_space_tile_width_matches_oracle(n, cols):
+    """All candidates of the pass (16 and 8 columns, shared and single tiles) where the last tile is ragged."""
+    shape = (n,) + cols
+    cell = np.diag([0.3 * max(m, 12) for m in shape])
+    pos = lattice_positions(cell, (max(1, round(n * 0.3 / 4.8)), 1, 1), n + 3)
+    rho = W.renormalise(W.apply_noise(W.gaussian_density(cell, shape, pos, 3.0, 1.0) + 5e-3, 0.03, n), cell,
+                        3.0 * len(pos))
+    kw = dict(n_knots=7)
+    for pick in range(10):                     # (indices past the candidates run the first one)
+        E, V, Eo, Vo, og, _ = run_both(cell, shape, pos, rho, kw, L.FP32_MIXED, Z=(3.0,), rc=(0.8,),
+                                       options=((L.OPTION_PICK_RECIP, pick),))
+        for k in ("TF", "vW", "NL", "H", "PP", "total"):
+            assert abs(E[k] - Eo[k]) / len(pos) <= 1e-6, (pick, k, E[k], Eo[k])
+        m = knot_mask(rho.astype(np.float32).astype(np.float64), 7)
+        assert np.linalg.norm((V - Vo)[m]) / np.linalg.norm(Vo[m]) <= 1e-4, pick
+
+
 @pytest.mark.parametrize("kw", [dict(n_knots=19, nl_potential=L.NLPOT_INTERP), dict(n_knots=5, kernel=L.KERNEL_WT_GLOBAL),
                                 dict(n_knots=6, mgp_x=1.0), dict(n_knots=40)])
 def test_any_length_modes_match_oracle(kw):
