@@ -77,10 +77,10 @@ template <typename T> struct Workspace {
     double *scal = nullptr, *energies = nullptr, *knots_d = nullptr;
     T *knots_t = nullptr, *invdk_t = nullptr, *part_minmax = nullptr;
     double *part_stats = nullptr, *part_ax0 = nullptr, *part_row = nullptr, *part_misc = nullptr;
-    unsigned *ticket = nullptr;       // stats completion counter
+    unsigned *ticket = nullptr;       // completion counters (stats; up to four sums of a launch)
     T *opt = nullptr;                 // optimiser fields (8 * N), allocated on demand
     T *opt_ext = nullptr;             // TN / L-BFGS fields (opt_ext_fields * N), on demand
-    T *td = nullptr;                  // TD-OFDFT fields (19 * N), on demand
+    T *td = nullptr;                  // TD-OFDFT fields (18 * N), on demand
     T *mgp_tab = nullptr;             // MGP correction table (kMgpTable points), on demand
     C *rhohat = nullptr;              // normalised rho_hat kept by an evaluation for the forces
     double mgp_y = 0.0;               // the y it was built for (0: not built)
@@ -209,7 +209,7 @@ int fail(ofdft_grid *g, int code, const char *what, cudaError_t e = cudaSuccess)
 static_assert(E_NUM == OFDFT_N_ENERGIES, "energy slots");
 constexpr long long kFormTableMax = 32LL << 20;   // doubles of the kept form-factor tables
 constexpr int kEnergySlot = 24;      // the energies' place behind the scalar slots (one copy fetches both)
-static_assert(S_FIN + 5 <= kEnergySlot, "scalar slots");
+static_assert(S_FIN + 5 <= kEnergySlot && kEnergySlot + E_NUM <= S_PAIR_MEAN && S_PAIR_MEAN < 64, "scalar slots");
 
 // every device allocation of a grid goes through here: the optional cap of
 // ofdft_set_option(OFDFT_OPTION_ALLOC_CAP) is checked first (out of memory past it)
@@ -489,8 +489,8 @@ template <typename T> int ensure_ws(ofdft_grid *g, int nslots) {
         CK(gmalloc(g, &w.part_ax0, 4 * (size_t)w.nb_ax0 * sizeof(double)), "cudaMalloc partials");
         CK(gmalloc(g, &w.part_row, (size_t)w.nb_row * sizeof(double)), "cudaMalloc partials");
         CK(gmalloc(g, &w.part_misc, 4096 * sizeof(double)), "cudaMalloc partials");
-        CK(gmalloc(g, &w.ticket, sizeof(unsigned)), "cudaMalloc ticket");
-        CK(cudaMemset(w.ticket, 0, sizeof(unsigned)), "memset ticket");
+        CK(gmalloc(g, &w.ticket, 4 * sizeof(unsigned)), "cudaMalloc ticket");
+        CK(cudaMemset(w.ticket, 0, 4 * sizeof(unsigned)), "memset ticket");
 
         w.ready = true;
     }
@@ -1130,18 +1130,18 @@ template <typename T> EvalArgs<T> plain_args(ofdft_grid *g, Workspace<T> &w, con
 template <typename T> PlainArgs<T> plain_any_args(Workspace<T> &w, ofdft_grid *g, int slot) {
     PlainArgs<T> a = w.pl;
     a.h = w.chan + (size_t)slot * g->NH;
+    a.hs = g->NH;
     a.tw0 = w.tw[0];
     a.tw2 = w.tw[2];
     a.scal = w.scal;
     a.c1 = a.scale = (T)1;
     return a;
 }
-// the n1 pencils of one slot, in place
-template <typename T> int plain_pencils(ofdft_grid *g, Workspace<T> &w, int slot, bool inverse) {
+// the n1 pencils of nf slots, in place
+template <typename T> int plain_pencils(ofdft_grid *g, Workspace<T> &w, int slot, bool inverse, int nf = 1) {
     EvalArgs<T> a = plain_args<T>(g, w, nullptr);
-    a.col_ch[0] = slot;
-    a.ncol_inv = 1;
-    a.col_inv_ch[0] = slot;
+    a.ncol = a.ncol_inv = nf;
+    for (int f = 0; f < nf; f++) a.col_ch[f] = a.col_inv_ch[f] = slot + f;
     CK(launch_pencils<T>(a, w.ks_plain, inverse, g->stream), "transform along n1");
     return OFDFT_OK;
 }
@@ -1150,7 +1150,7 @@ template <typename T> int plain_pencils(ofdft_grid *g, Workspace<T> &w, int slot
 template <typename T> int forward_plain(ofdft_grid *g, Workspace<T> &w, const T *field) {
     if (w.plain_any) {
         PlainArgs<T> p = plain_any_args<T>(w, g, CH_HPP);
-        p.u = field;
+        p.u[0] = field;
         CK(launch_plain_mean<T>(field, g->N, stats_blocks(g), w.part_stats, w.scal, w.ticket, g->stream), "mean");
         CK(launch_plain_rows<T>(p, false, g->stream), "forward rows");
         if (int rc = plain_pencils<T>(g, w, CH_HPP, false)) return rc;
@@ -1175,7 +1175,7 @@ template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot
         p.mode = PLAIN_INVERSE;
         CK(launch_plain_n0<T>(p, g->stream), "inverse transform along n0");
         if (int rc = plain_pencils<T>(g, w, slot, true)) return rc;
-        p.out = out;
+        p.out[0] = out;
         CK(launch_plain_rows<T>(p, true, g->stream), "inverse rows");
         return OFDFT_OK;
     }
@@ -1197,31 +1197,37 @@ template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot
 // out = c0 base + c1 (IFFT(f FFT(u)) + v u), f the factor of `mode` (PLAIN_KINETIC, PLAIN_CN or
 // PLAIN_PRECOND with parameters p1, p2; f0 = f(G = 0), applied to what the forward rows subtract);
 // v, base may be null.
-// out is neither u nor base.
+// out is neither u nor base.  filter_plain_n: the same of one or two fields, whose spectra take the
+// slots CH_HPP and CH_VW.
 template <typename T>
-int filter_plain(ofdft_grid *g, Workspace<T> &w, const T *u, int mode, double p1, double p2, double f0, T *out,
-                 const T *v = nullptr, const T *base = nullptr, double c0 = 0.0, double c1 = 1.0) {
+int filter_plain_n(ofdft_grid *g, Workspace<T> &w, int nf, const T *const *u, int mode, double p1, double p2, double f0,
+                   T *const *out, const T *v = nullptr, const T *const *base = nullptr, double c0 = 0.0,
+                   double c1 = 1.0) {
     typedef typename Vec2<T>::type C;
     const long long N = g->N;
     cudaStream_t s = g->stream;
     int rc;
     if (w.plain_any) {
+        static_assert(CH_VW == CH_HPP + 1, "the pair's spectra");
         PlainArgs<T> p = plain_any_args<T>(w, g, CH_HPP);
-        p.u = u;
+        p.nf = nf;
+        for (int f = 0; f < nf; f++) p.u[f] = u[f];
         p.sampled = 1;
         CK(launch_plain_rows<T>(p, false, s), "forward rows");
-        if ((rc = plain_pencils<T>(g, w, CH_HPP, false))) return rc;
+        if ((rc = plain_pencils<T>(g, w, CH_HPP, false, nf))) return rc;
         p.mode = mode;
         p.p1 = (T)p1;
         p.p2 = (T)p2;
         p.scale = (T)(1.0 / (double)N);
         CK(launch_plain_n0<T>(p, s), "filter along n0");
-        if ((rc = plain_pencils<T>(g, w, CH_HPP, true))) return rc;
-        p.out = out;
+        if ((rc = plain_pencils<T>(g, w, CH_HPP, true, nf))) return rc;
+        for (int f = 0; f < nf; f++) {
+            p.out[f] = out[f];
+            p.vu[f] = u[f];
+            p.base[f] = base ? base[f] : nullptr;
+        }
         p.madd = (T)f0;
         p.v = v;
-        p.vu = u;
-        p.base = base;
         p.c0 = (T)c0;
         p.c1 = (T)c1;
         CK(launch_plain_rows<T>(p, true, s), "inverse rows");
@@ -1229,16 +1235,22 @@ int filter_plain(ofdft_grid *g, Workspace<T> &w, const T *u, int mode, double p1
     }
     double bv[9];
     for (int i = 0; i < 9; i++) bv[i] = 2.0 * kPi * g->recip[i];
-    if ((rc = forward_plain<T>(g, w, u))) return rc;
-    if (mode == PLAIN_PRECOND) CK(launch_precond<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, p1, p2, s), "factor");
-    else
-        CK(launch_spectral_factor<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, mode == PLAIN_CN, p1, p2, s), "factor");
-    if ((rc = inverse_plain<T>(g, w, CH_HPP, out, u))) return rc;
-    if (f0 != 0.0) CK(launch_add_scaled_scalar<T>(out, w.scal + S_RHO_MEAN, f0, N, s), "mean");
-    if (v) CK(launch_add_vu<T>(out, v, u, 1.0, 1.0, N, s), "potential");
-    if (base) CK(launch_axpby<T>(out, base, c0, c1, N, s), "axpby");
-    else if (c1 != 1.0) CK(launch_axpby<T>(out, out, c1, 0.0, N, s), "axpby");
+    for (int f = 0; f < nf; f++) {
+        if ((rc = forward_plain<T>(g, w, u[f]))) return rc;
+        if (mode == PLAIN_PRECOND) CK(launch_precond<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, p1, p2, s), "factor");
+        else
+            CK(launch_spectral_factor<C>((C *)w.chan, g->n[0], g->n[1], g->n[2], bv, mode == PLAIN_CN, p1, p2, s), "factor");
+        if ((rc = inverse_plain<T>(g, w, CH_HPP, out[f], u[f]))) return rc;
+        if (f0 != 0.0) CK(launch_add_scaled_scalar<T>(out[f], w.scal + S_RHO_MEAN, f0, N, s), "mean");
+        if (v) CK(launch_add_vu<T>(out[f], v, u[f], 1.0, 1.0, N, s), "potential");
+        if (base) CK(launch_axpby<T>(out[f], base[f], c0, c1, N, s), "axpby");
+        else if (c1 != 1.0) CK(launch_axpby<T>(out[f], out[f], c1, 0.0, N, s), "axpby");
+    }
     return OFDFT_OK;
+}
+template <typename T>
+int filter_plain(ofdft_grid *g, Workspace<T> &w, const T *u, int mode, double p1, double p2, double f0, T *out) {
+    return filter_plain_n<T>(g, w, 1, &u, mode, p1, p2, f0, &out);
 }
 
 template <typename T> int ensure_pme_buffers(ofdft_grid *g) {
@@ -1632,18 +1644,31 @@ template <typename T> struct Dev {
     Workspace<T> *w;
     cudaError_t err = cudaSuccess;
     double dot(const T *a, const T *b, const T *c = nullptr) {
-        if (err != cudaSuccess) return std::nan("");
-        cudaError_t e = launch_dot<T>(a, b, c, g->N, w->part_misc, 2 * stats_blocks(g), w->part_misc + 2048, w->ticket,
-                                      g->stream, g->exact_sums != 0);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(g->h_pinned + 40, w->part_misc + 2048, sizeof(double), cudaMemcpyDeviceToHost,
-                                g->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
-        if (e != cudaSuccess) {
-            err = e;
-            return std::nan("");
-        }
-        return g->h_pinned[40];
+        DotSet<T> d = {{a}, {b}, {c}};
+        double v;
+        dots(d, 1, &v);
+        return v;
+    }
+    // n <= 4 products in one launch and one wait
+    void dots(const DotSet<T> &d, int n, double *v) {
+        const int nblk = (n > 2 ? 1 : 2) * stats_blocks(g);
+        if (err == cudaSuccess)
+            err = launch_dots<T>(d, n, g->N, w->part_misc, nblk, w->part_misc + 2048, w->ticket, g->stream,
+                                 g->exact_sums != 0);
+        fetch(n, v);
+    }
+    void cg_step(const CgStep<T> &p, int n, double *v) {
+        if (err == cudaSuccess)
+            err = launch_cg_step<T>(p, n, g->N, w->part_misc, 2 * stats_blocks(g), w->part_misc + 2048, w->ticket, g->stream,
+                                    g->exact_sums != 0);
+        fetch(n, v);
+    }
+    void fetch(int n, double *v) {
+        if (err == cudaSuccess)
+            err = cudaMemcpyAsync(g->h_pinned + 40, w->part_misc + 2048, n * sizeof(double), cudaMemcpyDeviceToHost,
+                                  g->stream);
+        if (err == cudaSuccess) err = cudaStreamSynchronize(g->stream);
+        for (int k = 0; k < n; k++) v[k] = err == cudaSuccess ? g->h_pinned[40 + k] : std::nan("");
     }
     // OFDFT_OK, or the status of the first failed product (message kept in the handle)
     int status() const {
@@ -2053,7 +2078,7 @@ int optimize_impl(ofdft_grid *g, T *psi, const ofdft_functional *f0, double Ne, 
 // equations (1 + tau^2 H^2) x = (1 - i tau H)^2 psi(t): H is real, so the real and imaginary
 // parts are two real symmetric positive definite systems, solved together by preconditioned
 // CG with M = 1 / (1 + tau^2 (G^2/2 + vbar)^2) diagonal in G.
-constexpr int kTdFields = 19;
+constexpr int kTdFields = 18;
 
 template <typename T>
 int td_impl(ofdft_grid *g, T *pre, T *pim, const T *rho0, const ofdft_functional *f0, const ofdft_td_options &o,
@@ -2069,8 +2094,8 @@ int td_impl(ofdft_grid *g, T *pre, T *pim, const T *rho0, const ofdft_functional
     T *p0[2] = {F[0], F[1]};           // psi(t)
     T *c[2] = {F[2], F[3]};            // right-hand sides
     T *r[2] = {F[4], F[5]}, *z[2] = {F[6], F[7]}, *q[2] = {F[8], F[9]}, *Aq[2] = {F[10], F[11]};
-    T *h1 = F[12], *hp[2] = {F[13], F[14]};
-    T *vt = F[15], *vn = F[16], *vm = F[17], *rho = F[18];
+    T *hp[2] = {F[12], F[13]};         // H psi(t) of the right-hand sides, then H u inside apply_a
+    T *vt = F[14], *vn = F[15], *vm = F[16], *rho = F[17];
     T *x[2] = {pre, pim};
     Dev<T> dv{g, &w};
     cudaStream_t s = g->stream;
@@ -2098,17 +2123,18 @@ int td_impl(ofdft_grid *g, T *pre, T *pim, const T *rho0, const ofdft_functional
         evals++;
         return e;
     };
-    auto apply_h = [&](const T *u, const T *v, T *out) -> int {   // out = K u + v u
-        return filter_plain<T>(g, w, u, PLAIN_KINETIC, 0.0, 0.0, 0.0, out, v);
+    // the operators on the real and imaginary parts together (or on the n parts still iterated)
+    auto apply_h = [&](int n, const T *const *u, const T *v, T *const *out) -> int {   // out = K u + v u
+        return filter_plain_n<T>(g, w, n, u, PLAIN_KINETIC, 0.0, 0.0, 0.0, out, v);
     };
-    auto apply_a = [&](const T *u, const T *v, T *out) -> int {   // out = (1 + tau^2 H^2) u
-        if (int e = apply_h(u, v, h1)) return e;
-        return filter_plain<T>(g, w, h1, PLAIN_KINETIC, 0.0, 0.0, 0.0, out, v, u, 1.0, tau * tau);
+    auto apply_a = [&](int n, const T *const *u, const T *v, T *const *out) -> int {   // out = (1 + tau^2 H^2) u
+        if (int e = apply_h(n, u, v, hp)) return e;
+        return filter_plain_n<T>(g, w, n, hp, PLAIN_KINETIC, 0.0, 0.0, 0.0, out, v, u, 1.0, tau * tau);
     };
     double vbar = 0.0;
-    auto apply_m = [&](const T *u, T *out) -> int {              // out = M u
+    auto apply_m = [&](int n, const T *const *u, T *const *out) -> int {              // out = M u
         const double a0 = tau * vbar;
-        return filter_plain<T>(g, w, u, PLAIN_CN, tau, vbar, 1.0 / (1.0 + a0 * a0), out);
+        return filter_plain_n<T>(g, w, n, u, PLAIN_CN, tau, vbar, 1.0 / (1.0 + a0 * a0), out);
     };
     // x <- psi(t + dt) for the Hamiltonian with potential v, x holding the initial guess
     // (x_is_psi: the guess is psi(t) itself, whose residual follows from the right-hand side)
@@ -2116,69 +2142,94 @@ int td_impl(ofdft_grid *g, T *pre, T *pim, const T *rho0, const ofdft_functional
         int e;
         vbar = 0.0;
         if (have_v) {   // v weighted by the density held in rho (any vbar gives the same solution)
-            const double sr = dv.dot(x[0], x[0]) + dv.dot(x[1], x[1]);
-            if (sr > 0.0) vbar = dv.dot(rho, v) / sr;
+            const DotSet<T> d = {{x[0], x[1], rho}, {x[0], x[1], v}, {}};
+            double sv[3];
+            dv.dots(d, 3, sv);
+            if (sv[0] + sv[1] > 0.0) vbar = sv[2] / (sv[0] + sv[1]);
         }
         // c = (1 - i tau H)^2 psi(t):  c_re = p_re + 2 tau H p_im - tau^2 H^2 p_re,
         //                               c_im = p_im - 2 tau H p_re - tau^2 H^2 p_im
-        for (int j = 0; j < 2; j++)
-            if ((e = apply_h(p0[j], v, hp[j]))) return e;
-        for (int j = 0; j < 2; j++) {
-            if ((e = apply_h(hp[j], v, c[j]))) return e;
-            if (x_is_psi) {
-                // r = c - (1 + tau^2 H^2) psi = -2 tau^2 H^2 p_j +- 2 tau H p_(other)
-                CK(launch_copy<T>(r[j], c[j], N, s), "copy");
-                CK(launch_axpby<T>(r[j], hp[1 - j], j == 0 ? 2.0 * tau : -2.0 * tau, -2.0 * tau * tau, N, s), "axpby");
-            }
-            CK(launch_axpby<T>(c[j], p0[j], 1.0, -tau * tau, N, s), "axpby");
-            CK(launch_axpby<T>(c[j], hp[1 - j], j == 0 ? 2.0 * tau : -2.0 * tau, 1.0, N, s), "axpby");
-        }
-        double nc[2], rz[2];
+        // (x_is_psi: r = c - (1 + tau^2 H^2) psi = -2 tau^2 H^2 p_j +- 2 tau H p_(other))
+        if ((e = apply_h(2, p0, v, hp)) || (e = apply_h(2, hp, v, c))) return e;
+        CK(launch_td_rhs<T>(p0, hp, c, x_is_psi ? r : nullptr, tau, N, s), "right-hand sides");
+        double nc[2], rr[2], rz[2];
         bool done[2];
-        int its = 0;
-        for (int j = 0; j < 2; j++) {
-            nc[j] = std::sqrt(dv.dot(c[j], c[j]));
-            done[j] = !(nc[j] > 0.0);
-            if (done[j]) {
-                CK(cudaMemsetAsync(x[j], 0, (size_t)N * sizeof(T), s), "memset");
-                continue;
+        int its = 0, n = 0, part[2];       // the n parts still iterated
+        {
+            const DotSet<T> d = {{c[0], c[1], r[0], r[1]}, {c[0], c[1], r[0], r[1]}, {}};
+            double sv[4];
+            dv.dots(d, x_is_psi ? 4 : 2, sv);
+            for (int j = 0; j < 2; j++) {
+                nc[j] = std::sqrt(sv[j]);
+                if (x_is_psi) rr[j] = sv[2 + j];
+                done[j] = !(nc[j] > 0.0);
+                if (done[j]) CK(cudaMemsetAsync(x[j], 0, (size_t)N * sizeof(T), s), "memset");
+                else part[n++] = j;
             }
-            if (!x_is_psi) {
-                if ((e = apply_a(x[j], v, r[j]))) return e;
-                CK(launch_axpby<T>(r[j], c[j], 1.0, -1.0, N, s), "axpby");  // r = c - A x
+        }
+        // fields of the parts still iterated
+        auto of = [&](T *const *f, T **o) {
+            for (int k = 0; k < n; k++) o[k] = f[part[k]];
+        };
+        T *xs[2], *rs[2], *zs[2], *qs[2], *As[2];
+        auto drop = [&](auto gone) {       // the parts for which gone(k) leave the iteration
+            int m = 0;
+            for (int k = 0; k < n; k++) {
+                if (gone(k)) done[part[k]] = true;
+                else part[m++] = part[k];
             }
-            if (std::sqrt(dv.dot(r[j], r[j])) <= tol * nc[j]) {
-                done[j] = true;
-                continue;
-            }
-            if ((e = apply_m(r[j], z[j]))) return e;
-            CK(launch_copy<T>(q[j], z[j], N, s), "copy");
-            rz[j] = dv.dot(r[j], z[j]);
+            n = m;
+            of(x, xs), of(r, rs), of(z, zs), of(q, qs), of(Aq, As);
+        };
+        drop([&](int) { return false; });
+        auto products = [&](T *const *a, T *const *b, double *out) {
+            DotSet<T> d = {};
+            for (int k = 0; k < n; k++) d.a[k] = a[k], d.b[k] = b[k];
+            dv.dots(d, n, out);
+        };
+        double sv[2];
+        if (n > 0 && !x_is_psi) {
+            if ((e = apply_a(n, xs, v, rs))) return e;
+            for (int k = 0; k < n; k++) CK(launch_axpby<T>(rs[k], c[part[k]], 1.0, -1.0, N, s), "axpby");  // r = c - A x
+            products(rs, rs, sv);
+            for (int k = 0; k < n; k++) rr[part[k]] = sv[k];
+        }
+        drop([&](int k) { return std::sqrt(rr[part[k]]) <= tol * nc[part[k]]; });
+        if (n > 0) {
+            if ((e = apply_m(n, rs, qs))) return e;
+            products(rs, qs, sv);
+            for (int k = 0; k < n; k++) rz[part[k]] = sv[k];
         }
         double res = 0.0;
-        while (!(done[0] && done[1]) && its < max_it) {
+        while (n > 0 && its < max_it) {
             its++;
-            for (int j = 0; j < 2; j++) {
-                if (done[j]) continue;
-                if ((e = apply_a(q[j], v, Aq[j]))) return e;
-                const double qAq = dv.dot(q[j], Aq[j]);
-                if (!(qAq > 0.0)) {
-                    done[j] = true;
-                    continue;
-                }
-                const double a = rz[j] / qAq;
-                CK(launch_axpby<T>(x[j], q[j], a, 1.0, N, s), "axpby");
-                CK(launch_axpby<T>(r[j], Aq[j], -a, 1.0, N, s), "axpby");
-                const double rn = std::sqrt(dv.dot(r[j], r[j])) / nc[j];
-                if (rn <= tol) {
-                    done[j] = true;
-                    res = std::max(res, rn);
-                    continue;
-                }
-                if ((e = apply_m(r[j], z[j]))) return e;
-                const double rz_new = dv.dot(r[j], z[j]);
-                CK(launch_axpby<T>(q[j], z[j], 1.0, rz_new / rz[j], N, s), "axpby");
-                rz[j] = rz_new;
+            if ((e = apply_a(n, qs, v, As))) return e;
+            double qAq[2];
+            products(qs, As, qAq);
+            CgStep<T> st = {};
+            int m = 0;
+            double al[2];
+            for (int k = 0; k < n; k++)
+                if (qAq[k] > 0.0) al[m++] = rz[part[k]] / qAq[k];
+            drop([&](int k) { return !(qAq[k] > 0.0); });
+            if (n == 0) break;
+            for (int k = 0; k < n; k++) {
+                st.x[k] = xs[k], st.r[k] = rs[k], st.q[k] = qs[k], st.w[k] = As[k];
+                st.al[k] = (T)al[k];
+            }
+            double rn[2];
+            dv.cg_step(st, n, rn);
+            for (int k = 0; k < n; k++) {
+                rn[k] = std::sqrt(rn[k]) / nc[part[k]];
+                if (rn[k] <= tol) res = std::max(res, rn[k]);
+            }
+            drop([&](int k) { return rn[k] <= tol; });
+            if (n == 0) break;
+            if ((e = apply_m(n, rs, zs))) return e;
+            products(rs, zs, sv);
+            for (int k = 0; k < n; k++) {
+                CK(launch_axpby<T>(qs[k], zs[k], 1.0, sv[k] / rz[part[k]], N, s), "axpby");
+                rz[part[k]] = sv[k];
             }
         }
         if (!(done[0] && done[1])) {

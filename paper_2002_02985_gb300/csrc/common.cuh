@@ -108,9 +108,9 @@ __device__ __forceinline__ void pdl_begin() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
 }
 // launch of a kernel that starts with pdl_begin
-inline cudaError_t launch_pdl(const void *k, unsigned grid, unsigned block, void **args, size_t smem, cudaStream_t s) {
+inline cudaError_t launch_pdl(const void *k, dim3 grid, unsigned block, void **args, size_t smem, cudaStream_t s) {
     cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(grid);
+    c.gridDim = grid;
     c.blockDim = dim3(block);
     c.dynamicSmemBytes = smem;
     c.stream = s;

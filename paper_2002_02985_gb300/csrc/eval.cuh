@@ -33,7 +33,8 @@ enum {
     S_KF_WT = 6, S_TIMEOUT = 7,   // S_TIMEOUT: bounded waits that expired (the copies then landed)
     S_FATAL = 8,                  // waits whose copies did not land within the second bound either
     S_NSCAL = 9,
-    S_FIN = 16                 // [16, 21): the finalize blocks' five sums
+    S_FIN = 16,                // [16, 21): the finalize blocks' five sums
+    S_PAIR_MEAN = 40           // S_RHO_MEAN of a plain filter's second field
 };
 // energy slots: total, TF, vW, NL, H, PP, XC
 enum { E_TOT = 0, E_TF = 1, E_VW = 2, E_NL = 3, E_H = 4, E_PP = 5, E_XC = 6, E_NUM = 7 };

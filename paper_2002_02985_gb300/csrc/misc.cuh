@@ -58,6 +58,26 @@ cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, 
 template <typename T>
 cudaError_t launch_dot(const T *a, const T *b, const T *c, long long N, double *partials, int nblk,
                        double *out, unsigned *ticket, cudaStream_t s, bool exact = false);
+// up to four products at once (row of blocks y: product y), out and ticket one entry each
+template <typename T> struct DotSet {
+    const T *a[4], *b[4], *c[4];
+};
+template <typename T>
+cudaError_t launch_dots(const DotSet<T> &d, int n, long long N, double *partials, int nblk, double *out,
+                        unsigned *ticket, cudaStream_t s, bool exact = false);
+// x += al q, r -= al w, out = <r, r> of up to two solves
+template <typename T> struct CgStep {
+    T *x[2], *r[2];
+    const T *q[2], *w[2];
+    T al[2];
+};
+template <typename T>
+cudaError_t launch_cg_step(const CgStep<T> &p, int n, long long N, double *partials, int nblk, double *out,
+                           unsigned *ticket, cudaStream_t s, bool exact = false);
+// right-hand sides (and first residuals, r not null) of a Crank-Nicolson step's two systems
+template <typename T>
+cudaError_t launch_td_rhs(const T *const *p, const T *const *h, T *const *c, T *const *r, double tau, long long N,
+                          cudaStream_t s);
 // y = alpha * x + beta * y (scalars read from device double pointers when given)
 template <typename T>
 cudaError_t launch_axpby(T *y, const T *x, double alpha, double beta, long long N, cudaStream_t s);

@@ -637,11 +637,34 @@ template cudaError_t launch_axis0_fft<double>(double2 *, int, long long, const F
                                               double, cudaStream_t, int);
 
 // ---------------------------------------------------------------- optimiser vectors
+// Sums over one grid-wide launch: the last block of a row of blocks to finish adds the row's partials
+// in order (a launch of its own took 5 us of the 14 a product costs at 128^3).  Row blockIdx.y has its
+// own partials, result and ticket.
+__device__ __forceinline__ void finish_sum(double acc, double *part, double *out, unsigned *ticket, double *sd) {
+    __shared__ bool last;
+    part += (size_t)blockIdx.y * gridDim.x;
+    acc = block_sum(acc, sd);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = acc;
+        __threadfence();
+        last = atomicAdd(ticket + blockIdx.y, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    acc = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) acc += __ldcg(part + k);
+    acc = block_sum(acc, sd);
+    if (threadIdx.x == 0) {
+        out[blockIdx.y] = acc;
+        ticket[blockIdx.y] = 0u;
+    }
+}
 template <typename T>
-__global__ void __launch_bounds__(256) dot_kernel(const T *a, const T *b, const T *c, long long N, double *part,
+__global__ void __launch_bounds__(256) dot_kernel(const __grid_constant__ DotSet<T> d, long long N, double *part,
                                                   double *out, unsigned *ticket, bool exact) {
     __shared__ double sd[32];
-    __shared__ bool last;
+    const T *const a = d.a[blockIdx.y], *const b = d.b[blockIdx.y], *const c = d.c[blockIdx.y];
     double acc = 0.0;
     const long long stride = (long long)gridDim.x * blockDim.x;
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -664,30 +687,81 @@ __global__ void __launch_bounds__(256) dot_kernel(const T *a, const T *b, const 
             acc += v;
         }
     }
-    acc = block_sum(acc, sd);
-    // the last block to finish adds the blocks' partials in order (a launch of its own took 5 us of
-    // the 14 a product costs at 128^3)
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = acc;
-        __threadfence();
-        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    acc = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) acc += __ldcg(part + k);
-    acc = block_sum(acc, sd);
-    if (threadIdx.x == 0) {
-        *out = acc;
-        *ticket = 0u;
-    }
+    finish_sum(acc, part, out, ticket, sd);
 }
 
 template <typename T>
+cudaError_t launch_dots(const DotSet<T> &d, int n, long long N, double *partials, int nblk, double *out,
+                        unsigned *ticket, cudaStream_t s, bool exact) {
+    dot_kernel<T><<<dim3(nblk, n), 256, 0, s>>>(d, N, partials, out, ticket, exact);
+    return cudaGetLastError();
+}
+template <typename T>
 cudaError_t launch_dot(const T *a, const T *b, const T *c, long long N, double *partials, int nblk, double *out,
                        unsigned *ticket, cudaStream_t s, bool exact) {
-    dot_kernel<T><<<nblk, 256, 0, s>>>(a, b, c, N, partials, out, ticket, exact);
+    DotSet<T> d = {{a}, {b}, {c}};
+    return launch_dots<T>(d, 1, N, partials, nblk, out, ticket, s, exact);
+}
+
+// One step of up to two conjugate-gradient solves (row of blocks y: solve y): x += al q, r -= al w,
+// out = <r, r>.  One launch where the two updates and the product of each solve were three (2 x 25 us
+// at 128^3); sums grouped as in dot_kernel.
+template <typename T>
+__global__ void __launch_bounds__(256) cg_step_kernel(const __grid_constant__ CgStep<T> p, long long N, double *part,
+                                                      double *out, unsigned *ticket, bool exact) {
+    __shared__ double sd[32];
+    const int y = blockIdx.y;
+    T *const __restrict__ x = p.x[y], *const __restrict__ r = p.r[y];
+    const T *const __restrict__ q = p.q[y], *const __restrict__ w = p.w[y];
+    const T al = p.al[y];
+    double acc = 0.0;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    while (i < N) {
+        T g = 0;
+#pragma unroll
+        for (int u = 0; u < 8; u++, i += stride)
+            if (i < N) {
+                x[i] = al * q[i] + x[i];
+                const T v = -al * w[i] + r[i];
+                r[i] = v;
+                if (sizeof(T) == 8 || exact) acc += (double)(v * v);
+                else g += v * v;
+            }
+        acc += (double)g;
+    }
+    finish_sum(acc, part, out, ticket, sd);
+}
+template <typename T>
+cudaError_t launch_cg_step(const CgStep<T> &p, int n, long long N, double *partials, int nblk, double *out,
+                           unsigned *ticket, cudaStream_t s, bool exact) {
+    cg_step_kernel<T><<<dim3(nblk, n), 256, 0, s>>>(p, N, partials, out, ticket, exact);
+    return cudaGetLastError();
+}
+
+// c <- p - tau^2 c +- 2 tau hq (c holds H^2 p, hq = H of the other component; + for the real part) and,
+// where r is not null, r <- -2 tau^2 H^2 p +- 2 tau hq; both components in one pass
+template <typename T>
+__global__ void __launch_bounds__(256) td_rhs_kernel(const T *__restrict__ p0, const T *__restrict__ p1,
+                                                     const T *__restrict__ h0, const T *__restrict__ h1, T *__restrict__ c0,
+                                                     T *__restrict__ c1, T *__restrict__ r0, T *__restrict__ r1, T t2, T tt,
+                                                     long long N) {
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += stride) {
+        const T a = c0[i], b = c1[i], ha = h0[i], hb = h1[i];
+        c0[i] = t2 * hb + (p0[i] - tt * a);
+        c1[i] = -t2 * ha + (p1[i] - tt * b);
+        if (r0) {
+            r0[i] = t2 * hb + (T)-2 * tt * a;
+            r1[i] = -t2 * ha + (T)-2 * tt * b;
+        }
+    }
+}
+template <typename T>
+cudaError_t launch_td_rhs(const T *const *p, const T *const *h, T *const *c, T *const *r, double tau, long long N,
+                          cudaStream_t s) {
+    td_rhs_kernel<T><<<1216, 256, 0, s>>>(p[0], p[1], h[0], h[1], c[0], c[1], r ? r[0] : nullptr, r ? r[1] : nullptr,
+                                         (T)(2.0 * tau), (T)(tau * tau), N);
     return cudaGetLastError();
 }
 
@@ -1068,6 +1142,15 @@ cudaError_t launch_dipole(const T *re, const T *im, const T *rho0, int n0, int n
     return cudaGetLastError();
 }
 
+#define INST_TD(T)                                                                                             \
+    template cudaError_t launch_dots<T>(const DotSet<T> &, int, long long, double *, int, double *, unsigned *, \
+                                        cudaStream_t, bool);                                                    \
+    template cudaError_t launch_cg_step<T>(const CgStep<T> &, int, long long, double *, int, double *, unsigned *, \
+                                           cudaStream_t, bool);                                                 \
+    template cudaError_t launch_td_rhs<T>(const T *const *, const T *const *, T *const *, T *const *, double, long long, \
+                                          cudaStream_t);
+INST_TD(float)
+INST_TD(double)
 #define INST(T)                                                                                              \
     template cudaError_t launch_add_vu<T>(T *, const T *, const T *, double, double, long long, cudaStream_t); \
     template cudaError_t launch_abs2<T>(T *, const T *, const T *, long long, cudaStream_t);                 \

@@ -7,6 +7,8 @@
 // (the chain it replaces -- stats, per-channel rows, n0 transform, factor kernel, n0 transform,
 // rows, potential kernel -- took 133 us at 128^3, most of it in launches of 8 to 35 us that move
 // 17 MB each)
+// One field's launches fill less than a wave (512 blocks at 128^3, and four to eight fit an SM), so
+// two fields that take the same filter share each launch (blockIdx.y is the field).
 #include "any.cuh"
 #include "plain.cuh"
 
@@ -92,7 +94,9 @@ template <typename T> __device__ __forceinline__ typename Vec2<T>::type *plain_p
 // same order, so the same value) instead of waiting for a pass over the whole field; block 0
 // leaves it for the inverse rows.
 template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<T> &a) {
+    const int f = blockIdx.y;
     if (!a.sampled) return (T)a.scal[S_RHO_MEAN];
+    const T *const u = a.u[f];
     __shared__ T ws[kPlainThreads / 32];
     const long long N = (long long)a.n0 * a.n1 * a.n2, step = N / 1024 > 0 ? N / 1024 : 1;
     T s = 0;
@@ -100,7 +104,7 @@ template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<
     for (int k = 0; k < 1024 / kPlainThreads; k++) {
         long long i = (threadIdx.x + k * kPlainThreads) * step;
         if (i >= N) i %= N;                                   // (fields of fewer than 1024 points)
-        s += a.u[i];
+        s += u[i];
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -110,7 +114,7 @@ template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<
 #pragma unroll
     for (int k = 0; k < kPlainThreads / 32; k++) s += ws[k];
     s *= (T)(1.0 / 1024.0);
-    if (blockIdx.x == 0 && threadIdx.x == 0) const_cast<double *>(a.scal)[S_RHO_MEAN] = (double)s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) const_cast<double *>(a.scal)[f ? S_PAIR_MEAN : S_RHO_MEAN] = (double)s;
     return s;
 }
 template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_rows_fwd(const __grid_constant__ PlainArgs<T> a) {
@@ -121,6 +125,8 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
     C *const buf = (C *)smem_raw, *const scr = buf + n * ld;
     const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1);
     const T mean = plain_offset(a);
+    const T *const u = a.u[blockIdx.y];
+    C *const h = a.h + blockIdx.y * a.hs;
     if (a.vec) {
         // four consecutive points of a row per thread and step, several steps in flight
         const int n4 = n >> 2;
@@ -128,14 +134,14 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
         for (int idx = threadIdx.x; idx < (n4 << (lg + 1)); idx += kPlainThreads) {
             const int rr = (int)__umulhi((unsigned)idx, a.magic_n4), e = 4 * (idx - rr * n4);
             T x[4] = {mean, mean, mean, mean};
-            if (row0 + rr < R) load4(a.u + (size_t)(row0 + rr) * n + e, x);
+            if (row0 + rr < R) load4(u + (size_t)(row0 + rr) * n + e, x);
 #pragma unroll
             for (int q = 0; q < 4; q++) ((T *)(buf + (e + q) * ld + (rr >> 1)))[rr & 1] = x[q] - mean;
         }
     } else {
         for (int idx = threadIdx.x; idx < (n << (lg + 1)); idx += kPlainThreads) {
             const int rr = (int)__umulhi((unsigned)idx, a.magic_n), e = idx - rr * n;
-            const T x = row0 + rr < R ? a.u[(size_t)(row0 + rr) * n + e] - mean : (T)0;
+            const T x = row0 + rr < R ? u[(size_t)(row0 + rr) * n + e] - mean : (T)0;
             ((T *)(buf + e * ld + (rr >> 1)))[rr & 1] = x;
         }
     }
@@ -145,7 +151,7 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
         const int b = (int)__umulhi((unsigned)idx, a.magic_n2h), k = idx - b * n2h;
         const C A = Z[k * ld + b], Bv = Z[(k ? n - k : 0) * ld + b];
         const int r0 = row0 + 2 * b;
-        C *out = a.h + (size_t)r0 * n2h + k;
+        C *out = h + (size_t)r0 * n2h + k;
         if (r0 < R) out[0] = cmake<C>((T)0.5 * (A.x + Bv.x), (T)0.5 * (A.y - Bv.y));
         if (r0 + 1 < R) out[n2h] = cmake<C>((T)0.5 * (A.y + Bv.y), (T)0.5 * (Bv.x - A.x));
     }
@@ -159,13 +165,14 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = a.n2, n2h = a.n2h, lg = a.lgB, ld = (1 << lg) + 1;
     C *const buf = (C *)smem_raw, *const scr = buf + n * ld;
-    const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1);
+    const int R = a.n0 * a.n1, row0 = blockIdx.x << (lg + 1), f = blockIdx.y;
+    const C *const h = a.h + f * a.hs;
 #pragma unroll 4
     for (int idx = threadIdx.x; idx < n2h << lg; idx += kPlainThreads) {
         const int b = (int)__umulhi((unsigned)idx, a.magic_n2h), k = idx - b * n2h;
         const int r0 = row0 + 2 * b;
         const C zero = cmake<C>((T)0, (T)0);
-        const C *in = a.h + (size_t)r0 * n2h + k;
+        const C *in = h + (size_t)r0 * n2h + k;
         const C X0 = r0 < R ? in[0] : zero, X1 = r0 + 1 < R ? in[n2h] : zero;
         if (k == 0 || 2 * k == n) {
             buf[k * ld + b] = cmake<C>(X0.x, X1.x);
@@ -176,11 +183,11 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
     }
     __syncthreads();
     const C *Z = plain_passes<T>(a, +1, buf, scr);
-    const T shift = a.madd != (T)0 ? a.madd * (T)a.scal[S_RHO_MEAN] : (T)0;
+    const T shift = a.madd != (T)0 ? a.madd * (T)a.scal[f ? S_PAIR_MEAN : S_RHO_MEAN] : (T)0;
     if (a.vec) {
         const int n4 = n >> 2;
-        const T *const __restrict__ pv = a.v, *const __restrict__ pu = a.vu, *const __restrict__ pb = a.base;
-        T *const __restrict__ po = a.out;
+        const T *const __restrict__ pv = a.v, *const __restrict__ pu = a.vu[f], *const __restrict__ pb = a.base[f];
+        T *const __restrict__ po = a.out[f];
 #pragma unroll 4
         for (int idx = threadIdx.x; idx < (n4 << (lg + 1)); idx += kPlainThreads) {
             const int rr = (int)__umulhi((unsigned)idx, a.magic_n4), e = 4 * (idx - rr * n4);
@@ -207,8 +214,8 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
         if (row0 + rr >= R) break;
         const size_t i = (size_t)(row0 + rr) * n + e;
         T y = ((const T *)(Z + e * ld + (rr >> 1)))[rr & 1] + shift;
-        if (a.v) y += a.v[i] * a.vu[i];
-        a.out[i] = a.base ? a.c0 * a.base[i] + a.c1 * y : a.c1 * y;
+        if (a.v) y += a.v[i] * a.vu[f][i];
+        a.out[f][i] = a.base[f] ? a.c0 * a.base[f][i] + a.c1 * y : a.c1 * y;
     }
 }
 
@@ -230,7 +237,7 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
     C *X = (C *)smem_raw, *Y = X + (n << lg);
     const int w = threadIdx.x & (TW - 1), col = (blockIdx.x << lg) + w;
     const bool ok = col < PL;
-    const AnyGlobal<C> G{a.h + (ok ? col : 0), PL, ok};
+    const AnyGlobal<C> G{a.h + blockIdx.y * a.hs + (ok ? col : 0), PL, ok};
     auto dec = [&](int idx, int &b, int &j) {
         b = w;
         j = idx >> lg;
@@ -322,20 +329,24 @@ cudaError_t launch_plain_mean(const T *u, long long N, int nblk, double *part, d
 template <typename T> cudaError_t launch_plain_rows(const PlainArgs<T> &a_in, bool inverse, cudaStream_t s) {
     // 16-byte (FP32) accesses where every row of every field starts on such a boundary
     PlainArgs<T> a = a_in;
-    const uintptr_t at = (uintptr_t)a.u | (uintptr_t)a.out | (uintptr_t)a.v | (uintptr_t)a.vu | (uintptr_t)a.base;
+    uintptr_t at = (uintptr_t)a.v;
+    for (int f = 0; f < 2; f++)
+        at |= (uintptr_t)a.u[f] | (uintptr_t)a.out[f] | (uintptr_t)a.vu[f] | (uintptr_t)a.base[f];
     a.vec = a.n2 % 4 == 0 && a.n2 >= 8 && at % 16 == 0;
     const long long R = (long long)a.n0 * a.n1;
     const unsigned nb = (unsigned)((R + (2 << a.lgB) - 1) >> (a.lgB + 1));
     const size_t sm = 2 * 2 * sizeof(T) * (size_t)a.n2 * ((1 << a.lgB) + 1);
     void *args[] = {(void *)&a};
-    return launch_pdl(inverse ? (const void *)plain_rows_inv<T> : (const void *)plain_rows_fwd<T>, nb, kPlainThreads, args,
+    return launch_pdl(inverse ? (const void *)plain_rows_inv<T> : (const void *)plain_rows_fwd<T>,
+                      dim3(nb, a.nf > 1 ? 2 : 1), kPlainThreads, args,
                       sm, s);
 }
 template <typename T> cudaError_t launch_plain_n0(const PlainArgs<T> &a, cudaStream_t s) {
     const long long PL = (long long)a.n1 * a.n2h;
     const unsigned nb = (unsigned)((PL + (1 << a.lg0) - 1) >> a.lg0);
     void *args[] = {(void *)&a};
-    return launch_pdl((const void *)plain_n0<T>, nb, kPlainThreads, args, 2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s);
+    return launch_pdl((const void *)plain_n0<T>, dim3(nb, a.nf > 1 ? 2 : 1), kPlainThreads, args,
+                      2 * 2 * sizeof(T) * ((size_t)a.n0 << a.lg0), s);
 }
 #define INST(T)                                                                                                     \
     template bool plain_setup<T>(PlainArgs<T> &, int);                                                              \

@@ -16,13 +16,15 @@ template <typename T> struct PlainArgs {
     int lgB, lg0, mode;
     unsigned magic_n, magic_n2h, magic_n4;
     int vec;                     // set at the launch: four points per access
-    C *h;                        // half spectrum
+    int nf;                      // fields of the launch, one per blockIdx.y (0 counts as 1)
+    C *h;                        // half spectra, hs apart
+    long long hs;
     const C *tw0, *tw2;
     const double *scal;          // S_RHO_MEAN: the constant the forward rows subtract
     int sampled;                 // they take it from a sample of the field (and leave it there)
-    const T *u;                  // input field
-    T *out;
-    const T *v, *vu, *base;      // epilogue out = c0 base + c1 (y + madd mean + v vu)
+    const T *u[2];               // input fields
+    T *out[2];
+    const T *v, *vu[2], *base[2];   // epilogue out = c0 base + c1 (y + madd mean + v vu)
     T c0, c1, madd;
     T p1, p2, scale;
     T b[9];                      // 2 pi times the reciprocal vectors
