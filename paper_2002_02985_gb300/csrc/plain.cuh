@@ -1,4 +1,4 @@
-// Plain one-field transforms (plain.cu).
+// Plain transforms of one or two real fields (plain.cu).
 #pragma once
 
 #include "eval.cuh"
