@@ -133,8 +133,9 @@ template <typename T> void any_candidates(int role, int n, long long cols, int n
         AnyCt ct;
         if (sizeof(T) == 4 && (any_ct_rows_1(n, ct) || any_ct_rows_2(n, ct) || any_ct_rows_3(n, ct) || any_ct_rows_4(n, ct)))
             c.any = 2;
-        // the channel group fills half or a third of an SM's shared memory per block
-        for (int kb : {40, 76}) {
+        // the channel group fills a fifth, a quarter or a third of an SM's shared memory per block (512
+        // points: nine channels leave room for two blocks, seven for the three that the threads allow)
+        for (int kb : {40, 60, 76}) {
             const int G = std::min(34, (int)(kb * 1024 / (2 * (size_t)(n + 2) * 2 * sizeof(T))));
             if (G < 1 || G == last) continue;
             last = G;

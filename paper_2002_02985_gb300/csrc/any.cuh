@@ -604,8 +604,16 @@ template <typename T, int E__, bool INV, int R1 = 0, int R2 = 1, int R3 = 1> str
 // registers, 70 us with 160 and 72).  Longer rows keep two elements per thread, which spares the idle
 // threads of small channel groups (256^3, forward / inverse: 613 / 870 us against 648 / 900 us).
 constexpr int any_ct_E(int n) { return n <= 200 ? 1 : 2; }
-constexpr int any_ct_row_threads(int n) { return n <= 160 ? 160 : (n <= 200 ? 256 : 320); }
-constexpr int any_ct_row_blocks(int n) { return n <= 160 ? 5 : (n <= 200 ? 3 : 2); }
+// Beyond 256 points a block has one thread per two points and at least six warps, and 24 warps share an
+// SM at 80 registers (320 threads at two blocks per SM: whole evaluations of 256 x 256 x 320 and
+// 256 x 256 x 512 5.00 and 7.77 ms, now 4.60 and 7.22; 512^3 with 15 channels 28.99 -> 27.70 ms); 129 to 160 points take 192 threads, so that all
+// channels of an ordinary call go in one group (144^3: 0.690 -> 0.670 ms).
+constexpr int any_ct_row_threads(int n) {
+    return n <= 128 ? 160 : (n <= 160 ? 192 : (n <= 200 ? 256 : (n <= 256 ? 320 : (n <= 384 ? 192 : ((n + 63) / 64 * 32)))));
+}
+constexpr int any_ct_row_blocks(int n) {
+    return n <= 128 ? 5 : (n <= 160 ? 4 : (n <= 200 ? 3 : (n <= 256 ? 2 : 768 / any_ct_row_threads(n))));
+}
 template <typename T, int E>
 __global__ void __launch_bounds__(RowAny<T, E, false>::NT_, sizeof(T) == 4 ? 2 : 1)
     row_fwd_any_kernel(const __grid_constant__ EvalArgs<T> a, const EvalArgs<T> *__restrict__ ga, int bps) {
