@@ -141,7 +141,7 @@ struct ofdft_grid {
     long long vf_len = 0;
     bool vf_fresh = false;
     int *d_sp_ions = nullptr;    // the ions grouped by species (device), the groups' offsets (host)
-    std::vector<int> sp_off;
+    std::vector<int> sp_ions, sp_off;
     // smooth PME (ofdft_set_ions_pme): order > 0 selects it for V_ext(G) and forces
     int pme_order = 0;
     double2 *pmeB = nullptr;               // conj b_a tables [n0 | n1 | n2h]
@@ -218,6 +218,13 @@ template <typename P> cudaError_t gmalloc(ofdft_grid *g, P **p, size_t bytes) {
     const cudaError_t e = cudaMalloc((void **)p, bytes);
     if (e == cudaSuccess) g->alloc_bytes += bytes;
     return e;
+}
+
+// Host arrays go up on the grid's own stream: a copy from pageable memory on the legacy stream may
+// still be under way when the call returns, and a non-blocking stream does not wait for it.  src
+// stays as it is until the stream has been waited for.
+template <typename P> cudaError_t upload(ofdft_grid *g, P *dst, const P *src, size_t n) {
+    return cudaMemcpyAsync(dst, src, n * sizeof(P), cudaMemcpyHostToDevice, g->stream);
 }
 
 template <typename T> Workspace<T> &ws(ofdft_grid *g);
@@ -466,19 +473,21 @@ template <typename T> int ensure_ws(ofdft_grid *g, int nslots) {
     if (!w.ready) {
         int rc = choose_launch<T>(g, w);
         if (rc) return rc;
+        std::vector<C> tw[3];
         for (int a = 0; a < 3; a++) {
             const int n = g->n[a];
-            std::vector<C> h(n);
+            std::vector<C> &h = tw[a];
+            h.resize(n);
             for (int k = 0; k < n; k++) {
                 const double ang = -2.0 * kPi * (double)k / (double)n;
                 h[k].x = (T)std::cos(ang);
                 h[k].y = (T)std::sin(ang);
             }
             CK(gmalloc(g, &w.tw[a], n * sizeof(C)), "cudaMalloc twiddles");
-            CK(cudaMemcpy(w.tw[a], h.data(), n * sizeof(C), cudaMemcpyHostToDevice), "upload twiddles");
+            CK(upload(g, w.tw[a], h.data(), n), "upload twiddles");
         }
         CK(gmalloc(g, &w.scal, 64 * sizeof(double)), "cudaMalloc scalars");
-        CK(cudaMemset(w.scal, 0, 64 * sizeof(double)), "memset");
+        CK(cudaMemsetAsync(w.scal, 0, 64 * sizeof(double), g->stream), "memset");
         w.energies = w.scal + kEnergySlot;
         CK(gmalloc(g, &w.knots_d, OFDFT_MAX_KNOTS * sizeof(double)), "cudaMalloc knots");
         CK(gmalloc(g, &w.knots_t, OFDFT_MAX_KNOTS * sizeof(T)), "cudaMalloc knots");
@@ -490,8 +499,8 @@ template <typename T> int ensure_ws(ofdft_grid *g, int nslots) {
         CK(gmalloc(g, &w.part_row, (size_t)w.nb_row * sizeof(double)), "cudaMalloc partials");
         CK(gmalloc(g, &w.part_misc, 4096 * sizeof(double)), "cudaMalloc partials");
         CK(gmalloc(g, &w.ticket, 4 * sizeof(unsigned)), "cudaMalloc ticket");
-        CK(cudaMemset(w.ticket, 0, 4 * sizeof(unsigned)), "memset ticket");
-
+        CK(cudaMemsetAsync(w.ticket, 0, 4 * sizeof(unsigned), g->stream), "memset ticket");
+        CK(cudaStreamSynchronize(g->stream), "stream synchronize");   // (the host tables end here)
         w.ready = true;
     }
     if (nslots > w.nslots) {
@@ -2462,8 +2471,8 @@ int make_plan(ofdft_grid *g0, int n, ofdft_grid *const *grids, const std::vector
     CK(cudaMalloc(&p.dargs, (size_t)n * sizeof(EvalArgs<T>)), "cudaMalloc batch arguments");
     CK(cudaMalloc((void **)&p.dcol, (size_t)n * W * sizeof(double)), "cudaMalloc batch results");
     CK(cudaMallocHost((void **)&p.hcol, (size_t)n * W * sizeof(double)), "cudaMallocHost batch results");
-    CK(cudaMemcpy(p.dargs, ordered.data(), (size_t)n * sizeof(EvalArgs<T>), cudaMemcpyHostToDevice),
-       "upload batch arguments");
+    CK(upload(g, (EvalArgs<T> *)p.dargs, ordered.data(), n), "upload batch arguments");
+    CK(cudaStreamSynchronize(g->stream), "stream synchronize");
     return OFDFT_OK;
 }
 
@@ -2999,12 +3008,14 @@ int store_ions(ofdft_grid *g, const ofdft_ions *ions, const ofdft_species *sp) {
     for (int i = 0; i < n; i++) g->species_count[g->species[i]]++;
     g->sp_off.assign(sp->n_species + 1, 0);
     for (int s = 0; s < sp->n_species; s++) g->sp_off[s + 1] = g->sp_off[s] + g->species_count[s];
-    std::vector<int> lists(n), fill(g->sp_off.begin(), g->sp_off.end() - 1);
-    for (int i = 0; i < n; i++) lists[fill[g->species[i]]++] = i;
-    CK(cudaMemcpy(g->d_species, g->species.data(), n * sizeof(int), cudaMemcpyHostToDevice), "upload species");
-    CK(cudaMemcpy(g->d_sp_ions, lists.data(), n * sizeof(int), cudaMemcpyHostToDevice), "upload species lists");
-    CK(cudaMemcpy(g->d_Z, g->Z.data(), g->n_species * sizeof(double), cudaMemcpyHostToDevice), "upload Z");
-    CK(cudaMemcpy(g->d_rc, g->rc.data(), g->n_species * sizeof(double), cudaMemcpyHostToDevice), "upload rc");
+    std::vector<int> fill(g->sp_off.begin(), g->sp_off.end() - 1);
+    g->sp_ions.resize(n);
+    for (int i = 0; i < n; i++) g->sp_ions[fill[g->species[i]]++] = i;
+    // (the handle's own arrays: they change only after the wait above)
+    CK(upload(g, g->d_species, g->species.data(), n), "upload species");
+    CK(upload(g, g->d_sp_ions, g->sp_ions.data(), n), "upload species lists");
+    CK(upload(g, g->d_Z, g->Z.data(), g->n_species), "upload Z");
+    CK(upload(g, g->d_rc, g->rc.data(), g->n_species), "upload rc");
     g->have_ions = true;
     g->vext_fresh32 = g->vext_fresh64 = false;
     return OFDFT_OK;
@@ -3026,7 +3037,7 @@ int ofdft_set_ions(ofdft_grid *g, const ofdft_ions *ions, const ofdft_species *s
     }
     // per-axis phase tables e^{-2 pi i m_a f_a}, f = R . inv(cell) (fractional)
     if (!g->d_pos) CK(gmalloc(g, &g->d_pos, 3 * (size_t)n * sizeof(double)), "cudaMalloc positions");
-    CK(cudaMemcpy(g->d_pos, g->pos.data(), 3 * (size_t)n * sizeof(double), cudaMemcpyHostToDevice), "upload positions");
+    CK(upload(g, g->d_pos, g->pos.data(), 3 * (size_t)n), "upload positions");
     CK(launch_phases(g->n, g->n2h, n, g->recip, g->d_pos, g->ph, g->ph32, g->stream), "phase tables");
     return OFDFT_OK;
 }
@@ -3040,8 +3051,7 @@ int ofdft_set_ions_pme(ofdft_grid *g, const ofdft_ions *ions, const ofdft_specie
     if (rc) return rc;
     g->pme_order = order;
     if (!g->d_pos) CK(gmalloc(g, &g->d_pos, (size_t)3 * g->n_ions * sizeof(double)), "cudaMalloc positions");
-    CK(cudaMemcpy(g->d_pos, g->pos.data(), (size_t)3 * g->n_ions * sizeof(double), cudaMemcpyHostToDevice),
-       "upload positions");
+    CK(upload(g, g->d_pos, g->pos.data(), 3 * (size_t)g->n_ions), "upload positions");
     // conj b_a(k) = conj( e^{2 pi i (p-1) k/n} / sum_{j=0}^{p-2} M_p(j+1) e^{2 pi i k j/n} )
     std::vector<double> Mp(order + 1, 0.0);   // M_p at the integers 1..p-1
     {
@@ -3076,7 +3086,8 @@ int ofdft_set_ions_pme(ofdft_grid *g, const ofdft_ions *ions, const ofdft_specie
         off += na[ax];
     }
     if (!g->pmeB) CK(gmalloc(g, &g->pmeB, B.size() * sizeof(double2)), "cudaMalloc PME factors");
-    CK(cudaMemcpy(g->pmeB, B.data(), B.size() * sizeof(double2), cudaMemcpyHostToDevice), "upload PME factors");
+    CK(upload(g, g->pmeB, B.data(), B.size()), "upload PME factors");
+    CK(cudaStreamSynchronize(g->stream), "stream synchronize");
     return OFDFT_OK;
 }
 

@@ -1,0 +1,95 @@
+"""Host logic of the library on a machine without a GPU: its objects linked against a stand-in for
+the CUDA runtime (host_cuda.cpp) that keeps device memory on the host, runs no kernel and logs every
+copy, memset, launch and wait."""
+import ctypes as ct
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+from paper_2002_02985_gb300 import _lib as L
+from paper_2002_02985_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+STREAM = 0x5000                                # a stream of the caller's that is not the legacy one
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    B.build()
+    out = str(tmp_path_factory.mktemp("host") / "libofdft_host.so")
+    objs = [os.path.join(B.BUILD, s.replace(".cu", ".o")) for s in B.sources()]
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", inc, "-o", out,
+                    os.path.join(HERE, "host_cuda.cpp"), *objs, "-lpthread"], check=True)
+    saved, L._lib = L._lib, None
+    try:
+        lib = L.load(out)
+    finally:
+        L._lib = saved
+    lib.host_cuda_log.restype = ct.c_char_p
+    lib.host_cuda_cost.argtypes = [ct.c_char_p, ct.c_double]
+    return lib
+
+
+class Grid:
+    """A grid of the library on the stand-in runtime, with host arrays in the place of device ones."""
+
+    def __init__(self, lib, shape, side=8.0, stream=STREAM):
+        self.lib, self.shape = lib, shape
+        self.h = ct.c_void_p()
+        cell = (ct.c_double * 9)(*np.diag([side] * 3).ravel())
+        assert lib.ofdft_grid_create(cell, (ct.c_int * 3)(*shape), ct.c_void_p(stream), ct.byref(self.h)) == 0
+
+    def close(self):
+        self.lib.ofdft_grid_destroy(self.h)
+
+    def set_ions(self, n_species=1, pme=0):
+        n = max(4, n_species)
+        pos, sp = np.random.default_rng(n).uniform(0.0, 8.0, (n, 3)), np.arange(n, dtype=np.int32) % n_species
+        Z, rc = 1.0 + np.arange(n_species), 0.7 + 0.1 * np.arange(n_species)
+        ptr = lambda a, t: a.ctypes.data_as(ct.POINTER(t))
+        ions = L.CIons(n, ptr(pos, ct.c_double), ptr(sp, ct.c_int))
+        spec = L.CSpecies(n_species, ptr(Z, ct.c_double), ptr(rc, ct.c_double))
+        call = (ct.byref(ions), ct.byref(spec)) + ((pme,) if pme else ())
+        return (self.lib.ofdft_set_ions_pme if pme else self.lib.ofdft_set_ions)(self.h, *call)
+
+    def functional(self, precision=L.FP32_MIXED, knots=6, terms=L.TERMS_ALL):
+        return L.CFunctional(terms, 5.0 / 6.0, 5.0 / 6.0, knots, L.KNOTS_LOG, None, L.NLPOT_EXACT, L.KERNEL_LWT,
+                             precision, 0.0, 0.0, 0.0)
+
+    def density(self, precision=L.FP32_MIXED):
+        self.rho = np.full(self.shape, 0.01, np.float64 if precision == L.FP64 else np.float32)
+        return ct.c_void_p(self.rho.ctypes.data)
+
+    def evaluate(self, precision=L.FP32_MIXED, **kw):
+        E = (ct.c_double * L.N_ENERGIES)()
+        f = self.functional(precision, **kw)
+        return self.lib.ofdft_energy_potential(self.h, self.density(precision), ct.byref(f), E, None)
+
+
+def log(lib):
+    return [x.split() for x in lib.host_cuda_log().decode().splitlines()]
+
+
+def test_host_data_reaches_the_device_on_the_grids_stream(lib):
+    """Uploads and clears that kernels of the grid's stream read are made on that stream: a copy from
+    pageable memory (or a memset) on the legacy stream may still be under way when the call returns,
+    and a non-blocking stream does not wait for it."""
+    lib.host_cuda_reset()
+    a, b = Grid(lib, (24, 20, 18)), Grid(lib, (24, 20, 18))
+    for g in (a, b):
+        assert g.set_ions(2) == 0
+        for p in (L.FP32_MIXED, L.FP64):
+            assert g.evaluate(p) == 0
+    hs, f = (ct.c_void_p * 2)(a.h, b.h), a.functional()
+    rho = (ct.c_void_p * 2)(a.density(), b.density())
+    E = (ct.c_double * (2 * L.N_ENERGIES))()
+    assert lib.ofdft_energy_potential_batched(2, hs, rho, ct.byref(f), E, None, None) == 0
+    assert a.set_ions(1, pme=6) == 0 and a.evaluate() == 0
+    ops = log(lib)
+    assert [x for x in ops if x[0] in ("memcpy", "memset") and x[1] != "d2h"] == []
+    up = [x for x in ops if x[0] == "memcpyAsync" and x[1] == "h2d"]
+    assert up and {x[2] for x in up} == {"%x" % STREAM}
+    a.close(), b.close()
