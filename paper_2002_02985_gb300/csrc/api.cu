@@ -140,7 +140,8 @@ struct ofdft_grid {
     double *vf = nullptr;        // per-species v_s(|G|) / Omega in FP64 for the FP32 V_ext(G)
     long long vf_len = 0;
     bool vf_fresh = false;
-    int *d_sp_ions = nullptr;    // the ions grouped by species (device), the groups' offsets (host)
+    // the ions grouped by species, then the groups' offsets (device); both, the offsets alone (host)
+    int *d_sp_ions = nullptr;
     std::vector<int> sp_ions, sp_off;
     // smooth PME (ofdft_set_ions_pme): order > 0 selects it for V_ext(G) and forces
     int pme_order = 0;
@@ -589,7 +590,7 @@ template <typename T> int ensure_vext(ofdft_grid *g) {
             if (!g->vf_fresh) CK(launch_form_tables(a, g->vf, g->stream), "form factors");
             g->vf_fresh = true;
         }
-        e = launch_vext(a, nullptr, (float2 *)w.vext, g->stream, g->ph32, g->d_sp_ions, g->sp_off.data(),
+        e = launch_vext(a, nullptr, (float2 *)w.vext, g->stream, g->ph32, g->d_sp_ions, g->d_sp_ions + g->n_ions,
                         len <= kFormTableMax ? g->vf : nullptr);
     }
     else e = launch_vext(a, (double2 *)w.vext, nullptr, g->stream);
@@ -2990,7 +2991,7 @@ int store_ions(ofdft_grid *g, const ofdft_ions *ions, const ofdft_species *sp) {
         g->d_sp_ions = nullptr;
         g->d_Z = g->d_rc = nullptr;
         CK(gmalloc(g, &g->d_species, n * sizeof(int)), "cudaMalloc species");
-        CK(gmalloc(g, &g->d_sp_ions, n * sizeof(int)), "cudaMalloc species lists");
+        CK(gmalloc(g, &g->d_sp_ions, ((size_t)n + sp->n_species + 1) * sizeof(int)), "cudaMalloc species lists");
         CK(gmalloc(g, &g->d_Z, sp->n_species * sizeof(double)), "cudaMalloc Z");
         CK(gmalloc(g, &g->d_rc, sp->n_species * sizeof(double)), "cudaMalloc rc");
     }
@@ -3011,9 +3012,10 @@ int store_ions(ofdft_grid *g, const ofdft_ions *ions, const ofdft_species *sp) {
     std::vector<int> fill(g->sp_off.begin(), g->sp_off.end() - 1);
     g->sp_ions.resize(n);
     for (int i = 0; i < n; i++) g->sp_ions[fill[g->species[i]]++] = i;
+    g->sp_ions.insert(g->sp_ions.end(), g->sp_off.begin(), g->sp_off.end());
     // (the handle's own arrays: they change only after the wait above)
     CK(upload(g, g->d_species, g->species.data(), n), "upload species");
-    CK(upload(g, g->d_sp_ions, g->sp_ions.data(), n), "upload species lists");
+    CK(upload(g, g->d_sp_ions, g->sp_ions.data(), g->sp_ions.size()), "upload species lists");
     CK(upload(g, g->d_Z, g->Z.data(), g->n_species), "upload Z");
     CK(upload(g, g->d_rc, g->rc.data(), g->n_species), "upload rc");
     g->have_ions = true;

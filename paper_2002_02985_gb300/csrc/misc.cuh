@@ -20,7 +20,7 @@ struct IonArgs {
 };
 
 // vext64 != null: FP64 build; otherwise the FP32 build from the FP32 phase tables ph32 over the
-// ions grouped by species (sp_ions, HOST offsets sp_off); vf = the FP64 tables of
+// ions grouped by species (sp_ions, the groups' offsets sp_off, both device arrays); vf = the FP64 tables of
 // launch_form_tables ([n_species][NH]: v_s(|G|) / Omega), or null to evaluate them in place
 cudaError_t launch_vext(const IonArgs &a, double2 *vext64, float2 *vext32, cudaStream_t s,
                         const float2 *ph32 = nullptr, const int *sp_ions = nullptr, const int *sp_off = nullptr,

@@ -73,7 +73,10 @@ cudaError_t launch_form_tables(const IonArgs &a, double *vf, cudaStream_t st) {
 // FP32-mixed variant: S_s(G) is the complex product [rows (k0, k1) x ions] x [ions x k2] of
 // P01 = P0(k0) P1(k1) and P2(k2), formed in FP32 from the FP64 tables rounded once; groups of 8
 // ions are summed in FP32 and the groups as FP32 pairs (hi + lo, exact two-sums: about 48 bits,
-// without GB300's slow FP64 adds), the form factor and the sum over species in FP64.
+// without GB300's slow FP64 adds), the form factor and the sum over species in FP64, rounded to
+// FP32 once.  MULTI: several species in one launch, their FP64 sums in registers (one launch per
+// species that added to the stored FP32 values rounded once per species: opposite contributions
+// lost bits at every step, and V_ext crossed memory twice per species).
 //
 // Block: kVR rows x kVK values of k2; the ions come kVI at a time through shared memory, the next
 // kVI loaded into registers while the current ones are multiplied (the index and table gathers
@@ -92,8 +95,9 @@ __device__ __forceinline__ void pair_add(float2 &hi, float2 &lo, float2 x) {
     lo = __fadd2_rn(lo, __fadd2_rn(e1, e2));
     hi = s;
 }
-__global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 *ph32, const int *sp_ions, int s0,
-                                                        int s1, int s, const double *vf, float2 *v32, bool first) {
+template <bool MULTI>
+__global__ void __launch_bounds__(256, 2) vext_fast_kernel(IonArgs a, const float2 *ph32, const int *sp_ions,
+                                                        const int *sp_off, const double *vf, float2 *v32) {
     __shared__ __align__(16) float2 p01[kVI][kVR];
     __shared__ __align__(16) float4 p2s[kVI][kVK / 2];        // P2 of k2 pairs: (re, re', im, im')
     const int rows = a.n0 * a.n1, n2h = a.n2h;
@@ -101,11 +105,8 @@ __global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 
     const int tk = threadIdx.x & 15, tr = threadIdx.x >> 4;
     const float2 *P0 = ph32, *P1 = ph32 + (size_t)a.n_ions * a.n0, *P2 = P1 + (size_t)a.n_ions * a.n1;
     const float2 zero = make_float2(0.f, 0.f);
-    float2 hi[2][2][2], lo[2][2][2];                          // [row][k2 pair][re, im]
-#pragma unroll
-    for (int j = 0; j < 2; j++)
-#pragma unroll
-        for (int p = 0; p < 2; p++) hi[j][p][0] = hi[j][p][1] = lo[j][p][0] = lo[j][p][1] = zero;
+    [[maybe_unused]] double sum[2][4][2] = {};                // MULTI: [row][k2][re, im] over the species
+    int s1 = a.n_ions;
     // what this thread stages: ions i = it + 8 u (u < 4) of one row and of one pair of k2
     const int il = threadIdx.x & 31, it = threadIdx.x >> 5;
     const int row = r0 + il, k0 = row < rows ? row / a.n1 : 0, k1 = row < rows ? row - k0 * a.n1 : 0;
@@ -128,78 +129,99 @@ __global__ void __launch_bounds__(256) vext_fast_kernel(IonArgs a, const float2 
             }
         }
     };
-    load(s0);
-    for (int i0 = s0; i0 < s1; i0 += kVI) {
-        __syncthreads();
+    for (int s = 0; s < (MULTI ? a.n_species : 1); s++) {
+        float2 hi[2][2][2], lo[2][2][2];                          // [row][k2 pair][re, im]
 #pragma unroll
-        for (int v = 0; v < 4; v++) {
-            p01[it + 8 * v][il] =
-                make_float2(x[v].x * y[v].x - x[v].y * y[v].y, x[v].x * y[v].y + x[v].y * y[v].x);
-            p2s[it + 8 * v][il] = make_float4(u[v].x, w[v].x, u[v].y, w[v].y);
-        }
-        __syncthreads();
-        if (i0 + kVI < s1) load(i0 + kVI);
-        const int ni = min(kVI, s1 - i0);
-        for (int g = 0; g < ni; g += 8) {
-            float2 acc[2][2][2];
+        for (int j = 0; j < 2; j++)
 #pragma unroll
-            for (int j = 0; j < 2; j++)
+            for (int p = 0; p < 2; p++) hi[j][p][0] = hi[j][p][1] = lo[j][p][0] = lo[j][p][1] = zero;
+        const int s0 = MULTI ? sp_off[s] : 0;
+        if constexpr (MULTI) s1 = sp_off[s + 1];
+        load(s0);
+        for (int i0 = s0; i0 < s1; i0 += kVI) {
+            __syncthreads();
 #pragma unroll
-                for (int p = 0; p < 2; p++) acc[j][p][0] = acc[j][p][1] = zero;
+            for (int v = 0; v < 4; v++) {
+                p01[it + 8 * v][il] =
+                    make_float2(x[v].x * y[v].x - x[v].y * y[v].y, x[v].x * y[v].y + x[v].y * y[v].x);
+                p2s[it + 8 * v][il] = make_float4(u[v].x, w[v].x, u[v].y, w[v].y);
+            }
+            __syncthreads();
+            if (i0 + kVI < s1) load(i0 + kVI);
+            const int ni = min(kVI, s1 - i0);
+            for (int g = 0; g < ni; g += 8) {
+                float2 acc[2][2][2];
 #pragma unroll
-            for (int i = g; i < g + 8; i++) {                 // (ions past the list are zeros)
-                const float4 c01 = *reinterpret_cast<const float4 *>(&p01[i][2 * tr]);
-                const float4 qa = p2s[i][2 * tk], qb = p2s[i][2 * tk + 1];
-                const float cr[2] = {c01.x, c01.z}, ci[2] = {c01.y, c01.w};
-                const float2 Qr[2] = {make_float2(qa.x, qa.y), make_float2(qb.x, qb.y)};
-                const float2 Qi[2] = {make_float2(qa.z, qa.w), make_float2(qb.z, qb.w)};
+                for (int j = 0; j < 2; j++)
 #pragma unroll
-                for (int j = 0; j < 2; j++) {
-                    const float2 ar = make_float2(cr[j], cr[j]), ai = make_float2(ci[j], ci[j]);
-                    const float2 mi = make_float2(-ci[j], -ci[j]);
+                    for (int p = 0; p < 2; p++) acc[j][p][0] = acc[j][p][1] = zero;
 #pragma unroll
-                    for (int p = 0; p < 2; p++) {
-                        acc[j][p][0] = __ffma2_rn(mi, Qi[p], __ffma2_rn(ar, Qr[p], acc[j][p][0]));
-                        acc[j][p][1] = __ffma2_rn(ai, Qr[p], __ffma2_rn(ar, Qi[p], acc[j][p][1]));
+                for (int i = g; i < g + 8; i++) {                 // (ions past the list are zeros)
+                    const float4 c01 = *reinterpret_cast<const float4 *>(&p01[i][2 * tr]);
+                    const float4 qa = p2s[i][2 * tk], qb = p2s[i][2 * tk + 1];
+                    const float cr[2] = {c01.x, c01.z}, ci[2] = {c01.y, c01.w};
+                    const float2 Qr[2] = {make_float2(qa.x, qa.y), make_float2(qb.x, qb.y)};
+                    const float2 Qi[2] = {make_float2(qa.z, qa.w), make_float2(qb.z, qb.w)};
+#pragma unroll
+                    for (int j = 0; j < 2; j++) {
+                        const float2 ar = make_float2(cr[j], cr[j]), ai = make_float2(ci[j], ci[j]);
+                        const float2 mi = make_float2(-ci[j], -ci[j]);
+#pragma unroll
+                        for (int p = 0; p < 2; p++) {
+                            acc[j][p][0] = __ffma2_rn(mi, Qi[p], __ffma2_rn(ar, Qr[p], acc[j][p][0]));
+                            acc[j][p][1] = __ffma2_rn(ai, Qr[p], __ffma2_rn(ar, Qi[p], acc[j][p][1]));
+                        }
                     }
                 }
+#pragma unroll
+                for (int j = 0; j < 2; j++)
+#pragma unroll
+                    for (int p = 0; p < 2; p++)
+#pragma unroll
+                        for (int d = 0; d < 2; d++) pair_add(hi[j][p][d], lo[j][p][d], acc[j][p][d]);
             }
+        }
 #pragma unroll
-            for (int j = 0; j < 2; j++)
+        for (int j = 0; j < 2; j++) {
+            const int r = r0 + 2 * tr + j;
+            if (r >= rows) continue;
 #pragma unroll
-                for (int p = 0; p < 2; p++)
-#pragma unroll
-                    for (int d = 0; d < 2; d++) pair_add(hi[j][p][d], lo[j][p][d], acc[j][p][d]);
+            for (int q = 0; q < 4; q++) {
+                const int k = kc + 4 * tk + q, p = q >> 1;
+                if (k >= n2h) continue;
+                const long long e = (long long)r * n2h + k;
+                double v;
+                if (vf) {
+                    v = vf[(size_t)s * rows * n2h + e];
+                } else {
+                    double gx, gy, gz;
+                    int k0, k1, k2;
+                    gvec_of(a, e, gx, gy, gz, k0, k1, k2);
+                    v = pp_form(gx * gx + gy * gy + gz * gz, a.Z[s], a.rc[s]) / a.omega;
+                }
+                const double sr = (q & 1) ? (double)hi[j][p][0].y + (double)lo[j][p][0].y
+                                          : (double)hi[j][p][0].x + (double)lo[j][p][0].x;
+                const double si = (q & 1) ? (double)hi[j][p][1].y + (double)lo[j][p][1].y
+                                          : (double)hi[j][p][1].x + (double)lo[j][p][1].x;
+                if constexpr (MULTI) {
+                    sum[j][q][0] += v * sr;
+                    sum[j][q][1] += v * si;
+                } else {
+                    v32[e] = make_float2((float)(v * sr), (float)(v * si));
+                }
+            }
         }
     }
+    if constexpr (MULTI) {
 #pragma unroll
-    for (int j = 0; j < 2; j++) {
-        const int r = r0 + 2 * tr + j;
-        if (r >= rows) continue;
+        for (int j = 0; j < 2; j++) {
+            const int r = r0 + 2 * tr + j;
+            if (r >= rows) continue;
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int k = kc + 4 * tk + q, p = q >> 1;
-            if (k >= n2h) continue;
-            const long long e = (long long)r * n2h + k;
-            double v;
-            if (vf) {
-                v = vf[e];
-            } else {
-                double gx, gy, gz;
-                int k0, k1, k2;
-                gvec_of(a, e, gx, gy, gz, k0, k1, k2);
-                v = pp_form(gx * gx + gy * gy + gz * gz, a.Z[s], a.rc[s]) / a.omega;
+            for (int q = 0; q < 4; q++) {
+                const int k = kc + 4 * tk + q;
+                if (k < n2h) v32[(long long)r * n2h + k] = make_float2((float)sum[j][q][0], (float)sum[j][q][1]);
             }
-            const double sr = (q & 1) ? (double)hi[j][p][0].y + (double)lo[j][p][0].y
-                                      : (double)hi[j][p][0].x + (double)lo[j][p][0].x;
-            const double si = (q & 1) ? (double)hi[j][p][1].y + (double)lo[j][p][1].y
-                                      : (double)hi[j][p][1].x + (double)lo[j][p][1].x;
-            float2 o = make_float2((float)(v * sr), (float)(v * si));
-            if (!first) {
-                const float2 old = v32[e];
-                o = make_float2((float)(v * sr + (double)old.x), (float)(v * si + (double)old.y));
-            }
-            v32[e] = o;
         }
     }
 }
@@ -209,9 +231,8 @@ cudaError_t launch_vext(const IonArgs &a, double2 *vext64, float2 *vext32, cudaS
     const long long NH = (long long)a.n0 * a.n1 * a.n2h;
     if (ph32 && vext32 && !vext64) {
         const dim3 grid((unsigned)((a.n0 * a.n1 + kVR - 1) / kVR), (unsigned)((a.n2h + kVK - 1) / kVK));
-        for (int t = 0; t < a.n_species; t++)
-            vext_fast_kernel<<<grid, 256, 0, s>>>(a, ph32, sp_ions, sp_off[t], sp_off[t + 1], t,
-                                                  vf ? vf + (size_t)t * NH : nullptr, vext32, t == 0);
+        if (a.n_species > 1) vext_fast_kernel<true><<<grid, 256, 0, s>>>(a, ph32, sp_ions, sp_off, vf, vext32);
+        else vext_fast_kernel<false><<<grid, 256, 0, s>>>(a, ph32, sp_ions, sp_off, vf, vext32);
     } else {
         vext_kernel<<<(unsigned)((NH + 255) / 256), 256, 0, s>>>(a, vext64, vext32);
     }

@@ -1,0 +1,49 @@
+"""V_ext(G) of the FP32-mixed path with several species (vext_fast_kernel<true>): the species' terms are
+summed in FP64 and rounded once, whatever cancels between them."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import paper_2002_02985_gb300 as ofd  # noqa: E402
+from paper_2002_02985_gb300 import _lib as L  # noqa: E402
+
+PP = dict(terms=L.TERM_PP)
+
+
+def _potential(cell, shape, pos, species, Z, rc):
+    g = ofd.Grid(cell, shape)
+    g.set_ions(pos, species, Z, rc)
+    _, V = g.energy_potential(torch.full(shape, 0.01, dtype=torch.float32, device="cuda"), ofd.Functional(**PP))
+    return V.double()
+
+
+@pytest.mark.parametrize("shape", [(24, 20, 18), (9, 15, 250)])
+def test_species_that_cancel_leave_the_difference(shape):
+    """Ions of charge 1000 and -999 on the same sites are ions of charge 1: each coefficient is one FP64
+    difference (1000 x 2^-53) rounded to FP32 once, so at most one FP32 unit away from the single
+    species' and, over the transform, 2^-22 of its norm.  Rounding after each species would leave
+    1000 units."""
+    cell = np.diag([0.4 * n for n in shape])
+    pos = np.random.default_rng(3).uniform(0.0, 1.0, (5, 3)) @ cell
+    one = _potential(cell, shape, pos, np.zeros(5, np.int32), (1.0,), (0.8,))
+    two = _potential(cell, shape, np.concatenate([pos, pos]), np.repeat(np.arange(2, dtype=np.int32), 5),
+                     (1000.0, -999.0), (0.8, 0.8))
+    assert float((two - one).norm() / one.norm()) <= 2.0 ** -22
+
+
+@pytest.mark.parametrize("counts", [(1, 70), (33, 0, 5), (1, 1, 1, 1, 1)])
+def test_equal_species_match_one_species(counts):
+    """Ions labelled as several species of one charge and radius: groups around the tile of 32 and the
+    group of 8, a species without ions, as many species as ions.  Only the FP32 groups of 8 differ, so
+    every structure factor by at most ten roundings of terms whose norm is its own: 16 x 2^-24."""
+    shape, n = (20, 12, 27), sum(counts)
+    cell = np.diag([0.7 * m for m in shape])
+    pos = np.random.default_rng(n).uniform(0.0, 1.0, (n, 3)) @ cell
+    species = np.random.default_rng(n).permutation(np.repeat(np.arange(len(counts), dtype=np.int32), counts))
+    one = _potential(cell, shape, pos, np.zeros(n, np.int32), (3.0,), (0.8,))
+    many = _potential(cell, shape, pos, species, (3.0,) * len(counts), (0.8,) * len(counts))
+    assert float((many - one).norm() / one.norm()) <= 16 * 2.0 ** -24
