@@ -11,6 +11,7 @@
 // two fields that take the same filter share each launch (blockIdx.y is the field).
 #include "any.cuh"
 #include "plain.cuh"
+#include "sample.cuh"
 
 namespace ofdft {
 
@@ -90,7 +91,8 @@ template <typename T> __device__ __forceinline__ typename Vec2<T>::type *plain_p
 
 // What the rows subtract before the transform.  A transform alone takes the mean.  A filter only
 // needs a constant near it, so that the FP32 passes do not carry a large G = 0 term: the mean of
-// 1024 samples spread over the field, which every block takes for itself (the same loads in the
+// the field at 1024 points spread evenly over the cell (sample.cuh: within a tenth of the mean for
+// a density localised in the cell), which every block takes for itself (the same loads in the
 // same order, so the same value) instead of waiting for a pass over the whole field; block 0
 // leaves it for the inverse rows.
 template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<T> &a) {
@@ -98,14 +100,10 @@ template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<
     if (!a.sampled) return (T)a.scal[S_RHO_MEAN];
     const T *const u = a.u[f];
     __shared__ T ws[kPlainThreads / 32];
-    const long long N = (long long)a.n0 * a.n1 * a.n2, step = N / 1024 > 0 ? N / 1024 : 1;
     T s = 0;
 #pragma unroll
-    for (int k = 0; k < 1024 / kPlainThreads; k++) {
-        long long i = (threadIdx.x + k * kPlainThreads) * step;
-        if (i >= N) i %= N;                                   // (fields of fewer than 1024 points)
-        s += u[i];
-    }
+    for (int k = 0; k < kPlainSamples / kPlainThreads; k++)
+        s += u[plain_sample((int)threadIdx.x + k * kPlainThreads, a.n0, a.n1, a.n2)];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = s;
@@ -113,7 +111,7 @@ template <typename T> __device__ __forceinline__ T plain_offset(const PlainArgs<
     s = 0;
 #pragma unroll
     for (int k = 0; k < kPlainThreads / 32; k++) s += ws[k];
-    s *= (T)(1.0 / 1024.0);
+    s *= (T)(1.0 / kPlainSamples);
     if (blockIdx.x == 0 && threadIdx.x == 0) const_cast<double *>(a.scal)[f ? S_PAIR_MEAN : S_RHO_MEAN] = (double)s;
     return s;
 }
