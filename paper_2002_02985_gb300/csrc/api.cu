@@ -462,6 +462,7 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
     w.plain_any = g->kernel_choice == OFDFT_KERNELS_AUTO && !generic_only && plain_setup<T>(w.pl, g->nsm);
     cudaError_t e = prepare_kernels(w.ks);
     if (e == cudaSuccess) e = prepare_kernels(w.ks_plain);
+    if (e == cudaSuccess) e = prepare_axis0_fft<T>(g->n[0]);
     if (e != cudaSuccess) return fail(g, OFDFT_ERR_CUDA, "kernel attributes", e);
     const long long R = (long long)g->n[0] * g->n[1];
     w.nb_row = (int)(((R + 1) / 2 + min_brow - 1) / min_brow);

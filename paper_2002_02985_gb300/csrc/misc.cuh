@@ -46,7 +46,9 @@ cudaError_t launch_forces(const IonArgs &a, const C *rhohat, double *partials, i
 // F = the partials [n_ions][nchunk][3] summed over the chunks in order
 cudaError_t launch_reduce_force_partials(const double *part, int n_ions, int nchunk, double *F, cudaStream_t s);
 
-// plain forward FFT along n0 of a half spectrum (in place), used by forces
+// plain FFT along n0 of a half spectrum (in place); prepare_axis0_fft once on the device before the
+// first launch for n0
+template <typename T> cudaError_t prepare_axis0_fft(int n0);
 template <typename T>
 cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, const FFTPlan &p,
                              const typename Vec2<T>::type *tw, int TW, int thr, double scale, cudaStream_t s,

@@ -594,19 +594,28 @@ template <typename T, int N, int TWC>
 cudaError_t launch_axis0_fft_ct(typename Vec2<T>::type *data, long long P, const typename Vec2<T>::type *tw,
                                 double scale, cudaStream_t s, int dir) {
     typedef typename Vec2<T>::type C;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = allow_max_dynamic_smem(axis0_fft_ct_kernel<T, N, TWC, -1>);
-        if (e == cudaSuccess) e = allow_max_dynamic_smem(axis0_fft_ct_kernel<T, N, TWC, 1>);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
     const size_t sm = (size_t)N * sizeof(C) * (1 + TWC);
     const unsigned nb = (unsigned)((P + TWC - 1) / TWC);
     if (dir < 0) axis0_fft_ct_kernel<T, N, TWC, -1><<<nb, 256, sm, s>>>(data, P, tw, (T)scale);
     else axis0_fft_ct_kernel<T, N, TWC, 1><<<nb, 256, sm, s>>>(data, P, tw, (T)scale);
     return cudaGetLastError();
 }
+
+template <typename T> cudaError_t prepare_axis0_fft(int n0) {
+    constexpr int CAP = sizeof(T) == 4 ? 16 : 8;
+    auto both = [](auto fwd, auto inv) {
+        const cudaError_t e = allow_max_dynamic_smem(fwd);
+        return e == cudaSuccess ? allow_max_dynamic_smem(inv) : e;
+    };
+    if (n0 == 64) return both(axis0_fft_ct_kernel<T, 64, 32, -1>, axis0_fft_ct_kernel<T, 64, 32, 1>);
+    if (n0 == 96) return both(axis0_fft_ct_kernel<T, 96, 32, -1>, axis0_fft_ct_kernel<T, 96, 32, 1>);
+    if (n0 == 128) return both(axis0_fft_ct_kernel<T, 128, 32, -1>, axis0_fft_ct_kernel<T, 128, 32, 1>);
+    if (n0 == 192) return both(axis0_fft_ct_kernel<T, 192, 16, -1>, axis0_fft_ct_kernel<T, 192, 16, 1>);
+    if (n0 == 256) return both(axis0_fft_ct_kernel<T, 256, 16, -1>, axis0_fft_ct_kernel<T, 256, 16, 1>);
+    return both(axis0_fft_kernel<T, CAP, -1>, axis0_fft_kernel<T, CAP, 1>);
+}
+template cudaError_t prepare_axis0_fft<float>(int);
+template cudaError_t prepare_axis0_fft<double>(int);
 
 template <typename T>
 cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, const FFTPlan &p,
@@ -619,13 +628,6 @@ cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, 
     if (n0 == 128) return launch_axis0_fft_ct<T, 128, 32>(data, P, tw, scale, s, dir);
     if (n0 == 192) return launch_axis0_fft_ct<T, 192, 16>(data, P, tw, scale, s, dir);
     if (n0 == 256) return launch_axis0_fft_ct<T, 256, 16>(data, P, tw, scale, s, dir);
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = allow_max_dynamic_smem(axis0_fft_kernel<T, CAP, -1>);
-        if (e == cudaSuccess) e = allow_max_dynamic_smem(axis0_fft_kernel<T, CAP, 1>);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
     // a plain transform has one channel: wide column tiles (coalesced rows of up to 32 complex),
     // independent of the reciprocal-space kernel's tile.  Each thread stages at most CAP values
     // per pass, so a pass of radix R over TW columns needs (n0/R) TW / (CAP/R) threads: the tile

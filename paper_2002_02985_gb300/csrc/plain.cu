@@ -288,14 +288,12 @@ template <typename T> __global__ void __launch_bounds__(kPlainThreads, 4) plain_
 }
 
 // ---------------------------------------------------------------- launches
-template <typename T> static cudaError_t prepare_once() {
-    static const cudaError_t e = []() {
-        cudaError_t r = allow_max_dynamic_smem(plain_rows_fwd<T>);
-        if (r == cudaSuccess) r = allow_max_dynamic_smem(plain_rows_inv<T>);
-        if (r == cudaSuccess) r = allow_max_dynamic_smem(plain_n0<T>);
-        return r;
-    }();
-    return e;
+// (for every grid: the attribute belongs to the device that is current)
+template <typename T> static cudaError_t prepare_plain() {
+    cudaError_t r = allow_max_dynamic_smem(plain_rows_fwd<T>);
+    if (r == cudaSuccess) r = allow_max_dynamic_smem(plain_rows_inv<T>);
+    if (r == cudaSuccess) r = allow_max_dynamic_smem(plain_n0<T>);
+    return r;
 }
 
 template <typename T> bool plain_setup(PlainArgs<T> &a, int nsm) {
@@ -316,7 +314,7 @@ template <typename T> bool plain_setup(PlainArgs<T> &a, int nsm) {
     a.magic_n = (unsigned)(((1ull << 32) + a.n2 - 1) / a.n2);
     a.magic_n4 = a.n2 >= 8 ? (unsigned)(((1ull << 32) + a.n2 / 4 - 1) / (a.n2 / 4)) : 0;
     a.magic_n2h = (unsigned)(((1ull << 32) + a.n2h - 1) / a.n2h);
-    return prepare_once<T>() == cudaSuccess;
+    return prepare_plain<T>() == cudaSuccess;
 }
 template <typename T>
 cudaError_t launch_plain_mean(const T *u, long long N, int nblk, double *part, double *scal, unsigned *ticket,

@@ -93,3 +93,27 @@ def test_host_data_reaches_the_device_on_the_grids_stream(lib):
     up = [x for x in ops if x[0] == "memcpyAsync" and x[1] == "h2d"]
     assert up and {x[2] for x in up} == {"%x" % STREAM}
     a.close(), b.close()
+
+
+@pytest.mark.parametrize("kernels", [L.KERNELS_AUTO, L.KERNELS_GENERIC])
+@pytest.mark.parametrize("shape", [(192, 16, 192), (200, 16, 250)])
+def test_every_device_allows_the_kernels_shared_memory(lib, shape, kernels):
+    """More than 48 KB of dynamic shared memory is allowed per kernel and device: a grid on a second device
+    sets the attribute of every kernel that a grid on the first one did."""
+    seen = []
+    for device in (0, 1):
+        lib.host_cuda_device(device)
+        lib.host_cuda_reset()
+        g = Grid(lib, shape)
+        assert lib.ofdft_set_option(g.h, L.OPTION_KERNELS, ct.c_longlong(kernels)) == 0
+        for p, t in ((L.FP32_MIXED, np.float32), (L.FP64, np.float64)):
+            x = np.zeros(shape, t)
+            assert lib.ofdft_interpolate(g.h, ct.c_void_p(x.ctypes.data), g.h, ct.c_void_p(x.ctypes.data), p) == 0
+        ops = log(lib)
+        allowed = {x[1] for x in ops if x[0] == "attribute" and x[3] == str(device)}
+        assert {x[1] for x in ops if x[0] == "launch" and ("plain_" in x[1] or "axis0_fft" in x[1])
+                and "mean" not in x[1]} <= allowed
+        seen.append(allowed)
+        g.close()
+    lib.host_cuda_device(0)
+    assert seen[0] == seen[1]
