@@ -577,22 +577,27 @@ template <typename T> int ensure_vext(ofdft_grid *g) {
     IonArgs a = ion_args(g);
     cudaError_t e;
     if (sizeof(T) == 4) {
-        // the species' form factors in FP64, kept while Z and rc stay (up to 256 MB)
+        // the species' form factors in FP64, kept while Z and rc stay (up to 256 MB); the kernel evaluates
+        // them in place where memory does not allow a table
         const long long len = (long long)g->n_species * g->NH;
-        if (len <= kFormTableMax) {
-            if (g->vf_len < len) {
-                cudaFree(g->vf);
-                g->vf = nullptr;
-                g->vf_len = 0;
-                CK(gmalloc(g, &g->vf, (size_t)len * sizeof(double)), "cudaMalloc form factors");
-                g->vf_len = len;
-                g->vf_fresh = false;
+        if (g->vf_len < len) {
+            cudaFree(g->vf);
+            g->vf = nullptr;
+            g->vf_len = 0;
+            g->vf_fresh = false;
+            if (len <= kFormTableMax) {
+                const cudaError_t m = gmalloc(g, &g->vf, (size_t)len * sizeof(double));
+                if (m == cudaSuccess) g->vf_len = len;
+                else if (m == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+                else CK(m, "cudaMalloc form factors");
             }
-            if (!g->vf_fresh) CK(launch_form_tables(a, g->vf, g->stream), "form factors");
+        }
+        if (g->vf && !g->vf_fresh) {
+            CK(launch_form_tables(a, g->vf, g->stream), "form factors");
             g->vf_fresh = true;
         }
         e = launch_vext(a, nullptr, (float2 *)w.vext, g->stream, g->ph32, g->d_sp_ions, g->d_sp_ions + g->n_ions,
-                        len <= kFormTableMax ? g->vf : nullptr);
+                        g->vf);
     }
     else e = launch_vext(a, (double2 *)w.vext, nullptr, g->stream);
     CK(e, "structure factor kernel");

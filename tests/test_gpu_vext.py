@@ -47,3 +47,22 @@ def test_equal_species_match_one_species(counts):
     one = _potential(cell, shape, pos, np.zeros(n, np.int32), (3.0,), (0.8,))
     many = _potential(cell, shape, pos, species, (3.0,) * len(counts), (0.8,) * len(counts))
     assert float((many - one).norm() / one.norm()) <= 16 * 2.0 ** -24
+
+
+@pytest.mark.parametrize("n_species", [1, 8])
+def test_form_factors_in_place_match_the_table(n_species):
+    """Under a cap that admits the workspace but not the FP64 form factors the kernel evaluates them in
+    place, in FP64 too: at most one FP32 unit of a coefficient."""
+    shape = (32, 32, 32)
+    cell, NH = np.diag([9.0, 10.0, 11.0]), 32 * 32 * 17
+    pos = np.random.default_rng(n_species).uniform(0.0, 1.0, (24, 3)) @ cell
+    species = np.arange(24, dtype=np.int32) % n_species
+    Z, rc = tuple(1.0 + np.arange(n_species)), tuple(0.6 + 0.1 * np.arange(n_species))
+    V = []
+    for cap in (0, (3 + 1) * NH * 8 + (3 << 15 if n_species == 1 else 1 << 19)):
+        g = ofd.Grid(cell, shape)
+        g.set_ions(pos, species, Z, rc)
+        g.set_option(L.OPTION_ALLOC_CAP, cap)
+        V.append(g.energy_potential(torch.full(shape, 0.01, dtype=torch.float32, device="cuda"),
+                                    ofd.Functional(**PP))[1].double())
+    assert float((V[1] - V[0]).norm() / V[0].norm()) <= 2.0 ** -23

@@ -117,3 +117,25 @@ def test_every_device_allows_the_kernels_shared_memory(lib, shape, kernels):
         g.close()
     lib.host_cuda_device(0)
     assert seen[0] == seen[1]
+
+
+def test_form_factor_table_is_optional(lib):
+    """A cap that admits the workspace of an FP32 evaluation but not the FP64 form factors: the kernel
+    evaluates them in place.  One that does not admit the workspace is out of memory as before, and
+    without a cap the table is made once and kept."""
+    shape, species = (32, 32, 32), 8
+    NH = 32 * 32 * 17
+    need, table = (3 + 1) * NH * 8 + (1 << 19), species * NH * 8     # three spectra, V_ext, small arrays
+    assert (1 << 19) < table
+    for cap, rc, tables in ((need, 0, 0), (3 * NH * 8, L.OFDFT_ERR_OOM, 0), (0, 0, species)):
+        g = Grid(lib, shape)
+        assert g.set_ions(species) == 0
+        assert lib.ofdft_set_option(g.h, L.OPTION_ALLOC_CAP, ct.c_longlong(cap)) == 0
+        lib.host_cuda_reset()
+        for _ in range(2):
+            assert g.evaluate(terms=L.TERM_PP) == rc, cap
+        ops = [x for x in log(lib) if x[0] == "launch"]
+        assert sum("form_table" in x[1] for x in ops) == tables
+        if rc == 0:
+            assert sum("vext_fast" in x[1] for x in ops) == 1
+        g.close()
