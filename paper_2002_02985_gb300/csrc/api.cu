@@ -228,6 +228,15 @@ template <typename P> cudaError_t upload(ofdft_grid *g, P *dst, const P *src, si
     return cudaMemcpyAsync(dst, src, n * sizeof(P), cudaMemcpyHostToDevice, g->stream);
 }
 
+// whether the grid's stream is being captured: nothing may be allocated or timed then, and what is
+// launched has not run when the call returns
+bool capturing(ofdft_grid *g) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(g->stream, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return true;
+}
+
 template <typename T> Workspace<T> &ws(ofdft_grid *g);
 template <> Workspace<float> &ws<float>(ofdft_grid *g) { return g->w32; }
 template <> Workspace<double> &ws<double>(ofdft_grid *g) { return g->w64; }
@@ -578,9 +587,10 @@ template <typename T> int ensure_vext(ofdft_grid *g) {
     cudaError_t e;
     if (sizeof(T) == 4) {
         // the species' form factors in FP64, kept while Z and rc stay (up to 256 MB); the kernel evaluates
-        // them in place where memory does not allow a table
+        // them in place where memory does not allow a table and where a capture would have to make one
         const long long len = (long long)g->n_species * g->NH;
-        if (g->vf_len < len) {
+        const bool cap = capturing(g);
+        if (g->vf_len < len && !cap) {
             cudaFree(g->vf);
             g->vf = nullptr;
             g->vf_len = 0;
@@ -592,12 +602,12 @@ template <typename T> int ensure_vext(ofdft_grid *g) {
                 else CK(m, "cudaMalloc form factors");
             }
         }
-        if (g->vf && !g->vf_fresh) {
+        if (g->vf && !g->vf_fresh && !cap) {
             CK(launch_form_tables(a, g->vf, g->stream), "form factors");
             g->vf_fresh = true;
         }
         e = launch_vext(a, nullptr, (float2 *)w.vext, g->stream, g->ph32, g->d_sp_ions, g->d_sp_ions + g->n_ions,
-                        g->vf);
+                        g->vf_fresh ? g->vf : nullptr);
     }
     else e = launch_vext(a, (double2 *)w.vext, nullptr, g->stream);
     CK(e, "structure factor kernel");
@@ -757,11 +767,7 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
         w.tune_report = plan_report(w) + " (nothing timed)";
         return OFDFT_OK;
     }
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(g->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-        (void)cudaGetLastError();
-        return OFDFT_OK;                                  // not now: timing is impossible in a capture
-    }
+    if (capturing(g)) return OFDFT_OK;                    // not now: timing is impossible in a capture
     w.tuned = true;
     const int key[8] = {(int)sizeof(T), g->n[0], g->n[1], g->n[2], w.nslots, g->force_pick[0], g->force_pick[1],
                         g->force_pick[2]};

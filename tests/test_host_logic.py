@@ -139,3 +139,23 @@ def test_form_factor_table_is_optional(lib):
         if rc == 0:
             assert sum("vext_fast" in x[1] for x in ops) == 1
         g.close()
+
+
+def test_new_species_are_evaluated_inside_a_capture(lib):
+    """After one ordinary call an asynchronous evaluation can be captured, also when the ions have
+    become ions of more or other species since: no table is allocated, and none counts as made by a
+    launch that has only been captured."""
+    g = Grid(lib, (24, 20, 18))
+    f, E = g.functional(), np.zeros(L.N_ENERGIES)
+    call = lambda: lib.ofdft_energy_potential_async(g.h, g.density(), ct.byref(f), ct.c_void_p(E.ctypes.data), None)
+    made = lambda: sum(x[0] == "launch" and "form_table" in x[1] for x in log(lib))
+    assert g.set_ions(1) == 0 and g.evaluate() == 0
+    for n_species in (3, 2):
+        assert g.set_ions(n_species) == 0
+        lib.host_cuda_reset()
+        lib.host_cuda_capture(1)
+        rc = call()
+        lib.host_cuda_capture(0)
+        assert rc == 0 and made() == 0 and [x for x in log(lib) if x[0] == "refused"] == []
+    assert g.set_ions(2) == 0 and call() == 0 and made() == 2
+    g.close()
