@@ -90,6 +90,7 @@ template <typename T> struct Workspace {
     int grid_p1 = 0;
     // any-length kernels in use per role, their tile widths (log2), plans, largest row group
     int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0, split = 1;
+    bool no_split = false;            // memory did not allow the slots of shared tiles
     AnyPlan q0, q0i, q1, q2;
     int TW0_p = 0, thr_ax0_p = 0;     // the runtime-size n0 transform of plain fields
     bool plain_any = false;           // the any-length plain transforms (plain.cu) serve this grid
@@ -478,7 +479,22 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
     return OFDFT_OK;
 }
 
-template <typename T> int ensure_ws(ofdft_grid *g, int nslots) {
+// Term-2 slots that the blocks sharing a column tile take beyond an evaluation's other channels: the
+// pick's number of blocks, before tuning the largest of the candidates (one knot at least per block).
+template <typename T> int split_slots(const ofdft_grid *g, const Workspace<T> &w, const ofdft_functional *f) {
+    if (!f || !(f->terms & OFDFT_TERM_NL) || f->kernel != OFDFT_KERNEL_LWT || f->nl_potential != OFDFT_NLPOT_EXACT ||
+        w.no_split)
+        return 0;
+    auto slots = [&](int split) { return split > 1 && f->n_knots >= split ? split : 0; };
+    int n = slots(w.split);
+    if (!w.tuned && g->force_pick[TUNE_AXIS0] < 0)
+        for (const KernelCand &k : w.cand[TUNE_AXIS0]) n = std::max(n, slots(k.split));
+    return n;
+}
+
+// the workspace with nslots channels, and room for the shared tiles of an evaluation of f where memory
+// allows it (without, a block takes a tile's channels in turn)
+template <typename T> int ensure_ws(ofdft_grid *g, int nslots, const ofdft_functional *f = nullptr) {
     typedef typename Vec2<T>::type C;
     Workspace<T> &w = ws<T>(g);
     if (!w.ready) {
@@ -514,12 +530,34 @@ template <typename T> int ensure_ws(ofdft_grid *g, int nslots) {
         CK(cudaStreamSynchronize(g->stream), "stream synchronize");   // (the host tables end here)
         w.ready = true;
     }
+    const int extra = split_slots(g, w, f), all = nslots + extra;
     if (nslots > w.nslots) {
         if (w.chan) cudaFree(w.chan);
         w.chan = nullptr;
         w.nslots = 0;
-        CK(gmalloc(g, &w.chan, (size_t)nslots * g->NH * sizeof(C)), "cudaMalloc channel workspace");
-        w.nslots = nslots;
+        cudaError_t e = gmalloc(g, &w.chan, (size_t)all * g->NH * sizeof(C));
+        w.nslots = all;
+        if (e == cudaErrorMemoryAllocation && extra > 0) {
+            (void)cudaGetLastError();
+            w.no_split = true;
+            e = gmalloc(g, &w.chan, (size_t)nslots * g->NH * sizeof(C));
+            w.nslots = nslots;
+        }
+        if (e != cudaSuccess) w.nslots = 0;
+        CK(e, "cudaMalloc channel workspace");
+        g->generation++;
+    } else if (all > w.nslots && !capturing(g)) {
+        C *more = nullptr;
+        const cudaError_t e = gmalloc(g, &more, (size_t)all * g->NH * sizeof(C));
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            w.no_split = true;
+            return OFDFT_OK;
+        }
+        CK(e, "cudaMalloc channel workspace");
+        cudaFree(w.chan);
+        w.chan = more;
+        w.nslots = all;
         g->generation++;
     }
     return OFDFT_OK;
@@ -843,14 +881,10 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
     return OFDFT_OK;
 }
 
-// channel slots of an evaluation: Hartree + ions, vW, rho^beta (and K rho^alpha or the knots), and on
-// grids with fewer column tiles than SMs the term-2 slots of the blocks that share a tile
-int eval_slots(const ofdft_grid *g, const ofdft_functional *f) {
+// channel slots of an evaluation: Hartree + ions, vW, rho^beta (and K rho^alpha or the knots)
+int eval_slots(const ofdft_functional *f) {
     if (!(f->terms & OFDFT_TERM_NL)) return 3;
-    if (f->kernel != OFDFT_KERNEL_LWT) return 4;
-    const long long cols = (long long)g->n[1] * g->n2h;
-    const bool shared = f->nl_potential == OFDFT_NLPOT_EXACT && cols / 16 < g->nsm;
-    return 3 + f->n_knots + (shared ? kMaxSplit : 0);
+    return f->kernel != OFDFT_KERNEL_LWT ? 4 : 3 + f->n_knots;
 }
 
 // blocks of the stats kernel: a thread reads four points at a time, and a small grid makes no
@@ -924,7 +958,7 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     const bool nl = f->terms & OFDFT_TERM_NL;
     const bool lwt = nl && f->kernel == OFDFT_KERNEL_LWT;
     const int M = lwt ? f->n_knots : 0;
-    int rc = ensure_ws<T>(g, eval_slots(g, f));
+    int rc = ensure_ws<T>(g, eval_slots(f), f);
     if (rc) return rc;
     Workspace<T> &w = ws<T>(g);
     if (f->terms & OFDFT_TERM_PP) {
@@ -976,8 +1010,9 @@ int eval_args(ofdft_grid *g, const T *rho, const ofdft_functional *f, T *V, doub
     a.ticket = w.ticket;
     a.nb_stats = stats_blocks(g);
     a.clear_flags = 1;
-    // (a tile's channels are shared out by knots: one knot at least for every block)
-    a.ax0_split = lwt && M >= w.split ? w.split : 1;
+    // (a tile's channels are shared out by knots: one knot at least for every block, whose term 2 takes
+    // a slot of its own)
+    a.ax0_split = lwt && M >= w.split && (f->nl_potential != OFDFT_NLPOT_EXACT || w.nslots >= 3 + M + w.split) ? w.split : 1;
     a.t2_slot = CH_KNOT0 + M;
     a.nb_ax0 = w.ks.recip.k ? w.recip_grid : w.tile_nb_ax0 * a.ax0_split;
     a.nb_row = (int)((((long long)g->n[0] * g->n[1] + 1) / 2 + w.Brow - 1) / w.Brow);   // the row kernels' grid
@@ -2369,7 +2404,7 @@ cudaStream_t *batch_streams() {
 template <typename T>
 int prepare_batch_grid(ofdft_grid *g, const ofdft_functional *f, bool forces, const T *rho) {
     const bool nl = f->terms & OFDFT_TERM_NL;
-    int rc = ensure_ws<T>(g, eval_slots(g, f));
+    int rc = ensure_ws<T>(g, eval_slots(f), f);
     if (rc) return rc;
     if ((f->terms & OFDFT_TERM_PP) && (rc = ensure_vext<T>(g))) return rc;
     if (forces && (rc = ensure_force_buffers<T>(g))) return rc;

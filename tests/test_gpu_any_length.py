@@ -3,6 +3,8 @@ passes, odd lengths, lengths with and without compiled plans, the shortest and l
 rows of a ragged last pair and column tiles that do not divide the columns.  Bounds: FP64 1e-10 relative
 and 1e-9 Ha, FP32-mixed 1e-6 Ha/atom per term and 1e-4 of the potential away from the knots, as for every
 other kernel; a transform there and back returns the field to 100 roundings."""
+import re
+
 import numpy as np
 import pytest
 
@@ -93,3 +95,43 @@ def test_plain_transforms_return_the_field(shape, dtype):
     y = g.interpolate(x, g)
     eps = torch.finfo(dtype).eps
     assert float((y - x).abs().max()) <= 100 * eps * float(x.abs().max())
+
+
+def _shared_tile_picks(cell, shape, precision):
+    """Indices of the reciprocal-space candidates in which several blocks share a column tile (the list is in
+    the report of a grid whose kernels are all forced, which times nothing)."""
+    g = ofd.Grid(cell, shape)
+    for option in (L.OPTION_PICK_ROWS, L.OPTION_PICK_PENCIL, L.OPTION_PICK_RECIP):
+        g.set_option(option, 0)
+    dt = torch.float64 if precision == L.FP64 else torch.float32
+    g.energy_potential(torch.full(shape, 0.01, dtype=dt, device="cuda"),
+                       ofd.Functional(n_knots=9, terms=L.TERMS_ALL & ~L.TERM_PP, precision=precision))
+    seg = [x for x in g.tuning_report().split(";") if x.strip().startswith("recip")][0]
+    names = re.findall(r"\[([^\]]*)\]", seg)
+    return [i for i, x in enumerate(names) if re.search(r" s[2-8]$", x)]
+
+
+def _long_n0(n, cols):
+    shape = (n,) + cols
+    cell = np.diag([0.3 * max(m, 12) for m in shape])
+    pos = lattice_positions(cell, (max(1, round(n * 0.3 / 4.8)), 1, 1), n + 3)
+    rho = W.renormalise(W.apply_noise(W.gaussian_density(cell, shape, pos, 3.0, 1.0) + 5e-3, 0.03, n), cell,
+                        3.0 * len(pos))
+    return cell, shape, pos, rho
+
+
+def _close(E, V, Eo, Vo, rho, n_atoms, knots):
+    for k in ("TF", "vW", "NL", "H", "PP", "total"):
+        assert abs(E[k] - Eo[k]) / n_atoms <= 1e-6, (k, E[k], Eo[k])
+    m = knot_mask(rho.astype(np.float32).astype(np.float64), knots)
+    assert np.linalg.norm((V - Vo)[m]) / np.linalg.norm(Vo[m]) <= 1e-4
+
+
+def test_tiles_are_not_shared_where_memory_does_not_allow_their_slots():
+    """A cap between twelve channels and the eight slots more of a tile shared by eight blocks."""
+    cell, shape, pos, rho = _long_n0(375, (3, 8))
+    pick = _shared_tile_picks(cell, shape, L.FP32_MIXED)[-1]
+    NH = 375 * 3 * 5
+    E, V, Eo, Vo, og, g = run_both(cell, shape, pos, rho, dict(n_knots=9), L.FP32_MIXED, Z=(3.0,), rc=(0.8,),
+                                   options=((L.OPTION_PICK_RECIP, pick), (L.OPTION_ALLOC_CAP, 8 * NH * (12 + 1) + (1 << 18))))
+    _close(E, V, Eo, Vo, rho, len(pos), 9)

@@ -159,3 +159,35 @@ def test_new_species_are_evaluated_inside_a_capture(lib):
         assert rc == 0 and made() == 0 and [x for x in log(lib) if x[0] == "refused"] == []
     assert g.set_ions(2) == 0 and call() == 0 and made() == 2
     g.close()
+
+
+def test_slots_of_shared_tiles_are_optional(lib):
+    """The term-2 slots of blocks that share a column tile (32^3 has fewer tiles than SMs): none where
+    the knots are too few to be shared out, none where a cap does not admit them, and none added
+    inside a capture; the call itself succeeds as it did without shared tiles."""
+    NH, small = 32 * 32 * 17, 1 << 17
+    made = lambda: [int(x[3]) // (8 * NH) for x in log(lib) if x[0] == "malloc" and int(x[3]) >= 4 * 8 * NH]
+    terms = L.TERMS_ALL & ~L.TERM_PP
+    g = Grid(lib, (32, 32, 32))
+    lib.host_cuda_reset()
+    assert g.evaluate(knots=10, terms=terms) == 0 and made()[0] > 13
+    g.close()
+    for knots, slots in ((6, 9), (10, 13)):
+        g = Grid(lib, (32, 32, 32))
+        assert lib.ofdft_set_option(g.h, L.OPTION_ALLOC_CAP, ct.c_longlong(8 * NH * slots + small)) == 0
+        lib.host_cuda_reset()
+        assert g.evaluate(knots=knots, terms=terms) == 0 and made() == [slots]
+        assert g.evaluate(knots=knots, terms=terms) == 0 and made() == [slots]
+        g.close()
+    g = Grid(lib, (32, 32, 32))
+    f, E = g.functional(knots=10, terms=terms), np.zeros(L.N_ENERGIES)
+    f.nl_potential = L.NLPOT_INTERP
+    call = lambda: lib.ofdft_energy_potential_async(g.h, g.density(), ct.byref(f), ct.c_void_p(E.ctypes.data), None)
+    lib.host_cuda_reset()
+    assert call() == 0 and made() == [13]
+    f.nl_potential = L.NLPOT_EXACT
+    lib.host_cuda_capture(1)
+    rc = call()
+    lib.host_cuda_capture(0)
+    assert rc == 0 and [x for x in log(lib) if x[0] == "refused"] == []
+    g.close()
