@@ -132,6 +132,8 @@ def test_tiles_are_not_shared_where_memory_does_not_allow_their_slots():
     cell, shape, pos, rho = _long_n0(375, (3, 8))
     pick = _shared_tile_picks(cell, shape, L.FP32_MIXED)[-1]
     NH = 375 * 3 * 5
+    # (the channels and V_ext, the ions' phase tables in both precisions, 128 KB for the small arrays)
+    cap = 8 * NH * (12 + 1) + 24 * len(pos) * (375 + 3 + 5) + (1 << 17)
     E, V, Eo, Vo, og, g = run_both(cell, shape, pos, rho, dict(n_knots=9), L.FP32_MIXED, Z=(3.0,), rc=(0.8,),
-                                   options=((L.OPTION_PICK_RECIP, pick), (L.OPTION_ALLOC_CAP, 8 * NH * (12 + 1) + (1 << 18))))
+                                   options=((L.OPTION_PICK_RECIP, pick), (L.OPTION_ALLOC_CAP, cap)))
     _close(E, V, Eo, Vo, rho, len(pos), 9)
