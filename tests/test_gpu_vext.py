@@ -66,3 +66,49 @@ def test_form_factors_in_place_match_the_table(n_species):
         V.append(g.energy_potential(torch.full(shape, 0.01, dtype=torch.float32, device="cuda"),
                                     ofd.Functional(**PP))[1].double())
     assert float((V[1] - V[0]).norm() / V[0].norm()) <= 2.0 ** -23
+
+
+def _group_error(chain_of_four):
+    """rms error, against FP64, of the FP32 sum of eight products of phases p q (complex, so two products per
+    component): each product rounded and then added, or fused into two chains of four."""
+    f = np.float32
+    rng = np.random.default_rng(11)
+    p, q = (np.exp(2j * np.pi * rng.uniform(0.0, 1.0, (8, 200000))) for _ in range(2))
+    a, b, c, d = p.real.astype(f), p.imag.astype(f), q.real.astype(f), q.imag.astype(f)
+    fma = lambda x, y, z: (x.astype(np.float64) * y + z).astype(f)
+    exact = (a.astype(np.float64) * c - b.astype(np.float64) * d).sum(0)
+    if chain_of_four:
+        s = [np.zeros(p.shape[1], f) for _ in range(2)]
+        for i in range(8):
+            s[i // 4] = fma(-b[i], d[i], fma(a[i], c[i], s[i // 4]))
+        s = s[0] + s[1]
+    else:
+        s = np.zeros(p.shape[1], f)
+        for i in range(8):
+            s = s + fma(a[i], c[i], -(b[i] * d[i]))
+    return np.sqrt(np.mean((s - exact) ** 2))
+
+
+def test_groups_of_ions_lose_no_more_than_rounded_products():
+    """Ions of charge Z and, in another order, of charge -Z on the same sites: what is left of S(G) is the
+    rounding of the FP32 groups alone (the phases and their products are the same).  It is no larger than
+    with every product rounded and then added (a margin of 10 % for the 3000 samples; fused into one chain
+    of eight it would be 1.2 times that)."""
+    shape, n = (16, 18, 20), 480
+    cell = np.diag([8.0, 9.0, 10.0])
+    rng = np.random.default_rng(2)
+    pos = rng.uniform(0.0, 1.0, (n, 3)) @ cell
+    both = np.concatenate([pos, pos[rng.permutation(n)]])
+    V = _potential(cell, shape, both, np.repeat(np.arange(2, dtype=np.int32), n), (3.0, -3.0), (0.3, 0.3))
+    h = torch.fft.rfftn(V.reshape(shape), norm="forward").cpu().numpy()
+    m = [np.fft.fftfreq(x, 1.0 / x) for x in shape[:2]] + [np.arange(shape[2] // 2 + 1)]
+    q2 = sum(((2 * np.pi * k / cell[i, i]) ** 2).reshape([-1 if j == i else 1 for j in range(3)])
+             for i, k in enumerate(m))
+    q2[0, 0, 0] = 1.0
+    S = h / (-4.0 * np.pi * 3.0 * np.exp(-0.25 * 0.3 ** 2 * q2) / q2 / 720.0)
+    inner = np.ones(S.shape, bool)
+    inner[0, 0, 0] = inner[8] = inner[:, 9] = inner[:, :, 10] = False      # (Nyquist planes come back real)
+    rms = np.sqrt(np.mean(np.abs(S[inner]) ** 2) / 2.0)                    # per component
+    groups = 2 * n / 8
+    assert _group_error(True) <= 1.02 * _group_error(False)
+    assert rms <= 1.1 * np.sqrt(groups) * _group_error(False)
