@@ -191,3 +191,28 @@ def test_slots_of_shared_tiles_are_optional(lib):
     lib.host_cuda_capture(0)
     assert rc == 0 and [x for x in log(lib) if x[0] == "refused"] == []
     g.close()
+
+
+def test_tuner_runs_a_large_candidate_that_is_behind_once(lib):
+    """Beyond 2^24 points a configuration whose warm-up is clearly behind the best of its role is not timed
+    further, and the pick is the one that timing all of them would make; one that is ahead or level is."""
+    lib.host_cuda_cost(b"kernel", 1.0)
+    lib.host_cuda_cost(b"_any_kernel", 3.0)
+    try:
+        g = Grid(lib, (1024, 18, 1024))
+        lib.host_cuda_reset()
+        assert g.evaluate(knots=4, terms=L.TERMS_ALL & ~L.TERM_PP) == 0
+        report = lib.ofdft_tuning_report(g.h, L.FP32_MIXED).decode()
+        g.close()
+    finally:
+        lib.host_cuda_cost(b"", 0.0)
+    segments = {s.split(":")[0].strip(): s for s in report.split(";")}
+    launches = [x[1] for x in log(lib) if x[0] == "launch"]
+    for role, part in (("recip", "axis0_any_kernel"), ("rows", "row_fwd_any_kernel")):
+        behind = segments[role].count("[any")
+        assert behind > 0 and "-> any" not in segments[role], report
+        assert sum(part in x for x in launches) == behind, report
+    names = [x for x in segments["rows"].split("->")[0].split("[")[1:] if not x.startswith("any")]
+    assert len(names) > 1
+    level = sum("row_fwd" in x and "_any_kernel" not in x for x in launches)
+    assert level >= 3 * len(names)
