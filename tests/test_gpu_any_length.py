@@ -15,8 +15,12 @@ if not torch.cuda.is_available():
 
 import paper_2002_02985_gb300 as ofd  # noqa: E402
 import workloads as W  # noqa: E402
+from oracle import functionals as ofn  # noqa: E402
+from oracle import td as otd  # noqa: E402
+from oracle.evaluate import Functional as OFunc  # noqa: E402
+from oracle.grid import Grid as OGrid  # noqa: E402
 from paper_2002_02985_gb300 import _lib as L  # noqa: E402
-from test_gpu_parity import knot_mask, lattice_positions, run_both  # noqa: E402
+from test_gpu_parity import _config_case, _n_configurations, _role_cases, knot_mask, lattice_positions, run_both  # noqa: E402
 
 LENGTHS = (16, 18, 24, 27, 45, 75, 81, 90, 125, 162, 243, 250, 256, 270, 320, 375, 486, 512)
 ROLES = {"rows": ((5, 9), L.OPTION_PICK_ROWS), "pencil": ((9, 10), L.OPTION_PICK_PENCIL),
@@ -106,7 +110,7 @@ def _shared_tile_picks(cell, shape, precision):
     dt = torch.float64 if precision == L.FP64 else torch.float32
     g.energy_potential(torch.full(shape, 0.01, dtype=dt, device="cuda"),
                        ofd.Functional(n_knots=9, terms=L.TERMS_ALL & ~L.TERM_PP, precision=precision))
-    seg = [x for x in g.tuning_report().split(";") if x.strip().startswith("recip")][0]
+    seg = [x for x in g.tuning_report(precision).split(";") if x.strip().startswith("recip")][0]
     names = re.findall(r"\[([^\]]*)\]", seg)
     return [i for i, x in enumerate(names) if re.search(r" s[2-8]$", x)]
 
@@ -137,3 +141,107 @@ def test_tiles_are_not_shared_where_memory_does_not_allow_their_slots():
     E, V, Eo, Vo, og, g = run_both(cell, shape, pos, rho, dict(n_knots=9), L.FP32_MIXED, Z=(3.0,), rc=(0.8,),
                                    options=((L.OPTION_PICK_RECIP, pick), (L.OPTION_ALLOC_CAP, cap)))
     _close(E, V, Eo, Vo, rho, len(pos), 9)
+
+
+@pytest.mark.parametrize("n,cols,precision", [
+    (n, cols, p) for n, cols in ((45, (15, 8)), (128, (3, 5)), (225, (3, 5)), (250, (15, 8)), (375, (3, 5)), (486, (5, 8)))
+    for p in (L.FP32_MIXED, L.FP64) if (n, p) != (375, L.FP64)])          # (no FP64 form: too many threads)
+def test_shared_tiles_match_oracle(n, cols, precision):
+    """Every candidate whose column tiles are shared by several blocks: nine knots for up to eight blocks,
+    plans of two and three passes with radices 2, 3 and 5, the last tile ragged."""
+    cell, shape, pos, rho = _long_n0(n, cols)
+    picks = _shared_tile_picks(cell, shape, precision)
+    assert picks
+    for pick in picks:
+        E, V, Eo, Vo, og, _ = run_both(cell, shape, pos, rho, dict(n_knots=9), precision, Z=(3.0,), rc=(0.8,),
+                                       options=((L.OPTION_PICK_RECIP, pick),))
+        if precision == L.FP64:
+            assert abs(E["total"] - Eo["total"]) <= 1e-10 * max(1.0, abs(Eo["total"])), pick
+            assert np.max(np.abs(V - Vo)) <= 1e-9 * max(1.0, np.max(np.abs(Vo))), pick
+        else:
+            _close(E, V, Eo, Vo, rho, len(pos), 9)
+
+
+@pytest.mark.parametrize("n", (64, 80, 96, 120, 192, 1024))
+@pytest.mark.parametrize("role", range(3))
+def test_configurations_past_the_fifth_match_oracle(n, role):
+    """The candidates that the tests of the first five leave out."""
+    shape, option = _role_cases(n)[role]
+    count = _n_configurations(shape, ("rows", "pencil", "recip")[role])
+    cell, pos, rho = _config_case(shape)
+    for pick in range(5, count):
+        E, V, Eo, Vo, og, _ = run_both(cell, shape, pos, rho, dict(n_knots=6), L.FP32_MIXED, Z=(3.0,), rc=(0.8,),
+                                       options=((option, pick),))
+        _close(E, V, Eo, Vo, rho, len(pos), 6)
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+@pytest.mark.parametrize("role", sorted(ROLES))
+def test_any_length_configurations_past_the_third_match_oracle(role, n):
+    cell, shape, pos, rho = _case(role, n)
+    for pick in range(3, _n_configurations(shape, role)):
+        E, V, Eo, Vo, og, _ = run_both(cell, shape, pos, rho, dict(n_knots=7), L.FP32_MIXED, Z=(3.0,), rc=(0.8,),
+                                       options=((ROLES[role][1], pick),))
+        _close(E, V, Eo, Vo, rho, len(pos), 7)
+
+
+# odd rows (the scalar accesses) and rows of four points, a ragged last row pair, n0 of two and three passes
+FILTER_SHAPES = [(27, 25, 45), (125, 9, 15), (162, 6, 8), (16, 15, 250)]
+
+
+def _filter_case(shape, precision, sheared=True):
+    cell = np.diag([0.45 * max(m, 12) for m in shape])
+    if sheared:
+        cell[1, 0], cell[2, 1] = 0.6, -0.4
+    pos = np.array([[0.45, 0.5, 0.5], [0.55, 0.5, 0.5]]) @ cell
+    rho = W.renormalise(W.gaussian_density(cell, shape, pos, 2.0, 1.5) + 1e-4, cell, 4.0)
+    dt = torch.float64 if precision == L.FP64 else torch.float32
+    return cell, pos, rho, torch.from_numpy(np.ascontiguousarray(rho)).to("cuda", dt)
+
+
+def _propagate(cell, shape, pos, rho, precision, kernels):
+    g = ofd.Grid(cell, shape)
+    g.set_option(L.OPTION_KERNELS, kernels)
+    g.set_ions(pos, [0, 0], [2.0], [1.0])
+    re, im = rho.sqrt(), torch.zeros_like(rho)
+    g.td_kick(re, im, [0.05, 0.02, -0.03])
+    start = (re + 1j * im).to(torch.complex128).cpu().numpy()
+    f = ofd.Functional(terms=L.TERM_TF | L.TERM_VW | L.TERM_HARTREE | L.TERM_PP, precision=precision)
+    g.td_propagate(re, im, rho, f, 0.05, 2, solver_tol=1e-12 if precision == L.FP64 else 1e-7)
+    return start, (re + 1j * im).to(torch.complex128).cpu().numpy()
+
+
+@pytest.mark.parametrize("precision,tol", [(L.FP64, 1e-9), (L.FP32_MIXED, 2e-4)])
+@pytest.mark.parametrize("sheared", [True, False])
+@pytest.mark.parametrize("shape", FILTER_SHAPES)
+def test_filters_of_a_propagation_match_oracle_and_general_path(shape, sheared, precision, tol):
+    """H, H^2 and the preconditioner of both components (two fields, potential and base in the epilogue)."""
+    cell, pos, rho, rho_d = _filter_case(shape, precision, sheared)
+    start, psi = _propagate(cell, shape, pos, rho_d, precision, L.KERNELS_AUTO)
+    scale = np.max(np.abs(psi))
+    _, general = _propagate(cell, shape, pos, rho_d, precision, L.KERNELS_GENERIC)
+    assert np.max(np.abs(psi - general)) < tol * scale
+    if sheared and any(m % 2 == 0 for m in shape):
+        return          # on the Nyquist planes of a sheared cell the oracle's splitting iteration does not converge
+    og = OGrid(cell, shape)
+    Vg = ofn.external_potential_G(og, pos, [0, 0], [2.0], [1.0])
+    ref, _ = otd.propagate(og, start, rho_d.double().cpu().numpy(), OFunc(terms=("TF", "VW", "HARTREE", "PP")), Vg,
+                           0.05, 2, n_corrector=1)
+    assert np.max(np.abs(psi - ref)) < tol * scale
+
+
+@pytest.mark.parametrize("precision,tol", [(L.FP64, 1e-9), (L.FP32_MIXED, 1e-3)])
+@pytest.mark.parametrize("shape", FILTER_SHAPES)
+def test_preconditioned_iterations_match_general_path(shape, precision, tol):
+    """Three preconditioned iterations (FP32: each potential within 1e-4, as for every kernel)."""
+    cell, pos, rho, rho_d = _filter_case(shape, precision)
+    out = []
+    for kernels in (L.KERNELS_AUTO, L.KERNELS_GENERIC):
+        g = ofd.Grid(cell, shape)
+        g.set_option(L.OPTION_KERNELS, kernels)
+        g.set_ions(pos, [0, 0], [2.0], [1.0])
+        psi = (rho_d + 1e-3).sqrt()
+        f = ofd.Functional(terms=L.TERM_TF | L.TERM_VW | L.TERM_HARTREE | L.TERM_PP, precision=precision)
+        g.optimize_density(psi, f, 4.0, max_iter=3, precondition=True, raise_on_not_converged=False)
+        out.append(psi.double())
+    assert float((out[0] - out[1]).norm() / out[1].norm()) < tol
