@@ -92,7 +92,6 @@ template <typename T> struct Workspace {
     int any0 = 0, any1 = 0, any2 = 0, lg0 = 0, lg1 = 0, any_Gmax = 0, split = 1;
     bool no_split = false;            // memory did not allow the slots of shared tiles
     AnyPlan q0, q0i, q1, q2;
-    int TW0_p = 0, thr_ax0_p = 0;     // the runtime-size n0 transform of plain fields
     bool plain_any = false;           // the any-length plain transforms (plain.cu) serve this grid
     PlainArgs<T> pl;
     int row2_G = 0;                   // channel-batched row kernels in use: channels per group
@@ -100,7 +99,7 @@ template <typename T> struct Workspace {
     // plain one-channel transforms (preconditioner, interpolation, TD-OFDFT): the per-channel row
     // kernels where compiled (the channel-batched ones would leave most of each block idle)
     LaunchSet ks_plain;
-    int Brow_p = 0, thr_rowf_p = 0, thr_rowi_p = 0, row2_G_p = 0;
+    int Brow_p = 0, thr_rowf_p = 0, thr_rowi_p = 0;
     // persistent reciprocal-space kernel: its grid, and its tensor maps with the buffers
     // and channel count they were encoded for; the tile kernel's grid
     int recip_grid = 0, tile_nb_ax0 = 0;
@@ -375,8 +374,6 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
             TW /= 2;
         w.TW0 = TW;
         w.thr_ax0 = std::min(std::max(threads_for(g->plan[0], TW, cap), 128), tmax);
-        w.TW0_p = w.TW0;
-        w.thr_ax0_p = w.thr_ax0;
         w.Brow_p = w.Brow;
         w.thr_rowf_p = w.thr_rowi_p = w.thr_rowf;
         w.any0 = w.any1 = w.any2 = 0;
@@ -453,14 +450,12 @@ template <typename T> int choose_launch(ofdft_grid *g, Workspace<T> &w) {
     // runtime-size ones
     w.ks_plain.pen_fwd = w.ks.pen_fwd;
     w.ks_plain.pen_inv = w.ks.pen_inv;
-    w.row2_G_p = 0;
     for (const KernelCand &k : w.cand[TUNE_ROWS])
         if (!k.batched) {
             w.ks_plain.row_fwd = k.k1;
             w.ks_plain.row_inv = k.k2;
             w.Brow_p = k.B;
             w.thr_rowf_p = w.thr_rowi_p = k.nt;
-            w.row2_G_p = 0;
             break;
         }
     std::memset(&w.pl, 0, sizeof(w.pl));
@@ -1193,7 +1188,7 @@ template <typename T> EvalArgs<T> plain_args(ofdft_grid *g, Workspace<T> &w, con
     a.tw0 = w.tw[0]; a.tw1 = w.tw[1]; a.tw2 = w.tw[2];
     a.Brow = w.Brow_p; a.thr_rowf = w.thr_rowf_p; a.thr_rowi = w.thr_rowi_p;
     a.TW1 = w.TW1; a.thr_p1 = w.thr_p1; a.TW0 = w.TW0; a.thr_ax0 = w.thr_ax0; a.grid_p1 = w.grid_p1;
-    a.row2_G = w.row2_G_p; a.ax0_scr = w.ax0_scr;
+    a.row2_G = 0; a.ax0_scr = w.ax0_scr;
     any_args_of(g, w, a);
     a.nfwd = 1; a.fwd_ch[0] = CH_HPP; a.ncol = 1; a.col_ch[0] = CH_HPP;
     return a;
@@ -1234,7 +1229,7 @@ template <typename T> int forward_plain(ofdft_grid *g, Workspace<T> &w, const T 
     }
     EvalArgs<T> a = plain_args<T>(g, w, field);
     CK(launch_forward_rows_cols<T>(a, w.ks_plain, g->stream), "forward transform");
-    CK(launch_axis0_fft<T>(w.chan, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0], w.tw[0], w.TW0_p, w.thr_ax0_p,
+    CK(launch_axis0_fft<T>(w.chan, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0], w.tw[0],
                            1.0 / (double)g->N, g->stream, -1),
        "forward transform along n0");
     return OFDFT_OK;
@@ -1261,7 +1256,7 @@ template <typename T> int inverse_plain(ofdft_grid *g, Workspace<T> &w, int slot
     a.inv_ch[0] = slot;
     a.inv_kind[0] = CONS_ADD;
     CK(launch_axis0_fft<T>((C *)w.chan + (size_t)slot * g->NH, g->n[0], (long long)g->n[1] * g->n2h, g->plan[0],
-                           w.tw[0], w.TW0_p, w.thr_ax0_p, 1.0, g->stream, +1),
+                           w.tw[0], 1.0, g->stream, +1),
        "inverse transform along n0");
     CK(launch_inverse_cols_rows<T>(a, w.ks_plain, g->stream), "inverse transform");
     return OFDFT_OK;
@@ -2419,7 +2414,6 @@ cudaStream_t *batch_streams() {
 
 template <typename T>
 int prepare_batch_grid(ofdft_grid *g, const ofdft_functional *f, bool forces, const T *rho) {
-    const bool nl = f->terms & OFDFT_TERM_NL;
     int rc = ensure_ws<T>(g, eval_slots(f), f);
     if (rc) return rc;
     if ((f->terms & OFDFT_TERM_PP) && (rc = ensure_vext<T>(g))) return rc;

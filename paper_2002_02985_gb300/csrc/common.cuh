@@ -239,29 +239,4 @@ template <int K> __device__ __forceinline__ void block_sum_n_f32warp(double (&v)
     }
 }
 
-template <typename T> __device__ __forceinline__ T block_min(T v, T *scratch) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) { T w = __shfl_down_sync(0xffffffffu, v, o); v = w < v ? w : v; }
-    __syncthreads();
-    if (lane == 0) scratch[warp] = v;
-    __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    v = (threadIdx.x < nw) ? scratch[threadIdx.x] : scratch[0];
-    if (warp == 0)
-        for (int o = 16; o > 0; o >>= 1) { T w = __shfl_down_sync(0xffffffffu, v, o); v = w < v ? w : v; }
-    return v;
-}
-template <typename T> __device__ __forceinline__ T block_max(T v, T *scratch) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) { T w = __shfl_down_sync(0xffffffffu, v, o); v = w > v ? w : v; }
-    __syncthreads();
-    if (lane == 0) scratch[warp] = v;
-    __syncthreads();
-    const int nw = (blockDim.x + 31) >> 5;
-    v = (threadIdx.x < nw) ? scratch[threadIdx.x] : scratch[0];
-    if (warp == 0)
-        for (int o = 16; o > 0; o >>= 1) { T w = __shfl_down_sync(0xffffffffu, v, o); v = w > v ? w : v; }
-    return v;
-}
-
 }  // namespace ofdft

@@ -51,16 +51,12 @@ cudaError_t launch_reduce_force_partials(const double *part, int n_ions, int nch
 template <typename T> cudaError_t prepare_axis0_fft(int n0);
 template <typename T>
 cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, const FFTPlan &p,
-                             const typename Vec2<T>::type *tw, int TW, int thr, double scale, cudaStream_t s,
-                             int dir = -1);
+                             const typename Vec2<T>::type *tw, double scale, cudaStream_t s, int dir = -1);
 
 // ---- optimiser vector kernels (all reductions FP64, fixed order) ----------
-// out[slot] = sum_i a_i b_i (c_i if c != null)
-// (ticket: zero between launches; exact: every FP32 product converted and summed in FP64, for tests of the default grouping)
-template <typename T>
-cudaError_t launch_dot(const T *a, const T *b, const T *c, long long N, double *partials, int nblk,
-                       double *out, unsigned *ticket, cudaStream_t s, bool exact = false);
-// up to four products at once (row of blocks y: product y), out and ticket one entry each
+// up to four products sum_i a_i b_i (c_i if c != null) at once (row of blocks y: product y), out and
+// ticket one entry each (ticket: zero between launches; exact: every FP32 product converted and summed
+// in FP64, for tests of the default grouping)
 template <typename T> struct DotSet {
     const T *a[4], *b[4], *c[4];
 };
@@ -93,7 +89,7 @@ cudaError_t launch_grad(T *g, const T *psi, const T *V, double mu, double dV, lo
 // rho = psi^2 (and optional scale of psi)
 template <typename T>
 cudaError_t launch_square(T *rho, T *psi, double scale, long long N, cudaStream_t s);
-// d = -g + beta d ; dot partial <d, g> computed by launch_dot afterwards
+// d = -g + beta d ; dot partial <d, g> computed by launch_dots afterwards
 template <typename T> cudaError_t launch_copy(T *dst, const T *src, long long N, cudaStream_t s);
 // Fourier interpolation between two grids of one cell on normalised half spectra (layouts
 // [k0][k1][k2], k2 <= n2/2): frequencies present on both grids are copied; a Nyquist term

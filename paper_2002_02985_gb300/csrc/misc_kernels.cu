@@ -630,7 +630,7 @@ template cudaError_t prepare_axis0_fft<double>(int);
 
 template <typename T>
 cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, const FFTPlan &p,
-                             const typename Vec2<T>::type *tw, int TW, int thr, double scale, cudaStream_t s, int dir) {
+                             const typename Vec2<T>::type *tw, double scale, cudaStream_t s, int dir) {
     typedef typename Vec2<T>::type C;
     constexpr int CAP = sizeof(T) == 4 ? 16 : 8;
     // compile-time forms for the common lengths
@@ -643,8 +643,6 @@ cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, 
     // independent of the reciprocal-space kernel's tile.  Each thread stages at most CAP values
     // per pass, so a pass of radix R over TW columns needs (n0/R) TW / (CAP/R) threads: the tile
     // is narrowed until every pass fits in 512 threads and 96 KB
-    (void)TW;
-    (void)thr;
     auto need = [&](int cols) {
         long long nt = 32;
         for (int i = 0; i < p.npass; i++) {
@@ -654,10 +652,9 @@ cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, 
         }
         return (int)((nt + 31) / 32 * 32);
     };
-    int tw_cols = 32;
-    while (tw_cols > 1 && ((size_t)n0 * sizeof(C) * (1 + tw_cols) > 96 * 1024 || need(tw_cols) > 512)) tw_cols /= 2;
-    TW = tw_cols;
-    thr = need(TW) > 256 ? need(TW) : 256;
+    int TW = 32;
+    while (TW > 1 && ((size_t)n0 * sizeof(C) * (1 + TW) > 96 * 1024 || need(TW) > 512)) TW /= 2;
+    const int thr = need(TW) > 256 ? need(TW) : 256;
     if (thr > 512) return cudaErrorInvalidConfiguration;
     const size_t sm = (size_t)n0 * sizeof(C) * (1 + TW);
     const unsigned nb = (unsigned)((P + TW - 1) / TW);
@@ -665,10 +662,10 @@ cudaError_t launch_axis0_fft(typename Vec2<T>::type *data, int n0, long long P, 
     else axis0_fft_kernel<T, CAP, 1><<<nb, thr, sm, s>>>(data, n0, P, p, tw, TW, (T)scale);
     return cudaGetLastError();
 }
-template cudaError_t launch_axis0_fft<float>(float2 *, int, long long, const FFTPlan &, const float2 *, int, int,
-                                             double, cudaStream_t, int);
-template cudaError_t launch_axis0_fft<double>(double2 *, int, long long, const FFTPlan &, const double2 *, int, int,
-                                              double, cudaStream_t, int);
+template cudaError_t launch_axis0_fft<float>(float2 *, int, long long, const FFTPlan &, const float2 *, double,
+                                             cudaStream_t, int);
+template cudaError_t launch_axis0_fft<double>(double2 *, int, long long, const FFTPlan &, const double2 *, double,
+                                              cudaStream_t, int);
 
 // ---------------------------------------------------------------- optimiser vectors
 // Sums over one grid-wide launch: the last block of a row of blocks to finish adds the row's partials
@@ -730,13 +727,6 @@ cudaError_t launch_dots(const DotSet<T> &d, int n, long long N, double *partials
     dot_kernel<T><<<dim3(nblk, n), 256, 0, s>>>(d, N, partials, out, ticket, exact);
     return cudaGetLastError();
 }
-template <typename T>
-cudaError_t launch_dot(const T *a, const T *b, const T *c, long long N, double *partials, int nblk, double *out,
-                       unsigned *ticket, cudaStream_t s, bool exact) {
-    DotSet<T> d = {{a}, {b}, {c}};
-    return launch_dots<T>(d, 1, N, partials, nblk, out, ticket, s, exact);
-}
-
 // One step of up to two conjugate-gradient solves (row of blocks y: solve y): x += al q, r -= al w,
 // out = <r, r>.  One launch where the two updates and the product of each solve were three (2 x 25 us
 // at 128^3); sums grouped as in dot_kernel.
@@ -1195,8 +1185,6 @@ INST_TD(double)
     template cudaError_t launch_hvp<T>(T *, const T *, const T *, const T *, const T *, double, double,      \
                                        double, long long, cudaStream_t);                                     \
     template cudaError_t launch_add_scalar<T>(T *, const double *, long long, cudaStream_t);                  \
-    template cudaError_t launch_dot<T>(const T *, const T *, const T *, long long, double *, int, double *,    \
-                                       unsigned *, cudaStream_t, bool);                                                \
     template cudaError_t launch_axpby<T>(T *, const T *, double, double, long long, cudaStream_t);           \
     template cudaError_t launch_rotate<T>(T *, T *, const T *, const T *, double, double, long long,         \
                                           cudaStream_t);                                                     \
