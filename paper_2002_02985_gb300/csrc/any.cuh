@@ -485,7 +485,8 @@ __device__ __forceinline__ void axis0_any_body(const EvalArgs<T> &a, const int b
         else any_pass<+1>(qi.p[np - 1], qi.p[np - 1].nb << lg, tw, dec, sh(S), G);
     }
     double r4[4] = {eH, eV, eP, eN};
-    // (a tile shared by several blocks: FP64 throughout, its few blocks hide the slow adds)
+    // (a tile shared by several blocks: the block's sum in FP64, its few blocks hide the slow adds; the terms of
+    // a thread's RL frequencies are added in FP32 in either case)
     if (sizeof(T) == 4 && S == 1) block_sum_n_f32warp<4>(r4, sd);
     else block_sum_n<4>(r4, sd);
     if (threadIdx.x == 0)
@@ -604,10 +605,11 @@ template <typename T, int E__, bool INV, int R1 = 0, int R2 = 1, int R3 = 1> str
 // registers, 70 us with 160 and 72).  Longer rows keep two elements per thread, which spares the idle
 // threads of small channel groups (256^3, forward / inverse: 613 / 870 us against 648 / 900 us).
 constexpr int any_ct_E(int n) { return n <= 200 ? 1 : 2; }
-// Beyond 256 points a block has one thread per two points and at least six warps, and 24 warps share an
-// SM at 80 registers (320 threads at two blocks per SM: whole evaluations of 256 x 256 x 320 and
-// 256 x 256 x 512 5.00 and 7.77 ms, now 4.60 and 7.22; 512^3 with 15 channels 28.99 -> 27.70 ms); 129 to 160 points take 192 threads, so that all
-// channels of an ordinary call go in one group (144^3: 0.690 -> 0.670 ms).
+// Beyond 256 points a block has one thread per two points and at least six warps, and 24 warps (21 from 385
+// to 448 points, three blocks of 7) share an SM at 80 registers (320 threads at two blocks per SM: whole
+// evaluations of 256 x 256 x 320 and 256 x 256 x 512 5.00 and 7.77 ms, now 4.60 and 7.22; 512^3 with 15
+// channels 28.99 -> 27.70 ms); 129 to 160 points take 192 threads, so that all channels of an ordinary call
+// go in one group (144^3: 0.690 -> 0.670 ms).
 constexpr int any_ct_row_threads(int n) {
     return n <= 128 ? 160 : (n <= 160 ? 192 : (n <= 200 ? 256 : (n <= 256 ? 320 : (n <= 384 ? 192 : ((n + 63) / 64 * 32)))));
 }
