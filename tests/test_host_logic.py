@@ -216,3 +216,19 @@ def test_tuner_runs_a_large_candidate_that_is_behind_once(lib):
     assert len(names) > 1
     level = sum("row_fwd" in x and "_any_kernel" not in x for x in launches)
     assert level >= 3 * len(names)
+
+
+@pytest.mark.parametrize("n2,cost,pick", [(30, 0.92, "pencil"), (27, 0.5, "ctpencil")])
+def test_tuner_keeps_the_earlier_of_two_level_candidates_on_small_grids(lib, n2, cost, pick):
+    """Up to 2^18 points a candidate replaces an earlier one only when it is ahead by more than such short
+    timings scatter, so that the picks, and with them the results' last bits, are those of every process."""
+    lib.host_cuda_cost(b"kernel", 1.0)
+    lib.host_cuda_cost(b"pencil_ct_kernel", cost)
+    try:
+        g = Grid(lib, (24, 32, n2))
+        assert g.evaluate(knots=5, terms=L.TERMS_ALL & ~L.TERM_PP) == 0
+        report = lib.ofdft_tuning_report(g.h, L.FP32_MIXED).decode()
+        g.close()
+    finally:
+        lib.host_cuda_cost(b"", 0.0)
+    assert [s for s in report.split(";") if s.strip().startswith("pencil")][0].split("-> ")[1].split()[0] == pick, report
