@@ -833,9 +833,10 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
     const int reps = large ? 2 : 5;
     constexpr float kBehind = 1.01f;
     float plan_ms = 0.f;                                                          // the plan in place, if timed
-    // Five evaluations of a small grid scatter by 1 to 2 % (32^3: 54.4 to 56.1 us): there a candidate has to be
-    // ahead by more than that, so that the picks, and the results' last bits, are those of every process.
-    const float ahead = g->N <= (1LL << 18) ? 0.96f : 1.0f;
+    // Five evaluations of less than 0.1 ms scatter by 1 to 2 % (32^3: 54.4 to 56.1 us): there a candidate has to
+    // be ahead by more than that, so that the picks, and the results' last bits, are those of every process.
+    // (longer ones take the best: the same margin for FP64 at 32^3, 0.25 ms, cost 1.4 % of an optimisation)
+    auto ahead = [](float ms, float best_ms) { return ms < (best_ms < 0.1f ? 0.96f : 1.0f) * best_ms; };
     w.tuning = true;
     int rc = OFDFT_OK;
     std::string rep;
@@ -869,7 +870,7 @@ template <typename T> int autotune(ofdft_grid *g, Workspace<T> &w, const T *rho,
             char buf[96];
             std::snprintf(buf, sizeof(buf), " [%s] %.4f ms", w.cand[r][c].name, ms);
             rep += buf;
-            if (best < 0 || ms < ahead * best_ms) {
+            if (best < 0 || ahead(ms, best_ms)) {
                 best = c;
                 best_ms = ms;
             }

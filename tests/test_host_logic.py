@@ -220,10 +220,11 @@ def test_tuner_runs_a_large_candidate_that_is_behind_once(lib):
 
 @pytest.mark.parametrize("n2,cost,pick", [(30, 0.92, "pencil"), (27, 0.5, "ctpencil")])
 def test_tuner_keeps_the_earlier_of_two_level_candidates_on_small_grids(lib, n2, cost, pick):
-    """Up to 2^18 points a candidate replaces an earlier one only when it is ahead by more than such short
-    timings scatter, so that the picks, and with them the results' last bits, are those of every process."""
-    lib.host_cuda_cost(b"kernel", 1.0)
-    lib.host_cuda_cost(b"pencil_ct_kernel", cost)
+    """Where an evaluation takes less than 0.1 ms a candidate replaces an earlier one only when it is ahead by
+    more than such short timings scatter, so that the picks, and with them the results' last bits, are those
+    of every process."""
+    lib.host_cuda_cost(b"kernel", 0.01)
+    lib.host_cuda_cost(b"pencil_ct_kernel", 0.01 * cost)
     try:
         g = Grid(lib, (24, 32, n2))
         assert g.evaluate(knots=5, terms=L.TERMS_ALL & ~L.TERM_PP) == 0
